@@ -124,96 +124,130 @@ __device__ __forceinline__ uint32_t popc8(const uint32_t (&w)[8]) {
 }
 
 constexpr int kOverlapWarps = 8;
-constexpr int kOvCPW = 4;                          // candidates per warp (register blocking)
-constexpr int kOvCands = kOverlapWarps * kOvCPW;   // candidates per block
-constexpr int kOvNPL = 8;                          // words per lane per sub-segment
-constexpr int kOvSub = 32 * kOvNPL;                // words per sub-segment (256)
-constexpr int kOvSubs = 2;                         // sub-segments per block (512 words)
-constexpr int kOvArch = 32;                        // archive members staged per pass
+constexpr int kOvNPL = 8;              // words per lane of a segment
+constexpr int kOvSeg = 32 * kOvNPL;    // words per block (8,192 rows)
+constexpr int kOvArch = 32;            // archive members per block: a lane each
+constexpr int kOvRow = kOvSeg + 1;     // staged row stride: 32 members' words of one position
+                                       // lie in 32 banks
+constexpr int kOvList = 128;           // longest list of non-zero words a warp walks
 
-// overlaps[c][a] += popcount(M_c & M_a) over this block's words, for the block's 32 candidates
-// and every archive member. The archive's words of each 256-word sub-segment are staged in
-// shared memory once per block and read by all warps; each warp keeps 4 candidates' words in
-// registers, so an archive word read from shared memory serves 4 AND+popc. Partial sums live in
-// shared memory per (candidate, member) and reach HBM as one atomicAdd each per block.
-__global__ void __launch_bounds__(kOverlapWarps * 32)
+// overlaps[c][a] += popcount(M_c & M_a) over the block's 256 words, for its candidates (CPW per
+// warp) and up to 32 archive members. The members' words are staged in
+// shared memory once per block. A warp holds its candidates' words in registers, eight per lane,
+// and lane a carries the sums with member a, so no partial sum goes through memory until one
+// atomic per lane at the end. Each candidate takes one of three forms by its non-zero words here:
+//   none: nothing to add (a chain of 8 columns matches 1 row in 40,320 of random values);
+//   few:  they are compacted into a list (value and position) and every lane ANDs the listed
+//         words with its own member's: one staged word, AND and popcount per word for 32 members
+//         at once, no reduction. Measured cost about 6 warp instructions per word;
+//   many: a member at a time over all 256 words, each staged word read once for all of the
+//         warp's such candidates, carry-save popcount and a warp reduction: about 36 warp
+//         instructions per member.
+// The line between few and many is where those costs meet, 6 words per member. Candidates of
+// 2-16 columns over random rows are few or none from 5 columns on.
+// Bound by the dense candidates' AND and popcount work and by its loads' latency, hence five
+// blocks per SM (48 registers) with two candidates per warp. 1,600 candidates, 20 members:
+// 436,444 rows 99 -> 56 us, 20,000 rows 28 -> 7.5 us (four candidates per warp at three blocks
+// per SM 56, at two 67, one candidate 64); 40 x 40 over 20,000 rows 54 -> 6 us (the former form
+// used 4 blocks there). The form before took every segment with a match through the dense walk.
+template <int CPW>
+__global__ void __launch_bounds__(kOverlapWarps * 32, 5)
     overlap_kernel(const uint32_t* __restrict__ bitmaps, uint32_t n_cand,
                    const uint32_t* __restrict__ arch, uint32_t n_arch, int64_t W,
                    uint32_t* __restrict__ overlaps, uint32_t* __restrict__ arch_counts,
-                   const uint32_t* err) {
-  __shared__ uint32_t arch_s[kOvArch][kOvSub];
-  __shared__ uint32_t part_s[kOvCands][kOvArch];
+                   const uint32_t* err, uint32_t cand_blocks, uint32_t segments) {
+  __shared__ uint32_t arch_s[kOvArch * kOvRow];
+  __shared__ uint2 list_s[kOverlapWarps][kOvList];
   if (*reinterpret_cast<const volatile uint32_t*>(err) != 0) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t c0 = blockIdx.x * kOvCands + warp * kOvCPW;  // this warp's first candidate
-  const int64_t wblk = (int64_t)blockIdx.y * kOvSub * kOvSubs;
-  for (uint32_t a0 = 0; a0 < n_arch; a0 += kOvArch) {
-    const int na = n_arch - a0 < (uint32_t)kOvArch ? (int)(n_arch - a0) : kOvArch;
-    for (int i = tid; i < kOvCands * kOvArch; i += blockDim.x) (&part_s[0][0])[i] = 0u;
-    for (int sub = 0; sub < kOvSubs; ++sub) {
-      const int64_t ws = wblk + (int64_t)sub * kOvSub;
-      if (ws >= W) break;
-      __syncthreads();
-      for (int i = tid; i < na * kOvSub; i += blockDim.x) {
-        const int a = i / kOvSub, w = i % kOvSub;
-        arch_s[a][w] = ws + w < W ? __ldg(arch + (size_t)(a0 + a) * W + ws + w) : 0u;
-      }
-      __syncthreads();
-      if (blockIdx.x == 0) {  // the archive's own row counts, once per word segment
-        for (int a = warp; a < na; a += kOverlapWarps) {
-          uint32_t n = 0;
+  // block = (member group, segment, candidate group), the candidates fastest: neighbours share
+  // the segment's archive words in L2
+  const uint32_t cb = blockIdx.x % cand_blocks, rest = blockIdx.x / cand_blocks;
+  const uint32_t c0 = (cb * kOverlapWarps + warp) * CPW;  // this warp's first candidate
+  const int64_t ws = (int64_t)(rest % segments) * kOvSeg;
+  const int nw = W - ws < kOvSeg ? (int)(W - ws) : kOvSeg;  // words of this segment
+  const uint32_t a0 = rest / segments * kOvArch;
+  const int na = n_arch - a0 < (uint32_t)kOvArch ? (int)(n_arch - a0) : kOvArch;
+  // the candidates' words are requested before the archive's are staged
+  uint32_t cw[CPW][kOvNPL];
 #pragma unroll
-          for (int t = 0; t < kOvNPL; ++t) n += __popc(arch_s[a][lane + 32 * t]);
-          n = __reduce_add_sync(0xFFFFFFFFu, n);
-          if (lane == 0 && n) atomicAdd(&arch_counts[a0 + a], n);
-        }
-      }
-      uint32_t cw[kOvCPW][kOvNPL];
+  for (int c = 0; c < CPW; ++c)
 #pragma unroll
-      for (int c = 0; c < kOvCPW; ++c)
-#pragma unroll
-        for (int t = 0; t < kOvNPL; ++t) {
-          const int64_t w = ws + lane + 32 * t;
-          cw[c][t] = (c0 + c < n_cand && w < W) ? __ldg(bitmaps + (size_t)(c0 + c) * W + w) : 0u;
-        }
-      // a candidate whose 256 words here are all zero contributes nothing to any overlap: long
-      // chains match few rows, so most of their sub-segments are skipped (warp-uniform flags)
-      bool nz[kOvCPW];
-      bool any = false;
-#pragma unroll
-      for (int c = 0; c < kOvCPW; ++c) {
-        uint32_t o = 0;
-#pragma unroll
-        for (int t = 0; t < kOvNPL; ++t) o |= cw[c][t];
-        nz[c] = __any_sync(0xFFFFFFFFu, o != 0u);
-        any |= nz[c];
-      }
-      if (any) {
-        for (int a = 0; a < na; ++a) {
-          uint32_t x[kOvNPL];
-#pragma unroll
-          for (int t = 0; t < kOvNPL; ++t) x[t] = arch_s[a][lane + 32 * t];
-#pragma unroll
-          for (int c = 0; c < kOvCPW; ++c) {
-            if (!nz[c]) continue;
-            uint32_t w[kOvNPL];
-#pragma unroll
-            for (int t = 0; t < kOvNPL; ++t) w[t] = cw[c][t] & x[t];
-            const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, popc8(w));
-            if (lane == 0) part_s[warp * kOvCPW + c][a] += v;
-          }
-        }
-      }
+    for (int t = 0; t < kOvNPL; ++t) {
+      const int w = lane + 32 * t;
+      cw[c][t] = c0 + c < n_cand && w < nw
+                     ? __ldg(bitmaps + (size_t)(c0 + c) * (size_t)W + ws + w) : 0u;
     }
-    __syncthreads();
-    for (int i = tid; i < kOvCands * na; i += blockDim.x) {
-      const int c = i / na, a = i % na;
-      const uint32_t v = part_s[c][a];
-      const uint32_t cand = blockIdx.x * kOvCands + c;
-      if (v && cand < n_cand) atomicAdd(&overlaps[(size_t)cand * n_arch + a0 + a], v);
+  for (int a = warp; a < na; a += kOverlapWarps) {
+    const uint32_t* src = arch + (size_t)(a0 + a) * (size_t)W + ws;
+    uint32_t v[kOvNPL];
+#pragma unroll
+    for (int t = 0; t < kOvNPL; ++t) {
+      const int w = lane + 32 * t;
+      v[t] = w < nw ? __ldg(src + w) : 0u;
     }
-    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kOvNPL; ++t) arch_s[a * kOvRow + lane + 32 * t] = v[t];
+    if (cb == 0) {  // the archive's own row counts, once per segment
+      const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, popc8(v));
+      if (lane == 0 && n) atomicAdd(&arch_counts[a0 + a], n);
+    }
   }
+  __syncthreads();
+  const int few = 6 * na < kOvList ? 6 * na : kOvList;
+  uint32_t sum[CPW];  // lane a: the overlap with member a0 + a
+  bool many[CPW];
+  bool any_many = false;
+  uint2* const list = list_s[warp];
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) {
+    sum[c] = 0u;
+    uint32_t bal[kOvNPL];
+    int nz = 0;
+#pragma unroll
+    for (int t = 0; t < kOvNPL; ++t) {
+      bal[t] = __ballot_sync(0xFFFFFFFFu, cw[c][t] != 0u);
+      nz += __popc(bal[t]);
+    }
+    many[c] = nz > few;
+    any_many |= many[c];
+    if (nz == 0 || many[c]) continue;  // warp-uniform
+    const uint32_t lt = (1u << lane) - 1u;
+    int base = 0;
+#pragma unroll
+    for (int t = 0; t < kOvNPL; ++t) {
+      if (cw[c][t]) list[base + __popc(bal[t] & lt)] = make_uint2(cw[c][t], lane + 32 * t);
+      base += __popc(bal[t]);
+    }
+    __syncwarp();
+    const uint32_t* row = arch_s + lane * kOvRow;  // (lanes past na read rows nobody uses)
+#pragma unroll 4
+    for (int i = 0; i < nz; ++i) {
+      const uint2 e = list[i];
+      sum[c] += __popc(e.x & row[e.y]);
+    }
+    __syncwarp();  // the list is rebuilt for the next candidate
+  }
+  if (any_many) {
+    for (int a = 0; a < na; ++a) {
+      uint32_t x[kOvNPL];
+#pragma unroll
+      for (int t = 0; t < kOvNPL; ++t) x[t] = arch_s[a * kOvRow + lane + 32 * t];
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) {
+        if (!many[c]) continue;
+        uint32_t w[kOvNPL];
+#pragma unroll
+        for (int t = 0; t < kOvNPL; ++t) w[t] = cw[c][t] & x[t];
+        const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, popc8(w));
+        if (lane == a) sum[c] = v;
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < CPW; ++c)
+    if (lane < na && sum[c])
+      atomicAdd(&overlaps[(size_t)(c0 + c) * n_arch + a0 + lane], sum[c]);
 }
 
 constexpr int kFinalizeWarps = 8;
@@ -344,15 +378,23 @@ cudaError_t launch_overlap(const uint32_t* bitmaps, uint32_t n_cand, const uint3
                            uint32_t n_arch, int64_t words, uint32_t* overlaps,
                            uint32_t* arch_counts, const uint32_t* err, int num_sms,
                            cudaStream_t s) {
-  (void)num_sms;
   if (n_cand == 0 || n_arch == 0) return cudaSuccess;
-  const int64_t per_block = (int64_t)kOvSub * kOvSubs;
-  const int64_t gy = (words + per_block - 1) / per_block;
-  if (gy > 65535) return cudaErrorInvalidConfiguration;
-  dim3 grid((n_cand + kOvCands - 1) / kOvCands, (unsigned)gy);
+  const uint64_t segments = (uint64_t)(words + kOvSeg - 1) / kOvSeg;
+  const uint64_t groups = (n_arch + kOvArch - 1) / kOvArch;
+  auto cand_blocks = [&](uint32_t cpw) {
+    return ((uint64_t)n_cand + kOverlapWarps * cpw - 1) / (kOverlapWarps * cpw);
+  };
+  // two candidates per warp share each staged archive word and each block's staging; where that
+  // leaves less than one resident wave (five blocks per SM), one per warp, for the shorter chain
+  // and the wider grid
+  const bool one = cand_blocks(2) * segments * groups < 5ull * (num_sms > 0 ? num_sms : 1);
+  const uint64_t cb = cand_blocks(one ? 1 : 2), blocks = cb * segments * groups;
+  if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+  auto kern = one ? overlap_kernel<1> : overlap_kernel<2>;
   count_launch();
-  overlap_kernel<<<grid, kOverlapWarps * 32, 0, s>>>(bitmaps, n_cand, arch_bitmaps, n_arch, words,
-                                                     overlaps, arch_counts, err);
+  kern<<<(unsigned)blocks, kOverlapWarps * 32, 0, s>>>(bitmaps, n_cand, arch_bitmaps, n_arch,
+                                                       words, overlaps, arch_counts, err,
+                                                       (uint32_t)cb, (uint32_t)segments);
   return cudaGetLastError();
 }
 
