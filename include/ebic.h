@@ -97,7 +97,7 @@ int ebic_free_matrix(ebic_matrix* m);
 /*
  * Shape of a loaded matrix. Any output pointer may be NULL.
  *   words      W = ceil(rows/32), the bitmap length per candidate
- *   rank_bits  8 (cols <= 127) or 16: the width of the stored ranks
+ *   rank_bits  8 (cols <= 127) or 16: the width of a rank
  */
 int ebic_matrix_info(const ebic_matrix* m, int64_t* rows, int32_t* cols, int64_t* words,
                      int32_t* rank_bits);
@@ -278,7 +278,7 @@ int ebic_fitness_reduced(const ebic_matrix* m, const uint16_t* cols, const uint3
 
 /*
  * Row-tile height of the evaluator for this matrix, in slabs (1, 2 or 4), or 0 for the
- * built-in choice. A slab is 512 rows for 8-bit ranks and 256, 128 or 64 rows for 16-bit ranks
+ * built-in choice. A slab is 512 rows up to 208 columns, then 256, 128 or 64
  * (ebic_matrix_get_tile reports it). The tile changes speed only, never results. The autotuner
  * sets it from timed sweeps. A tile whose shared-memory stage would not fit returns
  * EBIC_ERR_UNSUPPORTED. Not thread-safe with concurrent evaluations of the same matrix.

@@ -9,10 +9,9 @@
 //   * CTAs take items from one atomic counter (dynamic load balance across uneven candidate
 //     lengths, 2-64, and uneven matrix sizes) and prefetch the next item's row tile with TMA into
 //     the other of two shared-memory stages while they compute the current one;
-//   * every request keeps its own rank layout (8- or 16-bit ranks, VEC, tile height) and
-//     negative-trend option; a switch per item selects the matching instantiation of the same
-//     inner loop as the single-population evaluator, so results are identical to it;
-//   * tensor maps of all matrices sit in a device array.
+//   * every request keeps its own rank layout (bit planes, slab and tile height) and
+//     negative-trend option; the walk is the single-population evaluator's with the layout taken
+//     at run time, so results are identical to it.
 // A check kernel first validates every request's candidate list on the device (CSR shape,
 // column range, repeats) and zeroes its counts; a failed request gets no work items.
 #include <cstring>
@@ -28,19 +27,8 @@
 namespace ebic {
 namespace {
 
-// 32 warps per CTA: the cases the batch uses (8-bit ranks with tiles of at most 2 slabs, or 1
-// with negative trends; 16-bit ranks with 1 slab) all fit in 64 registers per thread.
 constexpr int kBatchThreads = 1024;
 constexpr int kBatchWarps = kBatchThreads / 32;
-
-// The largest tile height the batch uses for a request (results never depend on the tile).
-int batch_tile_cap(const Layout& L, bool neg) { return L.width == 8 ? (neg ? 1 : 2) : 1; }
-
-// layout cases: 0..2 = 8-bit ranks, VEC 4, TS 1/2/4; 3 = 16-bit VEC 4; 4 = VEC 2; 5 = VEC 1
-int layout_case(const Layout& L, int ts) {
-  if (L.width == 8) return ts == 1 ? 0 : ts == 2 ? 1 : 2;
-  return L.vec == 4 ? 3 : L.vec == 2 ? 4 : 5;
-}
 
 struct BatchReq {
   const uint16_t* cand_cols;
@@ -48,17 +36,16 @@ struct BatchReq {
   uint32_t* counts;
   uint32_t* bitmaps;  // may be null: counts only
   uint32_t* status;   // the matrix's deferred-status word
-  int64_t slabs, groups, words;
+  const uint32_t* ranks;  // the matrix's bit planes
+  int64_t slabs, words;
   uint32_t n_cand;
   uint32_t cand_base;  // sum of n_cand of the requests before this one
-  int32_t lcase;       // layout case
-  int32_t vec;         // row groups per slab
+  int32_t planes;      // bit planes of a code
+  int32_t slab_high;   // bitmap words per slab
   int32_t neg;
-  int32_t ts;
-  int32_t col_box, n_col_boxes;
-  uint32_t stage_bytes;
+  int32_t ts;          // slabs per row tile
+  uint32_t pitch_bytes, slab_bytes;
   int32_t chunk_cols;
-  uint32_t tmap;       // index into the tensor-map array
   const uint32_t* pairs;  // the matrix's pair table: the request runs on the batched pair pass
   uint32_t pair_stride;
   int32_t pair_cols;
@@ -326,70 +313,25 @@ __global__ void batch_plan_kernel(const BatchReq* __restrict__ reqs, BatchHeader
 }
 
 // One row tile of one request for every candidate of the staged chunk.
-template <int WIDTH, int VEC, int TS, bool NEG>
+template <bool NEG>
 __device__ __forceinline__ void batch_tile(const uint8_t* stage, const BatchReq& q,
                                            const uint16_t* ccols, const uint16_t* coffs,
                                            uint32_t lo, uint32_t nc, int64_t tile, int lane,
-                                           int warp, const uint32_t (&trot)[5],
-                                           const uint32_t (&tsel)[5]) {
-  constexpr int GT = TS * VEC;
-  constexpr int WPT = GT * Swar<WIDTH>::WPG;
-  const uint32_t col_stride = TS * 128 * VEC;
-  const uint8_t* lane_base = stage + lane * 4 * VEC;
-  const int64_t word0 = tile * WPT;
-  const int64_t g0 = tile * GT;
-  for (uint32_t ci = warp; ci < nc; ci += kBatchWarps) {
-    const int o = coffs[ci];
-    const int L = coffs[ci + 1] - o;
-    uint32_t acc[GT];
-    trend_masks<WIDTH, VEC, TS, NEG>(lane_base, col_stride, ccols + o, L, acc);
-    const uint32_t cand = lo + ci;
-    uint32_t cnt = 0;
-    if (q.bitmaps) {
-      uint32_t* out = q.bitmaps + (size_t)cand * (size_t)q.words;
-#pragma unroll
-      for (int b = 0; b < (GT + WIDTH - 1) / WIDTH; ++b) {
-        const uint32_t w = transpose32(pack_block<WIDTH, GT>(acc, b), trot, tsel);
-        const int g = b * WIDTH + (lane % WIDTH);
-        const int64_t widx = word0 + g * Swar<WIDTH>::WPG + lane / WIDTH;
-        if (g < GT && widx < q.words) {
-          out[widx] = w;
-          cnt += __popc(w);
-        }
-      }
-    } else {
-#pragma unroll
-      for (int g = 0; g < GT; ++g)
-        if (g0 + g < q.groups) cnt += __popc(acc[g]);
-    }
-    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if (lane == 0 && cnt) atomicAdd(&q.counts[cand], cnt);
-  }
-}
-
-template <bool NEG>
-__device__ __forceinline__ void batch_tile_case(int lcase, const uint8_t* stage,
-                                                const BatchReq& q, const uint16_t* ccols,
-                                                const uint16_t* coffs, uint32_t lo, uint32_t nc,
-                                                int64_t tile, int lane, int warp,
-                                                const uint32_t (&trot)[5],
-                                                const uint32_t (&tsel)[5]) {
-  switch (lcase) {
-    case 0: batch_tile<8, 4, 1, NEG>(stage, q, ccols, coffs, lo, nc, tile, lane, warp, trot, tsel); break;
-    case 1:
-      if constexpr (!NEG)
-        batch_tile<8, 4, 2, NEG>(stage, q, ccols, coffs, lo, nc, tile, lane, warp, trot, tsel);
-      break;
-    case 3: batch_tile<16, 4, 1, NEG>(stage, q, ccols, coffs, lo, nc, tile, lane, warp, trot, tsel); break;
-    case 4: batch_tile<16, 2, 1, NEG>(stage, q, ccols, coffs, lo, nc, tile, lane, warp, trot, tsel); break;
-    default: batch_tile<16, 1, 1, NEG>(stage, q, ccols, coffs, lo, nc, tile, lane, warp, trot, tsel); break;
-  }
+                                           int warp) {
+  const TileShape sh{q.planes, q.slab_high, q.ts, q.pitch_bytes};
+  const uint32_t group = 32u / (uint32_t)min(32, q.slab_high * q.ts);  // candidates per warp
+  uint32_t c = (uint32_t)warp * group;
+  eval_tile<0, 0, NEG>(sh, stage, ccols, coffs, lo, nc, tile * q.ts * q.slab_high, q.words,
+                       q.counts, q.bitmaps, q.words, lane, [&]() {
+                         const uint32_t r = c;
+                         c += kBatchWarps * group;
+                         return r;
+                       });
 }
 
 // Shared memory: [stage 0][stage 1][chunk columns (chunk_cap + slack)][chunk offsets]
 __global__ void __launch_bounds__(kBatchThreads, 1)
-    batch_eval_kernel(const BatchReq* __restrict__ reqs, const CUtensorMap* __restrict__ tmaps,
-                      BatchHeader* hdr, const unsigned long long* __restrict__ start,
+    batch_eval_kernel(const BatchReq* __restrict__ reqs, BatchHeader* hdr, const unsigned long long* __restrict__ start,
                       uint32_t stage_cap, int32_t chunk_cap, uint64_t timeout_ns,
                       uint32_t* err_out) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -402,8 +344,6 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   __shared__ int it_stage;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t trot[5], tsel[5];
-  transpose_consts(lane, trot, tsel);
   const uint32_t n_req = hdr->n_req;
   const unsigned long long total = hdr->total_items;
   uint8_t* const stage0 = smem;
@@ -438,13 +378,13 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     const unsigned long long local = g - dec_lo;
     const long long n_tiles = (rq.slabs + rq.ts - 1) / rq.ts;
     const long long tile = (long long)(local % (unsigned long long)n_tiles);
-    const uint32_t col_stride = (uint32_t)rq.ts * 128u * (uint32_t)rq.vec;
-    uint8_t* dst = s ? stage1 : stage0;
-    dev::acquire_tensormap(&tmaps[rq.tmap]);
-    dev::mbar_arrive_expect_tx(&full_bar[s], rq.stage_bytes);
-    for (int b = 0; b < rq.n_col_boxes; ++b)
-      dev::tma_load_3d(dst + (size_t)b * rq.col_box * col_stride, &tmaps[rq.tmap], &full_bar[s],
-                       0, (int32_t)(tile * rq.ts), b * rq.col_box);
+    const long long q0 = tile * rq.ts;
+    const uint32_t slabs = (uint32_t)(rq.slabs - q0 < rq.ts ? rq.slabs - q0 : rq.ts);
+    const uint32_t bytes = (slabs - 1u) * rq.pitch_bytes + rq.slab_bytes;
+    dev::mbar_arrive_expect_tx(&full_bar[s], bytes);
+    dev::bulk_load(s ? stage1 : stage0,
+                   reinterpret_cast<const uint8_t*>(rq.ranks) + (size_t)q0 * rq.pitch_bytes, bytes,
+                   &full_bar[s]);
   };
 
   if (tid == 0) {
@@ -502,16 +442,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     if (!__syncthreads_and(ok)) { timed_out = true; break; }
     const uint8_t* stage = s ? stage1 : stage0;
     if (q.neg)
-      batch_tile_case<true>(q.lcase, stage, q, ccols, coffs, cur_lo, cur_nc, tile, lane, warp,
-                            trot, tsel);
+      batch_tile<true>(stage, q, ccols, coffs, cur_lo, cur_nc, tile, lane, warp);
     else
-      batch_tile_case<false>(q.lcase, stage, q, ccols, coffs, cur_lo, cur_nc, tile, lane, warp,
-                             trot, tsel);
+      batch_tile<false>(stage, q, ccols, coffs, cur_lo, cur_nc, tile, lane, warp);
     __syncthreads();  // every warp is done with stage s
     if (tid == 0) {  // item_s[s] is next read two iterations on, after further barriers
       const unsigned long long gn = next_item();
       item_s[s] = gn;
-      if (gn < total) issue(gn, s);
+      if (gn < total) {
+        dev::fence_proxy_async();  // the stage's reads before the copy
+        issue(gn, s);
+      }
     }
   }
   if (timed_out && tid == 0) {
@@ -686,7 +627,6 @@ namespace {
 
 struct HostPlan {
   std::vector<BatchReq> reqs;
-  std::vector<CUtensorMap> tmaps;
   std::vector<int32_t> ncols;
   uint32_t total_cand = 0;
   uint32_t stage_cap = 0;
@@ -752,14 +692,11 @@ bool is_dev(const void* p, int dev) {
 int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_cap,
                HostPlan* hp) {
   hp->reqs.clear();
-  hp->tmaps.clear();
   hp->ncols.clear();
   hp->total_cand = 0;
   uint64_t total = 0;
   uint32_t cap = fixed_stage_cap;
   std::vector<EvalArgs> args(n);
-  std::vector<EvalConfig> cfgs(n);
-  std::vector<const CUtensorMap*> maps(n);
   for (uint32_t i = 0; i < n; ++i) {
     const ebic_eval_request& r = reqs[i];
     if (!r.m) return set_last_error(EBIC_ERR_INVALID_ARG, "request has a NULL matrix");
@@ -792,8 +729,7 @@ int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_c
         return set_last_error(EBIC_ERR_INVALID_ARG,
                               (who + "the archive and fitness must be device buffers").c_str());
     }
-    int rc = matrix_eval_plan(r.m, r.n_cand > 0 ? r.n_cand : 1, 0, &args[i], &cfgs[i], &maps[i],
-                              batch_tile_cap(v.L, (r.flags & EBIC_NEGATIVE_TRENDS) != 0));
+    int rc = matrix_eval_plan(r.m, &args[i]);
     if (rc != EBIC_OK) return rc;
     if (!fixed_stage_cap && args[i].stage_bytes > cap) cap = args[i].stage_bytes;
     if (args[i].stage_bytes > cap)
@@ -819,21 +755,24 @@ int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_c
     MatrixView v;
     matrix_view(r.m, &v);
     q.status = v.status;
+    q.ranks = a.ranks;
     q.slabs = a.slabs;
-    q.groups = a.groups;
     q.words = a.words;
     q.n_cand = r.n_cand;
     q.cand_base = base;
-    q.lcase = layout_case(v.L, cfgs[i].ts);
-    q.vec = v.L.vec;
+    q.planes = a.planes;
+    q.slab_high = a.slab_high;
     q.neg = (r.flags & EBIC_NEGATIVE_TRENDS) ? 1 : 0;
-    q.ts = cfgs[i].ts;
-    q.col_box = a.col_box;
-    q.n_col_boxes = a.n_col_boxes;
-    q.stage_bytes = a.stage_bytes;
-    // chunks: about 2 items per SM over the whole batch is enough with dynamic scheduling
-    q.chunk_cols = std::min<int32_t>(hp->chunk_cap, std::max<int32_t>(64, a.chunk_cols));
-    q.tmap = i;
+    q.ts = a.ts;
+    q.pitch_bytes = a.pitch_bytes;
+    q.slab_bytes = a.slab_bytes;
+    // chunks: about two items per SM of the request alone (its list's length is known on the
+    // device only; 16 columns per candidate stand for it)
+    const int64_t tiles = (a.slabs + a.ts - 1) / a.ts;
+    const int64_t want = std::max<int64_t>(1, (2ll * hp->num_sms + tiles - 1) / tiles);
+    const int64_t cc = ((int64_t)r.n_cand * 16 + want - 1) / want;
+    q.chunk_cols = (int32_t)std::max<int64_t>(
+        64, std::min<int64_t>(std::min(hp->chunk_cap, a.chunk_cols), (cc + 63) / 64 * 64));
     q.pairs = v.pairs;
     q.pair_stride = v.pair_stride;
     q.pair_cols = v.L.cols;
@@ -845,7 +784,6 @@ int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_c
       q.arch_offsets = r.arch_offsets;
       q.arch_src = r.arch_bitmaps;
     }
-    hp->tmaps.push_back(*maps[i]);
     hp->ncols.push_back(v.L.cols);
     hp->reqs.push_back(q);
     base += r.n_cand;
@@ -870,7 +808,6 @@ int cerr(cudaError_t e, const char* what) {
 // Device-side buffers of one batch (capacity n_max requests).
 struct DeviceBatch {
   BatchReq* reqs = nullptr;
-  CUtensorMap* tmaps = nullptr;
   int32_t* ncols = nullptr;
   uint32_t* req_err = nullptr;
   unsigned long long* start = nullptr;
@@ -883,7 +820,7 @@ struct DeviceBatch {
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 size_t batch_bytes(uint32_t n_max) {
-  return align256(sizeof(BatchReq) * n_max) + align256(sizeof(CUtensorMap) * n_max) +
+  return align256(sizeof(BatchReq) * n_max) +
          align256(4 * (size_t)n_max) + align256(4 * (size_t)n_max) +
          align256(8 * ((size_t)n_max + 1)) + align256(32 * ((size_t)n_max + 1)) +
          align256(sizeof(BatchHeader)) + 256;
@@ -893,8 +830,6 @@ void carve(uint8_t* base, uint32_t n_max, DeviceBatch* d) {
   size_t o = 0;
   d->reqs = reinterpret_cast<BatchReq*>(base + o);
   o += align256(sizeof(BatchReq) * n_max);
-  d->tmaps = reinterpret_cast<CUtensorMap*>(base + o);
-  o += align256(sizeof(CUtensorMap) * n_max);
   d->ncols = reinterpret_cast<int32_t*>(base + o);
   o += align256(4 * (size_t)n_max);
   d->req_err = reinterpret_cast<uint32_t*>(base + o);
@@ -937,7 +872,7 @@ int launch_batch(const DeviceBatch& d, uint32_t stage_cap, int32_t chunk_cap, in
                                                          (unsigned long long)num_sms);
   B_CUDA(cudaGetLastError());
   count_launch();
-  batch_eval_kernel<<<num_sms, kBatchThreads, smem, s>>>(d.reqs, d.tmaps, d.hdr, d.start,
+  batch_eval_kernel<<<num_sms, kBatchThreads, smem, s>>>(d.reqs, d.hdr, d.start,
                                                           stage_cap, chunk_cap, 1000000000ull,
                                                           d.err);
   B_CUDA(cudaGetLastError());
@@ -981,7 +916,7 @@ struct ebic_batch {
   int device = 0;
   int num_sms = 0;
   uint8_t* dmem = nullptr;   // device buffers
-  uint8_t* hmem = nullptr;   // pinned mirror of the request/tensor-map/ncols/header part
+  uint8_t* hmem = nullptr;   // pinned mirror of the request/ncols/header part
   DeviceBatch d, h;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t done = nullptr;
@@ -1015,9 +950,6 @@ int ebic_eval_batch(const ebic_eval_request* reqs, uint32_t n_req, void* stream)
   place_fitness(&hp, static_cast<uint8_t*>(mem) + bb, &h.zero, &h.n_zero);
   cudaError_t e = cudaMemcpyAsync(d.reqs, hp.reqs.data(), sizeof(BatchReq) * n_req,
                                   cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d.tmaps, hp.tmaps.data(), sizeof(CUtensorMap) * n_req,
-                        cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d.ncols, hp.ncols.data(), 4 * (size_t)n_req, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d.hdr, &h, sizeof(h), cudaMemcpyHostToDevice, s);
@@ -1122,7 +1054,6 @@ int ebic_batch_run(ebic_batch* b, const ebic_eval_request* reqs, uint32_t n_req,
   if (hp.fit_bytes) place_fitness(&hp, b->fmem, &b->h.hdr->zero, &b->h.hdr->n_zero);
   if (n_req > 0) {
     std::memcpy(b->h.reqs, hp.reqs.data(), sizeof(BatchReq) * n_req);
-    std::memcpy(b->h.tmaps, hp.tmaps.data(), sizeof(CUtensorMap) * n_req);
     std::memcpy(b->h.ncols, hp.ncols.data(), 4 * (size_t)n_req);
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);

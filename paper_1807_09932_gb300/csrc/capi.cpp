@@ -1,9 +1,7 @@
 // Host runtime and C ABI of the EBIC GB300 library: argument checks, placement of host/device
-// buffers, stream-ordered scratch, tensor-map setup, launch planning and error reporting.
+// buffers, stream-ordered scratch, launch planning and error reporting.
 // Every computational step runs in this library's CUDA kernels; this file only moves data and
 // launches them.
-#include <cudaTypedefs.h>
-
 #include <algorithm>
 #include <climits>
 #include <atomic>
@@ -26,9 +24,6 @@ struct ebic_matrix {
   uint32_t* ranks = nullptr;   // device rank matrix
   uint32_t* status = nullptr;  // device deferred-status word
   int num_sms = 0;
-  std::mutex mu;
-  CUtensorMap tmap[3];         // one per tile height TS = 1, 2, 4
-  bool tmap_ok[3] = {false, false, false};
   int tile = 0;                // 0: built-in tile choice; else the TS every evaluation uses
   int chunk = 0;               // 0: built-in chunk size; else candidate columns per chunk
   uint32_t* pairs = nullptr;   // pair table [cols*cols][pair_stride], padding zero, or null
@@ -267,40 +262,6 @@ std::string check_candidates_host(const uint16_t* cols, const uint32_t* offsets,
   return why.empty() ? check_columns_host(cols, offsets, n, ncols) : why;
 }
 
-// Tensor map over the rank matrix: dims {32*VEC words, Q slabs, C columns}, box
-// {32*VEC, TS, col_box}. Built once per (matrix, TS) and cached.
-int get_tmap(ebic_matrix* m, int ts, int col_box, const CUtensorMap** out) {
-  const int idx = ts == 1 ? 0 : ts == 2 ? 1 : 2;
-  std::lock_guard<std::mutex> lk(m->mu);
-  if (!m->tmap_ok[idx]) {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    if (!encode) {
-      cudaDriverEntryPointQueryResult q;
-      void* fn = nullptr;
-      cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                       cudaEnableDefault, &q);
-      if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
-        return fail(EBIC_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-      encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
-    const Layout& L = m->L;
-    const cuuint64_t wps = 32ull * (cuuint64_t)L.vec;
-    cuuint64_t dims[3] = {wps, (cuuint64_t)L.slabs, (cuuint64_t)L.cols};
-    cuuint64_t strides[2] = {wps * 4ull, (cuuint64_t)L.slabs * wps * 4ull};
-    cuuint32_t box[3] = {(cuuint32_t)wps, (cuuint32_t)ts, (cuuint32_t)col_box};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = encode(&m->tmap[idx], CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, m->ranks, dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS)
-      return fail(EBIC_ERR_CUDA, "cuTensorMapEncodeTiled failed with code " + std::to_string(r));
-    m->tmap_ok[idx] = true;
-  }
-  *out = &m->tmap[idx];
-  return EBIC_OK;
-}
-
 // ---- diagnostics: launch counter and per-kernel CUDA-event timing --------------------------
 std::atomic<int64_t> g_launches{0};
 std::atomic<bool> g_timing{false};
@@ -366,62 +327,49 @@ Layout make_layout(int64_t rows, int32_t cols) {
   L.rows = rows;
   L.cols = cols;
   L.words = (rows + 31) / 32;
-  if (cols <= 127) {
-    L.width = 8;
-    L.vec = 4;
-  } else {
-    L.width = 16;
-    L.vec = (int64_t)cols * 512 <= kStageMax ? 4 : (int64_t)cols * 256 <= kStageMax ? 2 : 1;
-  }
-  L.rows_per_group = L.width == 8 ? 128 : 64;
-  L.words_per_group = L.rows_per_group / 32;
-  const int64_t g = (rows + L.rows_per_group - 1) / L.rows_per_group;
-  L.slabs = (g + L.vec - 1) / L.vec;
-  L.groups = L.slabs * L.vec;
+  L.width = cols <= 127 ? 8 : 16;
+  while ((1 << L.planes) <= cols) ++L.planes;
+  while ((int64_t)cols * L.planes * L.slab_high * 4 > kStageMax) L.slab_high /= 2;
+  L.slabs = (L.words + L.slab_high - 1) / L.slab_high;
+  L.slab_bytes = (uint32_t)(cols * L.planes * L.slab_high * 4);
+  // (a multiple of 16 bytes for every layout: 64 x, 32 x, 16 x, or 10 planes x 8)
+  L.pitch_bytes = L.slab_bytes + (L.slab_high == 16 && L.slab_bytes / 64 % 2 == 0 ? 64 : 0);
   return L;
 }
 
-static void col_boxes(int32_t cols, int* nb, int* cb) {
-  *nb = (cols + 255) / 256;
-  *cb = (cols + *nb - 1) / *nb;
+// Tiles of several slabs (slabs of 16 words only: the others fill a stage by themselves): the
+// allowed heights are those whose rows would fit a stage at a byte per value.
+static bool tile_allowed(const Layout& L, int ts) {
+  return ts == 1 || (L.width == 8 && (int64_t)L.cols * ts * L.rows_per_slab() <= kStageMax);
 }
 
 int default_tile_slabs(const Layout& L) {
-  int nb, cb;
-  col_boxes(L.cols, &nb, &cb);
-  for (int ts = 4; ts >= 1; ts >>= 1) {
-    if (ts > L.slabs && ts > 1) continue;
-    if ((int64_t)nb * cb * ts * 128 * L.vec <= kStageMax) return ts;
-  }
+  for (int ts = 4; ts > 1; ts >>= 1)
+    if (ts <= L.slabs && tile_allowed(L, ts)) return ts;
   return 1;
 }
 
-bool plan_eval(const Layout& L, int ts, uint32_t n_cand, int64_t total_cols_hint, int grid,
-               EvalArgs* a, int32_t chunk_override) {
-  int nb, cb;
-  col_boxes(L.cols, &nb, &cb);
-  const int64_t col_stride = (int64_t)ts * 128 * L.vec;
-  const int64_t stage = (int64_t)nb * cb * col_stride;
+bool plan_eval(const Layout& L, const uint32_t* ranks, int ts, EvalArgs* a,
+               int32_t chunk_override) {
+  // one stage's copy: whole slabs at their pitch, the last without its padding
+  const int64_t stage = ((int64_t)(ts - 1) * L.pitch_bytes + L.slab_bytes + 127) / 128 * 128;
   // chunk buffers: (CC + slack) column slots and (CC + 1) offsets, 2 bytes each
   const int64_t left = kSmemDynMax - 2 * stage - 2 * (kChunkSlack + 1) - 256;
-  int64_t cc_max = std::min<int64_t>(kMaxChunkCols, left / 4);
-  cc_max = cc_max / 64 * 64;
-  if (cc_max < 64) return false;
-  const int64_t n_tiles = (L.slabs + ts - 1) / ts;
-  const int64_t total = total_cols_hint > 0 ? total_cols_hint : (int64_t)n_cand * 16;
-  const int64_t want_chunks = std::max<int64_t>(1, (2 * (int64_t)grid + n_tiles - 1) / n_tiles);
-  int64_t cc = (total + want_chunks - 1) / want_chunks;
-  if (chunk_override > 0) cc = chunk_override;
-  cc = (cc + 63) / 64 * 64;
-  cc = std::max<int64_t>(64, std::min(cc, cc_max));
-  a->cols = L.cols;
+  int64_t cc = std::min<int64_t>(kMaxChunkCols, left / 4) / 64 * 64;
+  if (cc < 64) return false;
+  // The largest chunk by default: the work is split evenly whatever the number of chunks, and
+  // each further chunk stages every row tile again.
+  if (chunk_override > 0) cc = std::min<int64_t>(cc, (chunk_override + 63) / 64 * 64);
+  a->ranks = ranks;
+  a->planes = L.planes;
+  a->slab_high = L.slab_high;
+  a->ts = ts;
+  a->pitch_bytes = L.pitch_bytes;
+  a->slab_bytes = L.slab_bytes;
   a->slabs = L.slabs;
-  a->groups = L.groups;
   a->words = L.words;
   a->bitmap_stride = L.words;
   a->chunk_cols = (int32_t)cc;
-  a->col_box = cb;
-  a->n_col_boxes = nb;
   a->stage_bytes = (uint32_t)stage;
   a->smem_bytes =
       (uint32_t)((2 * stage + 2 * (cc + kChunkSlack) + 2 * (cc + 1) + 15) / 16 * 16);
@@ -439,21 +387,11 @@ void matrix_view(const ebic_matrix* m, MatrixView* v) {
   v->total_rows = m->total_rows;
 }
 
-int matrix_eval_plan(const ebic_matrix* cm, uint32_t n_cand, int64_t total_cols_hint,
-                     EvalArgs* a, EvalConfig* cfg, const CUtensorMap** tmap, int ts_cap) {
-  ebic_matrix* m = const_cast<ebic_matrix*>(cm);
-  const Layout& L = m->L;
-  int ts = m->tile ? m->tile : default_tile_slabs(L);
-  while (ts > 1 && ts > L.slabs) ts >>= 1;
-  while (ts_cap > 0 && ts > ts_cap) ts >>= 1;
-  if (!plan_eval(L, ts, n_cand, total_cols_hint, m->num_sms, a, m->chunk))
+int matrix_eval_plan(const ebic_matrix* m, EvalArgs* a) {
+  int ts = m->tile ? m->tile : default_tile_slabs(m->L);
+  while (ts > 1 && ts > m->L.slabs) ts >>= 1;
+  if (!plan_eval(m->L, m->ranks, ts, a, m->chunk))
     return fail(EBIC_ERR_UNSUPPORTED, "no shared-memory plan for this matrix shape");
-  int rc = get_tmap(m, ts, a->col_box, tmap);
-  if (rc != EBIC_OK) return rc;
-  cfg->width = L.width;
-  cfg->vec = L.vec;
-  cfg->ts = ts;
-  cfg->grid = m->num_sms;
   return EBIC_OK;
 }
 
@@ -464,17 +402,6 @@ const char* check_candidates_host_c(const uint16_t* cols, const uint32_t* offset
   thread_local std::string why;
   why = check_candidates_host(cols, offsets, n, ncols);
   return why.c_str();
-}
-
-cudaError_t launch_eval(const EvalConfig& cfg, const CUtensorMap* tmap, const EvalArgs& a,
-                        cudaStream_t s) {
-  if (cfg.width == 8) return launch_eval_w8v4(cfg, tmap, a, s);
-  switch (cfg.vec) {
-    case 4: return launch_eval_w16v4(cfg, tmap, a, s);
-    case 2: return launch_eval_w16v2(cfg, tmap, a, s);
-    case 1: return launch_eval_w16v1(cfg, tmap, a, s);
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 }  // namespace ebic
@@ -498,20 +425,13 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     if (foreign_device(p, dev)) return fail(EBIC_ERR_INVALID_ARG, "buffer on another device");
 
   const bool host_lists = !on_device(cols, dev) && !on_device(offsets, dev);
-  int64_t total_hint = 0;
   if (host_lists) {
     std::string why = check_candidates_host(cols, offsets, n_cand, L.cols);
     if (!why.empty()) return fail(EBIC_ERR_INVALID_ARG, why);
-    total_hint = offsets[n_cand];
   }
 
-  int ts = m->tile ? m->tile : default_tile_slabs(L);
-  while (ts > 1 && ts > L.slabs) ts >>= 1;
   EvalArgs a;
-  if (!plan_eval(L, ts, n_cand, total_hint, m->num_sms, &a, m->chunk))
-    return fail(EBIC_ERR_UNSUPPORTED, "no shared-memory plan for this matrix shape");
-  const CUtensorMap* tmap = nullptr;
-  int rc = get_tmap(m, ts, a.col_box, &tmap);
+  int rc = matrix_eval_plan(m, &a);
   if (rc != EBIC_OK) return rc;
 
   Scratch sc(s);
@@ -583,26 +503,17 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     p.status = m->status;
     EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !timing_on(), s));
   } else {
-  a.n_cand = n_cand;
-  a.cand_cols = dcols;
-  a.cand_offsets = doffs;
-  a.counts = dcounts;
-  a.bitmaps = dbitmaps;
-  a.bitmap_stride = bitmap_stride;
-  a.err = err;
-  a.err_out = err;
-  a.status = m->status;
-  EvalConfig cfg;
-  cfg.width = L.width;
-  cfg.vec = L.vec;
-  cfg.ts = ts;
-  cfg.negative = (flags & EBIC_NEGATIVE_TRENDS) != 0;
-  cfg.bitmaps = dbitmaps != nullptr;
-  cfg.grid = m->num_sms;
-  {
+    a.n_cand = n_cand;
+    a.cand_cols = dcols;
+    a.cand_offsets = doffs;
+    a.counts = dcounts;
+    a.bitmaps = dbitmaps;
+    a.bitmap_stride = bitmap_stride;
+    a.err = err;
+    a.err_out = err;
+    a.status = m->status;
     Timed t(EBIC_TIMING_EVALUATE, s);
-    EBIC_CUDA(launch_eval(cfg, tmap, a, s));
-  }
+    EBIC_CUDA(launch_eval(a, neg, m->num_sms, !timing_on(), s));
   }
 
   if (counts_host || bitmaps_host) {
@@ -732,13 +643,14 @@ int ebic_matrix_ranks(const ebic_matrix* m, uint16_t* out, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   EBIC_CUDA(cudaMemcpyAsync(raw.data(), m->ranks, raw.size() * 4, cudaMemcpyDeviceToHost, s));
   EBIC_CUDA(cudaStreamSynchronize(s));
-  const uint32_t mask = L.width == 8 ? 0xFFu : 0xFFFFu;
+  const size_t pitch = L.pitch_bytes / 4;
   for (int64_t r = 0; r < L.rows; ++r) {
-    const int64_t g = r / L.rows_per_group, rr = r % L.rows_per_group;
-    const int64_t lane = rr & 31, k = rr >> 5, q = g / L.vec, j = g % L.vec;
+    const int64_t word = r >> 5, q = word / L.slab_high, w = word % L.slab_high;
+    const int bit = (int)(r & 31);
     for (int32_t c = 0; c < L.cols; ++c) {
-      const size_t w = (((size_t)c * L.slabs + q) * 32 + lane) * L.vec + j;
-      const uint32_t v = (raw[w] >> (L.width * k)) & mask;  // code 0 = missing, else rank + 1
+      const uint32_t* p = raw.data() + q * pitch + (size_t)c * L.planes * L.slab_high + w;
+      uint32_t v = 0;  // code 0 = missing, else rank + 1
+      for (int32_t b = 0; b < L.planes; ++b) v |= ((p[b * L.slab_high] >> bit) & 1u) << b;
       out[r * L.cols + c] = v == 0 ? 0xFFFFu : (uint16_t)(v - 1);
     }
   }
@@ -1200,11 +1112,8 @@ int ebic_matrix_set_tile(ebic_matrix* m, int32_t tile_slabs) {
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
   if (tile_slabs != 0 && tile_slabs != 1 && tile_slabs != 2 && tile_slabs != 4)
     return fail(EBIC_ERR_INVALID_ARG, "tile_slabs must be 0, 1, 2 or 4");
-  if (tile_slabs != 0) {
-    int nb = (m->L.cols + 255) / 256, cb = (m->L.cols + nb - 1) / nb;
-    if ((int64_t)nb * cb * tile_slabs * 128 * m->L.vec > kStageMax)
-      return fail(EBIC_ERR_UNSUPPORTED, "tile does not fit in shared memory for this matrix");
-  }
+  if (tile_slabs != 0 && !ebic::tile_allowed(m->L, tile_slabs))
+    return fail(EBIC_ERR_UNSUPPORTED, "tile does not fit in shared memory for this matrix");
   m->tile = tile_slabs;
   return EBIC_OK;
 }

@@ -1,17 +1,16 @@
 // Internal declarations of the EBIC GB300 library (not part of the public ABI).
 //
 // Rank-matrix layout in HBM (built once per matrix by the rank transform):
-//   Ranks are dense per-row ranks, stored in WIDTH = 8 bits (cols <= 127) or 16 bits. A 32-bit
-//   "lane word" packs 32/WIDTH rows of one column: byte/half k of the word of lane l in row
-//   group g holds row g*RPG + 32*k + l, where RPG = 32 * (32/WIDTH) rows per group (128 or 64).
-//   VEC consecutive groups form a slab. The matrix is stored column-major over slabs:
-//       word(c, q, l, j) = ((c * Q + q) * 32 + l) * VEC + j,   group g = q * VEC + j
-//   so that one 16-byte load per lane (VEC = 4) fetches four groups of one column, and a 3-D
-//   TMA box {32*VEC words, TS slabs, columns} lands in shared memory column-major with the TS
-//   slabs of one column contiguous.
-//   Stored codes: 0 marks a missing value (and every padding row past the end); a real value is
-//   stored as its dense rank + 1, in 1..cols. Since cols <= 127 (8-bit) or <= 32767 (16-bit), the
-//   top bit of every field is always 0, which the SWAR compare in the evaluator relies on.
+//   Ranks are dense per-row ranks. A missing value (and every padding row past the end) has code
+//   0, a real value its dense rank + 1, in 1..cols. Codes are stored as bit planes, NB of them
+//   (the bits of `cols`): a slab holds T bitmap words of rows (32 T rows) and is the contiguous
+//   block [column][plane][T words], word w of plane p of column c having bit p of that column's
+//   code for the 32 rows of the slab's bitmap word w, lowest row in the lowest bit. So a plane's
+//   words are in the order and bit order of the row bitmaps the evaluator writes, and a row tile
+//   of whole slabs is one contiguous copy. T is 16 where a slab of that height fits a pipeline
+//   stage (up to 208 columns), else 8, 4 or 2. Slabs of 16 words are an odd number of 64-byte
+//   units apart (one unit of padding where needed): the two halves of a warp that read the same
+//   column of two neighbouring slabs then hit different banks.
 #pragma once
 
 #include <cstddef>
@@ -30,6 +29,7 @@ constexpr uint32_t kUnusedDraws = 1u << 16;
 constexpr int kSmemLimit = 232448;            // 227 KB shared memory per CTA (static + dynamic)
 constexpr int kSmemDynMax = kSmemLimit - 2048;  // dynamic part: room for the kernels' static smem
 constexpr int kStageMax = 104 * 1024;         // per pipeline stage (two stages)
+constexpr int kMaxPlanes = 10;                // bits of kMaxCols
 constexpr int kMaxChunkCols = 16384;
 constexpr int kChunkSlack = 72;  // spare column slots past a chunk (candidate tail + prefetch)
 
@@ -38,19 +38,17 @@ constexpr uint32_t kErrInvalid = 1u;
 constexpr uint32_t kErrTimeout = 2u;
 
 struct Layout {
-  int32_t width = 8;         // bits per stored rank: 8 or 16
-  int32_t vec = 4;           // groups per slab: 4, 2 or 1
-  int32_t rows_per_group = 128;
-  int32_t words_per_group = 4;  // bitmap words produced by one group
+  int32_t width = 8;      // bits per rank as reported: 8 (cols <= 127) or 16
+  int32_t planes = 1;     // bit planes of a code: NB
+  int32_t slab_high = 16; // bitmap words per slab: T = 16, 8, 4 or 2
   int64_t rows = 0;
   int32_t cols = 0;
-  int64_t groups = 0;        // ceil(rows / rows_per_group), padded up to a whole slab
-  int64_t slabs = 0;         // Q
-  int64_t words = 0;         // W = ceil(rows / 32)
-  size_t rank_words() const { return (size_t)cols * (size_t)slabs * 32u * (size_t)vec; }
-  int64_t rows_per_slab() const { return (int64_t)rows_per_group * vec; }
-  int64_t words_per_slab() const { return (int64_t)words_per_group * vec; }
-  size_t slab_col_bytes() const { return 128u * (size_t)vec; }  // one column of one slab
+  int64_t slabs = 0;      // Q = ceil(rows / (32 T))
+  int64_t words = 0;      // W = ceil(rows / 32)
+  uint32_t slab_bytes = 0;  // one slab's planes: cols * NB * T words
+  uint32_t pitch_bytes = 0; // from slab to slab
+  size_t rank_words() const { return (size_t)slabs * pitch_bytes / 4; }
+  int64_t rows_per_slab() const { return 32ll * slab_high; }
 };
 
 // Diagnostics: every kernel launch of the library is counted (defined in capi.cpp).
@@ -92,9 +90,13 @@ cudaError_t launch_prepare(const PrepareArgs& a, cudaStream_t s);
 
 // ---- population evaluator ------------------------------------------------------------------
 struct EvalArgs {
-  int32_t cols = 0;          // matrix columns
+  const uint32_t* ranks = nullptr;  // the matrix's bit planes
+  int32_t planes = 0;        // NB
+  int32_t slab_high = 0;     // T
+  int32_t ts = 1;            // slabs per row tile
+  uint32_t pitch_bytes = 0;
+  uint32_t slab_bytes = 0;
   int64_t slabs = 0;         // Q
-  int64_t groups = 0;        // groups incl. slab padding (Q * VEC)
   int64_t words = 0;         // W
   uint32_t n_cand = 0;
   const uint16_t* cand_cols = nullptr;     // device CSR
@@ -103,8 +105,6 @@ struct EvalArgs {
   uint32_t* bitmaps = nullptr;             // device [n_cand][bitmap_stride] or null
   int64_t bitmap_stride = 0;               // words between candidates' bitmaps (>= W)
   int32_t chunk_cols = 0;    // CC: candidate columns staged per chunk
-  int32_t col_box = 0;       // columns per TMA box
-  int32_t n_col_boxes = 0;
   uint32_t stage_bytes = 0;  // bytes of one pipeline stage
   uint32_t smem_bytes = 0;   // dynamic shared memory of the launch
   const uint32_t* err = nullptr;  // per-call error word: non-zero -> do nothing
@@ -113,30 +113,17 @@ struct EvalArgs {
   uint64_t timeout_ns = 1000000000ull;
 };
 
-struct EvalConfig {
-  int width = 8, vec = 4, ts = 1;
-  bool negative = false, bitmaps = true;
-  int grid = 0;
-};
-
 // Tile choice and shared-memory plan for a matrix layout (host).
 int default_tile_slabs(const Layout& L);
-bool plan_eval(const Layout& L, int ts, uint32_t n_cand, int64_t total_cols_hint, int grid,
-               EvalArgs* a, int32_t chunk_override = 0);
+bool plan_eval(const Layout& L, const uint32_t* ranks, int ts, EvalArgs* a,
+               int32_t chunk_override = 0);
 
-cudaError_t launch_eval(const EvalConfig& cfg, const CUtensorMap* tmap, const EvalArgs& a,
-                        cudaStream_t s);
-// one translation unit per rank layout (width, VEC)
-cudaError_t launch_eval_w8v4(const EvalConfig&, const CUtensorMap*, const EvalArgs&, cudaStream_t);
-cudaError_t launch_eval_w16v4(const EvalConfig&, const CUtensorMap*, const EvalArgs&, cudaStream_t);
-cudaError_t launch_eval_w16v2(const EvalConfig&, const CUtensorMap*, const EvalArgs&, cudaStream_t);
-cudaError_t launch_eval_w16v1(const EvalConfig&, const CUtensorMap*, const EvalArgs&, cudaStream_t);
-// Ready every evaluator instantiation of a layout on the current device (shared-memory limit
-// raised, code loaded).
-cudaError_t ready_eval_w8v4();
-cudaError_t ready_eval_w16v4();
-cudaError_t ready_eval_w16v2();
-cudaError_t ready_eval_w16v1();
+// pdl: launch with programmatic stream serialization (the kernel waits for the preparation
+// itself, and has its first tiles copied meanwhile).
+cudaError_t launch_eval(const EvalArgs& a, bool negative, int grid, bool pdl, cudaStream_t s);
+// Ready every evaluator instantiation on the current device (shared-memory limit raised, code
+// loaded).
+cudaError_t ready_eval();
 // Load the list-check kernel's code on the current device.
 cudaError_t ready_prepare();
 
@@ -290,10 +277,9 @@ struct MatrixView {
 };
 // Read-only view of a matrix handle's shape and device words.
 void matrix_view(const ebic_matrix* m, MatrixView* v);
-// Tile choice, launch plan and tensor map for evaluating n_cand candidates on m (the same choice
+// Tile choice and launch plan for evaluating a population on m (the same choice
 // ebic_eval_population makes). Returns EBIC_OK or an error code with the last-error message set.
-int matrix_eval_plan(const ebic_matrix* m, uint32_t n_cand, int64_t total_cols_hint,
-                     EvalArgs* a, EvalConfig* cfg, const CUtensorMap** tmap, int ts_cap = 0);
+int matrix_eval_plan(const ebic_matrix* m, EvalArgs* a);
 // Record the calling thread's last-error message and return `code`.
 int set_last_error(int code, const char* msg);
 

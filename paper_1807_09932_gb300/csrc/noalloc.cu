@@ -53,10 +53,7 @@ int scratch_address(int dev, uint8_t** out) {
                             (std::string("cudaGetSymbolAddress(no-allocation scratch): ") +
                              cudaGetErrorString(e)).c_str());
     }
-    e = ready_eval_w8v4();
-    if (e == cudaSuccess) e = ready_eval_w16v4();
-    if (e == cudaSuccess) e = ready_eval_w16v2();
-    if (e == cudaSuccess) e = ready_eval_w16v1();
+    e = ready_eval();
     if (e == cudaSuccess) e = ready_prepare();
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
@@ -147,15 +144,14 @@ extern "C" int ebic_eval_population_noalloc(const ebic_matrix* m, const uint16_t
                           "cols and offsets must both be host memory or both device memory");
   const uint16_t* dcols = cols;
   const uint32_t* doffs = offsets;
-  int64_t total_hint = 0;
   if (!cols_dev) {
     // host lists: checked here, then staged into the fixed scratch if they fit
     const char* why = check_candidates_host_c(cols, offsets, n_cand, v.L.cols);
     if (why[0]) return set_last_error(EBIC_ERR_INVALID_ARG, why);
-    total_hint = offsets[n_cand];
+    const size_t total = offsets[n_cand];
     const size_t off_bytes = ((size_t)n_cand + 1) * sizeof(uint32_t);
     const size_t col_off = kNoAllocListsOffset + ((off_bytes + 255) / 256) * 256;
-    const size_t need = col_off + (size_t)total_hint * sizeof(uint16_t);
+    const size_t need = col_off + total * sizeof(uint16_t);
     if (need > kNoAllocScratchBytes)
       return set_last_error(
           EBIC_ERR_UNSUPPORTED,
@@ -167,7 +163,7 @@ extern "C" int ebic_eval_population_noalloc(const ebic_matrix* m, const uint16_t
     cudaError_t e = cudaMemcpyAsync(scratch + kNoAllocListsOffset, offsets, off_bytes,
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(scratch + col_off, cols, (size_t)total_hint * sizeof(uint16_t),
+      e = cudaMemcpyAsync(scratch + col_off, cols, total * sizeof(uint16_t),
                           cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_error(e, "staging the population into the scratch");
     doffs = reinterpret_cast<const uint32_t*>(scratch + kNoAllocListsOffset);
@@ -175,9 +171,7 @@ extern "C" int ebic_eval_population_noalloc(const ebic_matrix* m, const uint16_t
   }
 
   EvalArgs a;
-  EvalConfig cfg;
-  const CUtensorMap* tmap = nullptr;
-  rc = matrix_eval_plan(m, n_cand, total_hint, &a, &cfg, &tmap);
+  rc = matrix_eval_plan(m, &a);
   if (rc != EBIC_OK) return rc;
 
   cudaError_t e = cudaMemsetAsync(err, 0, sizeof(uint32_t), s);  // the status word starts at 0
@@ -201,9 +195,7 @@ extern "C" int ebic_eval_population_noalloc(const ebic_matrix* m, const uint16_t
   a.err = err;
   a.err_out = err;
   a.status = v.status;
-  cfg.negative = (flags & EBIC_NEGATIVE_TRENDS) != 0;
-  cfg.bitmaps = bitmaps != nullptr;
-  e = launch_eval(cfg, tmap, a, s);
+  e = launch_eval(a, (flags & EBIC_NEGATIVE_TRENDS) != 0, v.num_sms, true, s);
   if (e != cudaSuccess) return cuda_error(e, "evaluator launch");
   return EBIC_OK;
 }

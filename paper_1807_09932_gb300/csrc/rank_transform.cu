@@ -12,14 +12,13 @@
 // orders like the value (-0 folded onto +0, negatives bit-inverted, positives given the top bit),
 // so ties, signed zeros, infinities and subnormals are exact whatever the FTZ mode.
 //
-// One CTA per slab of rows (VEC row groups). Rows of up to 64 columns: one thread per row sorts
-// its (key, column) pairs with a compare-exchange network in registers and walks the sorted run.
-// Wider rows: each warp takes one row at a time. Up to 256 columns the keys are sorted in
-// registers and shuffles, and each column looks its key up in the sorted run; wider still,
-// (key << 32 | column) pairs are sorted in the warp's shared buffer and walked. In the warp forms
-// a warp prefix count of "first of a new key" flags over the sorted run gives the dense ranks. Ranks are written as bytes/halves into a shared slab tile
-// laid out as the HBM layout (with one padding word per column against bank conflicts), then the
-// tile is copied out with coalesced 32-bit stores, 128*VEC contiguous bytes per column.
+// Rows of up to 64 columns: one thread per row sorts single words (key and column) with a
+// compare-exchange network in registers and walks the sorted run. Wider rows: a warp takes one row
+// at a time, sorts its keys in registers and shuffles, and each column looks its key up in the
+// sorted run; a warp prefix count of "first of a new key" flags over the run gives the dense
+// ranks. Codes are dropped as bytes or halves into a shared tile, whose words a warp then turns
+// into bit planes by 32 x 32 bit transposes (a lane holds a row's code, afterwards a plane's word
+// for 32 rows) and writes out in the layout of ebic_internal.h.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -44,239 +43,183 @@ __device__ __forceinline__ uint32_t order_key(float x, int exclude, float fill) 
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-template <int WIDTH, int VEC>
-__global__ void __launch_bounds__(512) rank_transform_kernel(const float* __restrict__ X,
-                                                            int64_t R, int C, int64_t ld,
-                                                            int exclude, float fill,
-                                                            uint32_t* __restrict__ out,
-                                                            int64_t Q, int N, int nwarps) {
-  constexpr int RPG = WIDTH == 8 ? 128 : 64;  // rows per group
-  constexpr int RPS = RPG * VEC;              // rows per slab
-  constexpr uint32_t MISSING = 0u;  // code of a missing value and of padding rows
-  constexpr int TROW = 32 * VEC + 1;          // padded words per column in the tile
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t* tile = reinterpret_cast<uint32_t*>(smem);
-  unsigned long long* sortbuf =
-      reinterpret_cast<unsigned long long*>(smem + (((size_t)C * TROW * 4 + 15) & ~(size_t)15));
-
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t q = blockIdx.x;
-  unsigned long long* buf = sortbuf + (size_t)warp * N;
-  const int npl = N / 32;  // sorted positions per lane in the ranking pass
-
-  for (int rho = warp; rho < RPS; rho += nwarps) {
-    const int64_t r = q * RPS + rho;
-    const int j = rho / RPG, rr = rho % RPG, l = rr & 31, k = rr >> 5;
-    uint8_t* cell0 = reinterpret_cast<uint8_t*>(tile) + ((size_t)l * VEC + j) * 4 +
-                     (WIDTH == 8 ? k : 2 * k);
-    if (r >= R) {  // padding rows hold the missing code in every column
-      for (int c = lane; c < C; c += 32) {
-        uint8_t* cell = cell0 + (size_t)c * TROW * 4;
-        if (WIDTH == 8) *cell = (uint8_t)MISSING;
-        else *reinterpret_cast<uint16_t*>(cell) = (uint16_t)MISSING;
-      }
-      continue;
-    }
-    const float* row = X + r * ld;
-    for (int i = lane; i < N; i += 32)
-      buf[i] = i < C ? ((unsigned long long)order_key(row[i], exclude, fill) << 32) | (uint32_t)i
-                     : ~0ull;
-    __syncwarp();
-    // bitonic sort, ascending, N a power of two
-    for (int kk = 2; kk <= N; kk <<= 1) {
-      for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-        for (int p = lane; p < N / 2; p += 32) {
-          const int i = 2 * jj * (p / jj) + (p % jj);
-          const int ixj = i + jj;
-          const unsigned long long x = buf[i], y = buf[ixj];
-          const bool up = (i & kk) == 0;
-          if ((x > y) == up) { buf[i] = y; buf[ixj] = x; }
-        }
-        __syncwarp();
-      }
-    }
-    // dense rank: number of distinct keys up to and including this position, minus one
-    const int p0 = lane * npl;
-    uint32_t cnt = 0;
-    for (int t = 0; t < npl; ++t) {
-      const int p = p0 + t;
-      const uint32_t key = (uint32_t)(buf[p] >> 32);
-      const bool fresh = key != kMissingKey && (p == 0 || (uint32_t)(buf[p - 1] >> 32) != key);
-      cnt += fresh;
-    }
-    uint32_t incl = cnt;
+// 32x32 bit transpose across the warp: afterwards bit i of lane j is what bit j of lane i was.
+// Five butterfly stages; in stage s the off-diagonal s x s blocks of every 2s x 2s block swap.
+// rot[t] / sel[t] are the lane's rotation amount and bit mask of stage t (transpose_consts).
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, const uint32_t (&rot)[5],
+                                                const uint32_t (&sel)[5]) {
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= d) incl += v;
-    }
-    uint32_t run = incl - cnt;
-    for (int t = 0; t < npl; ++t) {
-      const int p = p0 + t;
-      const unsigned long long e = buf[p];
-      const uint32_t key = (uint32_t)(e >> 32), c = (uint32_t)e;
-      const bool fresh = key != kMissingKey && (p == 0 || (uint32_t)(buf[p - 1] >> 32) != key);
-      run += fresh;
-      if (c < (uint32_t)C) {
-        const uint32_t rank = key == kMissingKey ? MISSING : run;  // 1-based dense rank
-        uint8_t* cell = cell0 + (size_t)c * TROW * 4;
-        if (WIDTH == 8) *cell = (uint8_t)rank;
-        else *reinterpret_cast<uint16_t*>(cell) = (uint16_t)rank;
-      }
-    }
-    __syncwarp();
+  for (int t = 0; t < 5; ++t) {
+    const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, 16 >> t);
+    const uint32_t r = __funnelshift_l(y, y, rot[t]);  // rotate left
+    x = (x & ~sel[t]) | (r & sel[t]);
   }
-  __syncthreads();
-  // copy out: column c of slab q is 32*VEC contiguous words in HBM
-  const int wpc = 32 * VEC;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)C * wpc; idx += blockDim.x) {
-    const int64_t c = idx / wpc, i = idx % wpc;
-    out[(c * Q + q) * wpc + i] = tile[c * TROW + i];
+  return x;
+}
+
+__device__ __forceinline__ void transpose_consts(int lane, uint32_t (&rot)[5],
+                                                 uint32_t (&sel)[5]) {
+  // bits j with (j & s) != 0, for s = 16, 8, 4, 2, 1
+  const uint32_t right[5] = {0xFFFF0000u, 0xFF00FF00u, 0xF0F0F0F0u, 0xCCCCCCCCu, 0xAAAAAAAAu};
+#pragma unroll
+  for (int t = 0; t < 5; ++t) {
+    const int s = 16 >> t;
+    const bool top = (lane & s) == 0;  // top lanes take the partner's left bits into the right
+    rot[t] = top ? (uint32_t)s : (uint32_t)(32 - s);
+    sel[t] = top ? right[t] : ~right[t];
   }
 }
 
-// The same transform for rows of at most 32*E columns with the sort in registers: lane l holds
-// the row's sorted keys at positions l*E .. l*E+E-1 ("blocked" layout) after a bitonic network
-// whose exchanges are register min/max when partners share a lane (distance < E) and shuffles
-// otherwise. Only the 32-bit keys are sorted: the warp then writes the sorted keys and their
-// dense ranks to its shared buffer, and every lane finds the rank of each of its own columns by a
-// binary search of its key there. Each warp loads its next row while it ranks the current one.
+// Rows of 65 to 1,024 columns (32 E): a warp sorts a row's 32-bit keys in registers, lane l
+// holding positions l*E .. l*E+E-1, with a bitonic network whose every exchange is ascending (each
+// merge begins by comparing position i with its mirror image in the block, i ^ (2^s - 1)): an
+// exchange within a lane is one min and one max, one across lanes a shuffle and a min or max.
 template <int E>
-__device__ __forceinline__ void bitonic_sort_keys(uint32_t (&x)[E], int lane) {
+__device__ __forceinline__ void sort_keys(uint32_t (&x)[E], int lane) {
   constexpr int N = 32 * E;
 #pragma unroll
   for (int kk = 2; kk <= N; kk <<= 1) {
+    // the mirror step
+    if (kk <= E) {
 #pragma unroll
-    for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+      for (int e = 0; e < E; ++e) {
+        const int f = e ^ (kk - 1);
+        if (f < e) continue;
+        const uint32_t lo = min(x[e], x[f]), hi = max(x[e], x[f]);
+        x[e] = lo;
+        x[f] = hi;
+      }
+    } else {
+      const bool lower = (lane & (kk / E / 2)) == 0;
+      uint32_t y[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        y[e] = __shfl_xor_sync(0xFFFFFFFFu, x[E - 1 - e], kk / E - 1);
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[e] = lower ? min(x[e], y[e]) : max(x[e], y[e]);
+    }
+#pragma unroll
+    for (int jj = kk >> 2; jj > 0; jj >>= 1) {
       if (jj < E) {  // partners in this lane: elements e and e | jj
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           if (e & jj) continue;
-          const bool up = ((lane * E + e) & kk) == 0;
-          const uint32_t a = x[e], b = x[e | jj];
-          const uint32_t lo = min(a, b), hi = max(a, b);
-          x[e] = up ? lo : hi;
-          x[e | jj] = up ? hi : lo;
+          const uint32_t lo = min(x[e], x[e | jj]), hi = max(x[e], x[e | jj]);
+          x[e] = lo;
+          x[e | jj] = hi;
         }
       } else {  // partner in lane ^ (jj / E), same element
-        const int d = jj / E;
+        const bool lower = (lane & (jj / E)) == 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-          const int i = lane * E + e;
-          const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[e], d);
-          // the lower index of an ascending pair keeps the smaller key, and so on
-          const bool keep_min = ((i & jj) == 0) == ((i & kk) == 0);
-          x[e] = keep_min ? min(x[e], y) : max(x[e], y);
+          const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[e], jj / E);
+          x[e] = lower ? min(x[e], y) : max(x[e], y);
         }
       }
     }
   }
 }
 
-template <int WIDTH, int VEC, int E>
-__global__ void __launch_bounds__(512) rank_transform_reg_kernel(const float* __restrict__ X,
-                                                                int64_t R, int C, int64_t ld,
-                                                                int exclude, float fill,
-                                                                uint32_t* __restrict__ out,
-                                                                int64_t Q, int nwarps) {
-  constexpr int RPG = WIDTH == 8 ? 128 : 64;  // rows per group
-  constexpr int RPS = RPG * VEC;              // rows per slab
+// One CTA ranks 64 rows (two bitmap words): each warp a row at a time, the next row loaded while
+// it ranks the current one. The warp writes the sorted keys and their dense ranks to its shared
+// buffer, and every lane finds the rank of each of its own columns by a binary search of its key
+// there. The code goes into the tile as a half: word (column, l) has the codes of rows l and
+// 32 + l, one padding word per 32 so that a row's stores (one column per lane) hit 32 banks.
+// Bound by instruction issue: for 512 columns about 480 min/max and 480 shuffle-and-select
+// instructions for the sort and 600 for the search, per row. 50,021 x 457: 459 us (1,328 with
+// (key, column) pairs sorted in shared memory).
+constexpr int kWideWarps = 8;
+template <int E>
+__global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
+    const float* __restrict__ X, int64_t R, int C, int64_t ld, int exclude, float fill,
+    uint32_t* __restrict__ out, int planes, int slab_high, uint32_t pitch_words) {
   constexpr int N = 32 * E;
-  constexpr uint32_t MISSING = 0u;
-  constexpr int TROW = 32 * VEC + 1;
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t* tile = reinterpret_cast<uint32_t*>(smem);
+  constexpr int kRows = 64;
+  constexpr int TROW = 33;
+  extern __shared__ __align__(16) uint32_t smem_w[];
+  uint32_t* const tile = smem_w;  // [C][TROW]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the warp's sorted keys and their dense ranks
-  uint32_t* skey = reinterpret_cast<uint32_t*>(
-                       smem + (((size_t)C * TROW * 4 + 15) & ~(size_t)15)) + (size_t)warp * 2 * N;
-  uint32_t* srank = skey + N;
-  const int64_t q = blockIdx.x;
+  uint32_t* const skey = smem_w + C * TROW + warp * 2 * N;
+  uint32_t* const srank = skey + N;
+  const int64_t r0 = (int64_t)blockIdx.x * kRows;
   // the row's values as loaded: element e of lane l is column e*32 + l (coalesced)
   auto load_row = [&](int rho, float (&v)[E]) {
-    const int64_t r = q * RPS + rho;
+    const int64_t r = r0 + rho;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int c = e * 32 + lane;
-      v[e] = (rho < RPS && r < R && c < C) ? __ldg(X + r * ld + c) : 0.0f;
+      v[e] = (rho < kRows && r < R && c < C) ? __ldg(X + r * ld + c) : 0.0f;
     }
   };
   float cur[E];
   load_row(warp, cur);
-  for (int rho = warp; rho < RPS; rho += nwarps) {
-    const int64_t r = q * RPS + rho;
-    float nxt[E];
-    load_row(rho + nwarps, nxt);  // the warp's next row, while this one is ranked
-    const int j = rho / RPG, rr = rho % RPG, l = rr & 31, k = rr >> 5;
-    uint8_t* cell0 = reinterpret_cast<uint8_t*>(tile) + ((size_t)l * VEC + j) * 4 +
-                     (WIDTH == 8 ? k : 2 * k);
-    if (r >= R) {  // padding rows hold the missing code in every column
-      for (int c = lane; c < C; c += 32) {
-        uint8_t* cell = cell0 + (size_t)c * TROW * 4;
-        if (WIDTH == 8) *cell = (uint8_t)MISSING;
-        else *reinterpret_cast<uint16_t*>(cell) = (uint16_t)MISSING;
-      }
-    } else {
-      uint32_t v[E], x[E];  // keys of the lane's columns; the same, to be sorted
+  for (int rho = warp; rho < kRows; rho += kWideWarps) {
+    uint16_t* const cell0 = reinterpret_cast<uint16_t*>(tile + (rho & 31)) + (rho >> 5);
+    uint32_t v[E], x[E];  // keys of the lane's columns; the same, to be sorted
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        v[e] = e * 32 + lane < C ? order_key(cur[e], exclude, fill) : kMissingKey;
-        x[e] = v[e];
-      }
-      bitonic_sort_keys<E>(x, lane);
-      // dense rank of each sorted position: distinct keys up to and including it (the missing
-      // key, which also pads the row, sorts last and is never counted)
-      const uint32_t prev_last = __shfl_up_sync(0xFFFFFFFFu, x[E - 1], 1);
-      uint32_t fresh = 0, cnt = 0;  // fresh: bit e = position lane*E+e starts a new key
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const uint32_t before = e > 0 ? x[e - 1] : prev_last;
-        const bool f = x[e] != kMissingKey && ((lane == 0 && e == 0) || before != x[e]);
-        fresh |= (uint32_t)f << e;
-        cnt += f;
-      }
-      uint32_t incl = cnt;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= d) incl += t;
-      }
-      uint32_t run = incl - cnt;
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        run += (fresh >> e) & 1u;
-        skey[lane * E + e] = x[e];
-        srank[lane * E + e] = run;
-      }
-      __syncwarp();
-      // each column's rank: the first sorted position holding its key (lower bound)
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int c = e * 32 + lane;
-        if (c >= C) continue;
-        uint32_t rank = MISSING;
-        if (v[e] != kMissingKey) {
-          int pos = 0;
-#pragma unroll
-          for (int step = N / 2; step >= 1; step >>= 1)
-            if (skey[pos + step - 1] < v[e]) pos += step;
-          rank = srank[pos];  // 1-based dense rank
-        }
-        uint8_t* cell = cell0 + (size_t)c * TROW * 4;
-        if (WIDTH == 8) *cell = (uint8_t)rank;
-        else *reinterpret_cast<uint16_t*>(cell) = (uint16_t)rank;
-      }
-      __syncwarp();  // the buffer is rewritten for the next row
+    for (int e = 0; e < E; ++e) {
+      v[e] = e * 32 + lane < C ? order_key(cur[e], exclude, fill) : kMissingKey;
+      x[e] = v[e];
     }
+    load_row(rho + kWideWarps, cur);  // the warp's next row, while this one is ranked
+    if (r0 + rho >= R) {  // padding rows hold the missing code in every column
+      for (int c = lane; c < C; c += 32) cell0[c * (2 * TROW)] = 0u;
+      continue;
+    }
+    sort_keys<E>(x, lane);
+    // dense rank of each sorted position: distinct keys up to and including it (the missing
+    // key, which also pads the row, sorts last and is never counted)
+    const uint32_t prev_last = __shfl_up_sync(0xFFFFFFFFu, x[E - 1], 1);
+    uint32_t fresh = 0, cnt = 0;  // fresh: bit e = position lane*E+e starts a new key
 #pragma unroll
-    for (int e = 0; e < E; ++e) cur[e] = nxt[e];
+    for (int e = 0; e < E; ++e) {
+      const uint32_t before = e > 0 ? x[e - 1] : prev_last;
+      const bool f = x[e] != kMissingKey && ((lane == 0 && e == 0) || before != x[e]);
+      fresh |= (uint32_t)f << e;
+      cnt += f;
+    }
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+      if (lane >= d) incl += t;
+    }
+    uint32_t run = incl - cnt;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      run += (fresh >> e) & 1u;
+      skey[lane * E + e] = x[e];
+      srank[lane * E + e] = run;
+    }
+    __syncwarp();
+    // each column's rank: the first sorted position holding its key (lower bound)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int c = e * 32 + lane;
+      if (c >= C) continue;
+      uint32_t rank = 0u;
+      if (v[e] != kMissingKey) {
+        int pos = 0;
+#pragma unroll
+        for (int step = N / 2; step >= 1; step >>= 1)
+          if (skey[pos + step - 1] < v[e]) pos += step;
+        rank = srank[pos];  // 1-based dense rank
+      }
+      cell0[c * (2 * TROW)] = (uint16_t)rank;
+    }
+    __syncwarp();  // the buffer is rewritten for the next row
   }
   __syncthreads();
-  // copy out: column c of slab q is 32*VEC contiguous words in HBM
-  const int wpc = 32 * VEC;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)C * wpc; idx += blockDim.x) {
-    const int64_t c = idx / wpc, i = idx % wpc;
-    out[(c * Q + q) * wpc + i] = tile[c * TROW + i];
+  // the 64 rows' two words of every plane: after the transpose lane 16 h + p has plane p of word h
+  uint32_t rot[5], sel[5];
+  transpose_consts(lane, rot, sel);
+  const int64_t word = (int64_t)blockIdx.x * 2;
+  uint32_t* const slab = out + word / slab_high * pitch_words + word % slab_high;
+  const int p = lane & 15, h = lane >> 4;
+  for (int c = warp; c < C; c += kWideWarps) {
+    const uint32_t w = transpose32(tile[c * TROW + lane], rot, sel);
+    if (p < planes) slab[((size_t)c * planes + p) * slab_high + h] = w;
   }
 }
 
@@ -303,12 +246,11 @@ __global__ void __launch_bounds__(512) rank_transform_reg_kernel(const float* __
 // a positive value's its bits with the top bit set. Missing values sort last; the walk counts
 // them as one more value, and their columns, known from a bit mask, get code 0 afterwards.
 //
-// Work: each CTA ranks whole slabs of 512 rows, 16 batches of 32 rows (batch b: rows
-// 128 (b / 4) + 32 (b % 4) + lane), and drops the codes as bytes into a shared slab tile laid out
-// [column][chunk][lane], so that lane l always writes bank l, whatever the column; columns C..N-1
-// take the padding words. The tile is copied out with 16-byte stores into the HBM layout (word
-// 4 l + chunk of a column's 128 words of the slab); two tiles, one barrier per slab. Rows of at
-// least 32 columns on 16-byte boundaries (a multiple of four columns) take the TMA form: one CTA
+// Work: each CTA ranks whole slabs of 512 rows, 16 batches of 32 rows (batch b: the rows of the
+// slab's bitmap word b), and drops the codes as bytes into a shared slab tile laid out
+// [column][4][lane], so that lane l always writes bank l, whatever the column; columns C..N-1
+// take the padding words. The tile is written out as bit planes (planes_out); two tiles, one
+// barrier per slab. Rows of at least 32 columns on 16-byte boundaries (a multiple of four columns) take the TMA form: one CTA
 // of 16 warps per SM, each warp's next batch brought into shared memory by TMA while the current
 // one is sorted. Other rows are loaded by each lane straight into registers (8 warps, two CTAs
 // per SM).
@@ -475,14 +417,21 @@ __device__ __forceinline__ void padding_words(uint32_t (&v)[N], uint64_t& missin
   missing = C >= 64 ? ~0ull : ((1ull << C) - 1ull);
 }
 
-// Column c of slab q is 128 contiguous words; word 4 l + j is tile word 32 j + l.
-__device__ __forceinline__ void copy_out_tile(const uint32_t* tile, uint32_t* __restrict__ out,
-                                              int C, int64_t Q, int64_t q, int tid, int nthreads) {
-  for (int i = tid; i < C * 32; i += nthreads) {
-    const int c = i >> 5, l = i & 31;
-    const uint32_t* t = tile + c * 128 + l;
-    const uint4 w = make_uint4(t[0], t[32], t[64], t[96]);
-    *reinterpret_cast<uint4*>(out + ((int64_t)c * Q + q) * 128 + 4 * l) = w;
+// The tile's codes as the slab's bit planes, a warp per column: word (c, j, lane) holds in byte k
+// the code of row lane of bitmap word 4 k + j, so that after the 32 x 32 bit transposes of the
+// column's four words lane 8 k + p has words 4 k .. 4 k + 3 of plane p, one 16-byte store.
+__device__ __forceinline__ void planes_out(const uint32_t* tile, uint32_t* __restrict__ slab,
+                                           int C, int planes, int lane, int warp, int nwarps) {
+  uint32_t rot[5], sel[5];
+  transpose_consts(lane, rot, sel);
+  const int p = lane & 7, k = lane >> 3;
+  for (int c = warp; c < C; c += nwarps) {
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = transpose32(tile[c * 128 + 32 * j + lane], rot, sel);
+    if (p < planes)
+      *reinterpret_cast<uint4*>(slab + (c * planes + p) * 16 + 4 * k) =
+          make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -491,7 +440,7 @@ __device__ __forceinline__ void copy_out_tile(const uint32_t* tile, uint32_t* __
 template <int N, bool EXCL>
 __global__ void __launch_bounds__(kRankThreads, kRankBlocksPerSM) rank_rows_packed_kernel(
     const float* __restrict__ X, int64_t R, int C, int64_t ld, uint32_t fill_bits,
-    uint32_t* __restrict__ out, int64_t Q) {
+    uint32_t* __restrict__ out, int64_t Q, int planes, uint32_t pitch_words) {
   constexpr int kWarps = kRankThreads / 32;
   constexpr int tile_words = N * 128;
   constexpr uint32_t CM = N == 64 ? 63u : 31u;
@@ -504,8 +453,8 @@ __global__ void __launch_bounds__(kRankThreads, kRankBlocksPerSM) rank_rows_pack
   for (int64_t q = blockIdx.x; q < Q; q += gridDim.x, buf ^= 1) {
     uint32_t* tile = tiles + buf * tile_words;
     for (int b = warp; b < kRankSlabRows / 32; b += kWarps) {
-      const int j = b >> 2, k = b & 3;  // chunk, and the byte of the word
-      const int64_t r0 = q * kRankSlabRows + j * 128 + k * 32;
+      const int j = b & 3, k = b >> 2;  // word j, byte k of the column's tile words: see planes_out
+      const int64_t r0 = q * kRankSlabRows + b * 32;
       const bool live = r0 + lane < R;  // a padding row is ranked as a row of missing values
       const float* row = X + (live ? r0 + lane : 0) * ld;
       uint32_t v[N];
@@ -520,7 +469,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankBlocksPerSM) rank_rows_pack
                              sorted_k[warp]);
     }
     __syncthreads();
-    copy_out_tile(tile, out, C, Q, q, threadIdx.x, kRankThreads);
+    planes_out(tile, out + q * pitch_words, C, planes, lane, warp, kWarps);
   }
 }
 
@@ -536,8 +485,8 @@ __global__ void __launch_bounds__(kRankThreads, kRankBlocksPerSM) rank_rows_pack
 template <int N, bool EXCL>
 __global__ void __launch_bounds__(kStagedThreads, 1) rank_rows_tma_kernel(
     const __grid_constant__ CUtensorMap xmap, const float* __restrict__ X, int64_t R, int C,
-    int64_t ld, uint32_t fill_bits, uint32_t* __restrict__ out, int64_t Q,
-    uint32_t* __restrict__ status, uint64_t timeout_ns) {
+    int64_t ld, uint32_t fill_bits, uint32_t* __restrict__ out, int64_t Q, int planes,
+    uint32_t pitch_words, uint32_t* __restrict__ status, uint64_t timeout_ns) {
   constexpr int NB = N / 32;                       // 32-column boxes per row
   constexpr uint32_t kBoxBytes = 32u * 128u;        // 32 rows of 128 bytes
   constexpr uint32_t kStageBytes = NB * kBoxBytes;
@@ -549,7 +498,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) rank_rows_tma_kernel(
   __shared__ uint32_t sorted_w[kStagedWarps][N];
   __shared__ uint32_t sorted_k[kStagedWarps][N];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = warp >> 2, k = warp & 3;  // the warp's chunk and byte in every slab
+  const int j = warp & 3, k = warp >> 2;  // the warp's word and byte in every slab (planes_out)
   uint8_t* sbase = sraw + ((1024u - (dev::smem_addr(sraw) & 1023u)) & 1023u);
   uint8_t* stage = sbase + warp * kStageBytes;
   uint32_t* tiles = reinterpret_cast<uint32_t*>(sbase + kStagedWarps * kStageBytes);
@@ -560,13 +509,13 @@ __global__ void __launch_bounds__(kStagedThreads, 1) rank_rows_tma_kernel(
   }
   __syncwarp();
   auto issue = [&](int64_t q) {  // lane 0: the warp's batch of slab q
-    const int32_t y = (int32_t)(q * kRankSlabRows + j * 128 + k * 32);
+    const int32_t y = (int32_t)(q * kRankSlabRows + warp * 32);
     dev::mbar_arrive_expect_tx(bar, kStageBytes);
 #pragma unroll
     for (int bx = 0; bx < NB; ++bx) dev::tma_load_2d(stage + bx * kBoxBytes, &xmap, bar, bx * 32, y);
   };
   // a batch whose rows are all padding is not staged (its rows are never read)
-  auto staged = [&](int64_t q) { return q * kRankSlabRows + j * 128 + k * 32 < R; };
+  auto staged = [&](int64_t q) { return q * kRankSlabRows + warp * 32 < R; };
   int64_t q = blockIdx.x;
   uint32_t parity = 0;
   bool pending = false, bad = false;  // a copy is in flight; a wait of this warp expired
@@ -577,7 +526,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) rank_rows_tma_kernel(
   int buf = 0;
   for (; q < Q; q += gridDim.x, buf ^= 1) {
     uint32_t* tile = tiles + buf * tile_words;
-    const int64_t r0 = q * kRankSlabRows + j * 128 + k * 32;
+    const int64_t r0 = q * kRankSlabRows + warp * 32;
     const bool live = r0 + lane < R;
     if (pending && !bad) {
       if (dev::mbar_wait_bounded(bar, parity, timeout_ns)) {
@@ -619,7 +568,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) rank_rows_tma_kernel(
                            reinterpret_cast<uint8_t*>(tile + j * 32) + k, lane, sorted_w[warp],
                            sorted_k[warp]);
     __syncthreads();
-    copy_out_tile(tile, out, C, Q, q, threadIdx.x, kStagedThreads);
+    planes_out(tile, out + q * pitch_words, C, planes, lane, warp, kStagedWarps);
   }
   if (pending) (void)dev::mbar_wait_bounded(bar, parity, timeout_ns);  // none outlives the CTA
   if (bad && lane == 0) atomicOr(status, kErrTimeout);
@@ -682,7 +631,7 @@ cudaError_t launch_rank_packed_as(const Layout& L, const float* dX, int64_t ld, 
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(L.slabs, num_sms));
     count_launch();
     kern<<<grid, kStagedThreads, smem, s>>>(map, dX, L.rows, L.cols, ld, fb, ranks, L.slabs,
-                                            status, 1000000000ull);
+                                            L.planes, L.pitch_bytes / 4, status, 1000000000ull);
     return cudaGetLastError();
   }
   constexpr size_t smem = (size_t)2 * N * 128 * 4;
@@ -696,7 +645,8 @@ cudaError_t launch_rank_packed_as(const Layout& L, const float* dX, int64_t ld, 
   const int grid =
       (int)std::max<int64_t>(1, std::min<int64_t>(L.slabs, kRankBlocksPerSM * (int64_t)num_sms));
   count_launch();
-  kern<<<grid, kRankThreads, smem, s>>>(dX, L.rows, L.cols, ld, fb, ranks, L.slabs);
+  kern<<<grid, kRankThreads, smem, s>>>(dX, L.rows, L.cols, ld, fb, ranks, L.slabs, L.planes,
+                                        L.pitch_bytes / 4);
   return cudaGetLastError();
 }
 
@@ -708,54 +658,21 @@ cudaError_t launch_rank_packed(const Layout& L, const float* dX, int64_t ld, int
                  : launch_rank_packed_as<N, false>(L, dX, ld, fill, ranks, status, num_sms, s);
 }
 
-template <int WIDTH, int VEC, int E>
-cudaError_t launch_rank_reg(const Layout& L, const float* dX, int64_t ld, int exclude, float fill,
-                            uint32_t* ranks, cudaStream_t s) {
-  const size_t tile = (((size_t)L.cols * (32 * VEC + 1) * 4) + 15) & ~(size_t)15;
-  const size_t per_warp = (size_t)2 * 32 * E * 4;  // sorted keys and their ranks
-  int nwarps = (int)((kSmemDynMax - tile) / per_warp);
-  if (nwarps > 16) nwarps = 16;
-  if (nwarps < 1) return cudaErrorInvalidConfiguration;
-  const size_t smem = tile + per_warp * nwarps;
-  auto kern = rank_transform_reg_kernel<WIDTH, VEC, E>;
+template <int E>
+cudaError_t launch_rank_wide(const Layout& L, const float* dX, int64_t ld, int exclude, float fill,
+                             uint32_t* ranks, cudaStream_t s) {
+  const size_t smem = ((size_t)L.cols * 33 + (size_t)kWideWarps * 2 * 32 * E) * 4;
+  if (smem > (size_t)kSmemDynMax) return cudaErrorInvalidConfiguration;
+  const int64_t blocks = L.slabs * (L.slab_high / 2);
+  if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
+  auto kern = rank_wide_kernel<E>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
   count_launch();
-  kern<<<(unsigned)L.slabs, nwarps * 32, smem, s>>>(dX, L.rows, L.cols, ld, exclude, fill, ranks,
-                                                    L.slabs, nwarps);
-  return cudaGetLastError();
-}
-
-template <int WIDTH, int VEC>
-cudaError_t launch_rank_layout(const Layout& L, const float* dX, int64_t ld, int exclude,
-                               float fill, uint32_t* ranks, uint32_t* status, int num_sms,
-                               cudaStream_t s) {
-  if (WIDTH == 8 && VEC == 4) {
-    if (L.cols <= 32)
-      return launch_rank_packed<32>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-    if (L.cols <= 64)
-      return launch_rank_packed<64>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-  }
-  if (L.cols <= 32) return launch_rank_reg<WIDTH, VEC, 1>(L, dX, ld, exclude, fill, ranks, s);
-  if (L.cols <= 64) return launch_rank_reg<WIDTH, VEC, 2>(L, dX, ld, exclude, fill, ranks, s);
-  if (L.cols <= 128) return launch_rank_reg<WIDTH, VEC, 4>(L, dX, ld, exclude, fill, ranks, s);
-  if (L.cols <= 256) return launch_rank_reg<WIDTH, VEC, 8>(L, dX, ld, exclude, fill, ranks, s);
-  int N = 32;
-  while (N < L.cols) N <<= 1;
-  const size_t tile_bytes = (((size_t)L.cols * (32 * VEC + 1) * 4) + 15) & ~(size_t)15;
-  const size_t per_warp = (size_t)N * 8;
-  int nwarps = (int)((kSmemDynMax - tile_bytes) / per_warp);
-  if (nwarps > 16) nwarps = 16;
-  if (nwarps < 1) return cudaErrorInvalidConfiguration;
-  const size_t smem = tile_bytes + per_warp * nwarps;
-  auto kern = rank_transform_kernel<WIDTH, VEC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  count_launch();
-  kern<<<(unsigned)L.slabs, nwarps * 32, smem, s>>>(dX, L.rows, L.cols, ld, exclude, fill, ranks,
-                                                    L.slabs, N, nwarps);
+  kern<<<(unsigned)blocks, kWideWarps * 32, smem, s>>>(dX, L.rows, L.cols, ld, exclude, fill,
+                                                       ranks, L.planes, L.slab_high,
+                                                       L.pitch_bytes / 4);
   return cudaGetLastError();
 }
 
@@ -764,14 +681,15 @@ cudaError_t launch_rank_layout(const Layout& L, const float* dX, int64_t ld, int
 cudaError_t launch_rank_transform(const Layout& L, const float* dX, int64_t ld, int exclude,
                                   float fill, uint32_t* ranks, uint32_t* status, int num_sms,
                                   cudaStream_t s) {
-  if (L.width == 8)
-    return launch_rank_layout<8, 4>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-  switch (L.vec) {
-    case 4: return launch_rank_layout<16, 4>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-    case 2: return launch_rank_layout<16, 2>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-    case 1: return launch_rank_layout<16, 1>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
-    default: return cudaErrorInvalidValue;
-  }
+  if (L.cols <= 32)
+    return launch_rank_packed<32>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
+  if (L.cols <= 64)
+    return launch_rank_packed<64>(L, dX, ld, exclude, fill, ranks, status, num_sms, s);
+  if (L.cols <= 128) return launch_rank_wide<4>(L, dX, ld, exclude, fill, ranks, s);
+  if (L.cols <= 256) return launch_rank_wide<8>(L, dX, ld, exclude, fill, ranks, s);
+  if (L.cols <= 512) return launch_rank_wide<16>(L, dX, ld, exclude, fill, ranks, s);
+  if (L.cols <= 1024) return launch_rank_wide<32>(L, dX, ld, exclude, fill, ranks, s);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace ebic
