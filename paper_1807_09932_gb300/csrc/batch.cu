@@ -322,7 +322,7 @@ __device__ __forceinline__ void batch_tile(const uint8_t* stage, const BatchReq&
   const uint32_t group = 32u / (uint32_t)min(32, q.slab_high * q.ts);  // candidates per warp
   uint32_t c = (uint32_t)warp * group;
   eval_tile<0, 0, NEG>(sh, stage, ccols, coffs, lo, nc, tile * q.ts * q.slab_high, q.words,
-                       q.counts, q.bitmaps, q.words, lane, [&]() {
+                       q.counts, q.bitmaps, lane, [&]() {
                          const uint32_t r = c;
                          c += kBatchWarps * group;
                          return r;

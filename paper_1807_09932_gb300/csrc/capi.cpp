@@ -368,7 +368,6 @@ bool plan_eval(const Layout& L, const uint32_t* ranks, int ts, EvalArgs* a,
   a->slab_bytes = L.slab_bytes;
   a->slabs = L.slabs;
   a->words = L.words;
-  a->bitmap_stride = L.words;
   a->chunk_cols = (int32_t)cc;
   a->stage_bytes = (uint32_t)stage;
   a->smem_bytes =
@@ -406,11 +405,9 @@ const char* check_candidates_host_c(const uint16_t* cols, const uint32_t* offset
 
 }  // namespace ebic
 
-// ebic_eval_population with the candidates' bitmaps `bitmap_stride` words apart (the pair table
-// is built through this with its padded stride).
 static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
-                         uint32_t n_cand, uint32_t flags, uint32_t* counts, uint32_t* bitmaps,
-                         int64_t bitmap_stride, void* stream) {
+                                uint32_t n_cand, uint32_t flags, uint32_t* counts,
+                                uint32_t* bitmaps, void* stream) {
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
   if (flags & ~(EBIC_NEGATIVE_TRENDS | EBIC_EVAL_DIRECT))
     return fail(EBIC_ERR_INVALID_ARG, "unknown eval flag");
@@ -460,10 +457,10 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
   uint32_t* dbitmaps = nullptr;
   EBIC_CUDA(out_buffer(counts, n_cand, dev, sc, &dcounts, &counts_host));
   if (bitmaps)
-    EBIC_CUDA(out_buffer(bitmaps, (size_t)n_cand * bitmap_stride, dev, sc, &dbitmaps,
+    EBIC_CUDA(out_buffer(bitmaps, (size_t)n_cand * L.words, dev, sc, &dbitmaps,
                          &bitmaps_host));
 
-  const bool use_pairs = m->pairs && !(flags & EBIC_EVAL_DIRECT) && bitmap_stride == L.words;
+  const bool use_pairs = m->pairs && !(flags & EBIC_EVAL_DIRECT);
   const bool neg = (flags & EBIC_NEGATIVE_TRENDS) != 0;
   uint32_t* dterms = nullptr;  // the pair-table term lists, built by the preparation kernel
   if (use_pairs)
@@ -508,7 +505,6 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     a.cand_offsets = doffs;
     a.counts = dcounts;
     a.bitmaps = dbitmaps;
-    a.bitmap_stride = bitmap_stride;
     a.err = err;
     a.err_out = err;
     a.status = m->status;
@@ -520,7 +516,7 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     if (counts_host)
       EBIC_CUDA(cudaMemcpyAsync(counts, dcounts, (size_t)n_cand * 4, cudaMemcpyDeviceToHost, s));
     if (bitmaps_host)
-      EBIC_CUDA(cudaMemcpyAsync(bitmaps, dbitmaps, (size_t)n_cand * bitmap_stride * 4,
+      EBIC_CUDA(cudaMemcpyAsync(bitmaps, dbitmaps, (size_t)n_cand * L.words * 4,
                                 cudaMemcpyDeviceToHost, s));
     uint32_t bits = 0;
     EBIC_CUDA(cudaMemcpyAsync(&bits, err, 4, cudaMemcpyDeviceToHost, s));
@@ -662,8 +658,7 @@ int ebic_eval_population(const ebic_matrix* cm, const uint16_t* cols, const uint
                          void* stream) {
   ebic_matrix* m = const_cast<ebic_matrix*>(cm);
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
-  return eval_population_impl(m, cols, offsets, n_cand, flags, counts, bitmaps, m->L.words,
-                              stream);
+  return eval_population_impl(m, cols, offsets, n_cand, flags, counts, bitmaps, stream);
 }
 
 }  // extern "C"
@@ -1132,38 +1127,18 @@ int ebic_matrix_build_pairs(ebic_matrix* m, uint64_t max_bytes, void* stream, ui
     return fail(EBIC_ERR_UNSUPPORTED, "the pair table would exceed 2^32 words");
   DeviceGuard g(m->device);
   if (m->pairs) return EBIC_OK;
-  // the population of all ordered pairs (a, b), a != b, and of all singles (a), in table order
-  const uint32_t C = (uint32_t)L.cols, n = C * C;
-  std::vector<uint16_t> cols;
-  std::vector<uint32_t> offs(1, 0u);
-  cols.reserve((size_t)2 * n);
-  for (uint32_t a = 0; a < C; ++a)
-    for (uint32_t b = 0; b < C; ++b) {
-      cols.push_back((uint16_t)a);
-      if (b != a) cols.push_back((uint16_t)b);
-      offs.push_back((uint32_t)cols.size());
-    }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* table = nullptr;
-  uint32_t* counts = nullptr;
   cudaError_t e = cudaMalloc(&table, need);
-  if (e == cudaSuccess) e = cudaMalloc(&counts, (size_t)n * 4);
-  if (e == cudaSuccess) e = cudaMemsetAsync(table, 0, rows, s);  // the rows' padding words
-  if (e == cudaSuccess)  // the all-ones row after the table
-    e = cudaMemsetAsync(reinterpret_cast<char*>(table) + rows, 0xFF, (size_t)kOnesWords * 4, s);
-  if (e != cudaSuccess) {
-    if (table) cudaFree(table);
-    if (counts) cudaFree(counts);
-    return cuda_fail(e, "pair table allocation");
+  if (e != cudaSuccess) return cuda_fail(e, "pair table allocation");
+  {
+    Timed t(EBIC_TIMING_EVALUATE, s);
+    e = launch_pair_build(L, m->ranks, table, (uint32_t)stride, m->num_sms, s);
   }
-  int rc = eval_population_impl(m, cols.data(), offs.data(), n, EBIC_EVAL_DIRECT, counts, table,
-                                stride, stream);
-  cudaError_t e2 = cudaStreamSynchronize(s);
-  cudaFree(counts);
-  if (rc == EBIC_OK && e2 != cudaSuccess) rc = cuda_fail(e2, "pair table build");
-  if (rc != EBIC_OK) {
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
     cudaFree(table);
-    return rc;
+    return cuda_fail(e, "pair table build");
   }
   m->pairs = table;
   m->pair_stride = (uint32_t)stride;

@@ -102,8 +102,7 @@ struct EvalArgs {
   const uint16_t* cand_cols = nullptr;     // device CSR
   const uint32_t* cand_offsets = nullptr;  // device CSR
   uint32_t* counts = nullptr;              // device, zeroed before the launch
-  uint32_t* bitmaps = nullptr;             // device [n_cand][bitmap_stride] or null
-  int64_t bitmap_stride = 0;               // words between candidates' bitmaps (>= W)
+  uint32_t* bitmaps = nullptr;             // device [n_cand][words] or null
   int32_t chunk_cols = 0;    // CC: candidate columns staged per chunk
   uint32_t stage_bytes = 0;  // bytes of one pipeline stage
   uint32_t smem_bytes = 0;   // dynamic shared memory of the launch
@@ -177,6 +176,11 @@ struct PairArgs {
 // the stream itself, so its launch overlaps that kernel's tail).
 cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pdl,
                              cudaStream_t s);
+
+// Builds the pair table (rows of `stride` words and the all-ones row after them) from a matrix's
+// bit planes.
+cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,
+                              uint32_t stride, int num_sms, cudaStream_t s);
 
 // Preparation of the fused pass, one launch: checks the candidate list and (check_arch) the
 // archive list, zeroes counts, overlaps and archive counts, writes for every candidate the mask

@@ -132,7 +132,7 @@ __device__ __forceinline__ void eval_tile(const TileShape& sh, const uint8_t* st
                                           const uint16_t* ccols, const uint16_t* coffs,
                                           uint32_t lo, uint32_t c1, int64_t first_word,
                                           int64_t n_words, uint32_t* counts, uint32_t* bitmaps,
-                                          int64_t bitmap_stride, int lane, Take take) {
+                                          int lane, Take take) {
   const Walk<NB, T> walk{sh};
   const int t = walk.words();
   const int tile_words = t * sh.slabs;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void eval_tile(const TileShape& sh, const uint8_t* st
       const uint32_t x = walk.template chain<NEG>(base, ccols + o, in ? L : 0);
       cnt += __popc(x);
       if (bitmaps && in)
-        bitmaps[(size_t)(lo + ci) * (size_t)bitmap_stride + first_word + w] = x;
+        bitmaps[(size_t)(lo + ci) * (size_t)n_words + first_word + w] = x;
     }
     if (seg == 32) {
       cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
@@ -269,8 +269,8 @@ __global__ void __launch_bounds__(kEvalThreads, 1) eval_population_kernel(const 
       const uint32_t c0 = (uint32_t)((uint64_t)nc * s0 / kItemUnits);
       const uint32_t c1 = (uint32_t)((uint64_t)nc * s1 / kItemUnits);
       eval_tile<NB, T, NEG>(sh, s ? stage1 : stage0, ccols, coffs, lo, c1,
-                            tile * a.ts * sh.words, a.words, a.counts, a.bitmaps,
-                            a.bitmap_stride, lane, [&]() {
+                            tile * a.ts * sh.words, a.words, a.counts, a.bitmaps, lane,
+                            [&]() {
                               uint32_t u = 0;
                               if (lane == 0) u = atomicAdd(&next_s[s], group);
                               return c0 + __shfl_sync(0xFFFFFFFFu, u, 0);
