@@ -121,16 +121,25 @@ __device__ __forceinline__ void sort_keys(uint32_t (&x)[E], int lane) {
 }
 
 // One CTA ranks 64 rows (two bitmap words): each warp a row at a time, the next row loaded while
-// it ranks the current one. The warp writes the sorted keys and their dense ranks to its shared
-// buffer, and every lane finds the rank of each of its own columns by a binary search of its key
-// there. The code goes into the tile as a half: word (column, l) has the codes of rows l and
-// 32 + l, one padding word per 32 so that a row's stores (one column per lane) hit 32 banks.
-// Bound by instruction issue: for 512 columns about 480 min/max and 480 shuffle-and-select
-// instructions for the sort and 600 for the search, per row. 50,021 x 457: 459 us (1,328 with
-// (key, column) pairs sorted in shared memory).
-constexpr int kWideWarps = 8;
+// it ranks the current one. The warp writes the sorted keys to its shared buffer, and every lane
+// finds each of its own columns' keys there: first the lane that holds it, by a binary search of
+// the 32 lanes' last keys, then its place among that lane's E. Position l*E + e is kept at word
+// e*32 + l, so the stores are conflict-free and the search over lanes reads 32 neighbouring words
+// (different words never meet in a bank); only the log2 E steps within a lane's keys, a column of
+// one bank, can conflict. The dense rank of the place comes from the holding lane's registers by
+// two shuffles. The code goes into the tile as a half: word (column, l) has the codes of rows l
+// and 32 + l, one padding word per 32 so that a row's stores (one column per lane) hit 32 banks.
+// Bound by instruction issue and shared-memory wavefronts in about equal parts: for 512 columns
+// about 480 min/max and 480 shuffle-and-select instructions for the sort and 700 for the search,
+// per row. 50,021 x 457 240 us, 100,000 x 300 383, 20,000 x 832 278, 200,000 x 127 162 (library
+// events); with the sorted keys in order, searched as one run, and their ranks beside them 425,
+// 560, 755 and 176 (61 of 85 million wavefronts were bank conflicts); 50,021 x 457 with (key,
+// column) pairs sorted in shared memory 1,328. Three CTAs per SM up to 512 columns, one of 16
+// warps beyond.
 template <int E>
-__global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
+constexpr int kWideWarps = E == 32 ? 16 : 8;
+template <int E>
+__global__ void __launch_bounds__(kWideWarps<E> * 32, E == 32 ? 1 : E == 16 ? 3 : 4) rank_wide_kernel(
     const float* __restrict__ X, int64_t R, int C, int64_t ld, int exclude, float fill,
     uint32_t* __restrict__ out, int planes, int slab_high, uint32_t pitch_words) {
   constexpr int N = 32 * E;
@@ -139,9 +148,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
   extern __shared__ __align__(16) uint32_t smem_w[];
   uint32_t* const tile = smem_w;  // [C][TROW]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // the warp's sorted keys and their dense ranks
-  uint32_t* const skey = smem_w + C * TROW + warp * 2 * N;
-  uint32_t* const srank = skey + N;
+  uint32_t* const skey = smem_w + C * TROW + warp * N;  // the warp's sorted keys
   const int64_t r0 = (int64_t)blockIdx.x * kRows;
   // the row's values as loaded: element e of lane l is column e*32 + l (coalesced)
   auto load_row = [&](int rho, float (&v)[E]) {
@@ -154,7 +161,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
   };
   float cur[E];
   load_row(warp, cur);
-  for (int rho = warp; rho < kRows; rho += kWideWarps) {
+  for (int rho = warp; rho < kRows; rho += kWideWarps<E>) {
     uint16_t* const cell0 = reinterpret_cast<uint16_t*>(tile + (rho & 31)) + (rho >> 5);
     uint32_t v[E], x[E];  // keys of the lane's columns; the same, to be sorted
 #pragma unroll
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
       v[e] = e * 32 + lane < C ? order_key(cur[e], exclude, fill) : kMissingKey;
       x[e] = v[e];
     }
-    load_row(rho + kWideWarps, cur);  // the warp's next row, while this one is ranked
+    load_row(rho + kWideWarps<E>, cur);  // the warp's next row, while this one is ranked
     if (r0 + rho >= R) {  // padding rows hold the missing code in every column
       for (int c = lane; c < C; c += 32) cell0[c * (2 * TROW)] = 0u;
       continue;
@@ -185,28 +192,29 @@ __global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
       const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
       if (lane >= d) incl += t;
     }
-    uint32_t run = incl - cnt;
+    const uint32_t before_lane = incl - cnt;  // distinct keys in lower lanes
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      run += (fresh >> e) & 1u;
-      skey[lane * E + e] = x[e];
-      srank[lane * E + e] = run;
-    }
+    for (int e = 0; e < E; ++e) skey[e * 32 + lane] = x[e];
     __syncwarp();
-    // each column's rank: the first sorted position holding its key (lower bound)
+    // each column's rank: the first sorted position holding its key (it is there, so the search
+    // never passes the last one)
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int c = e * 32 + lane;
-      if (c >= C) continue;
-      uint32_t rank = 0u;
-      if (v[e] != kMissingKey) {
-        int pos = 0;
+      const uint32_t* at = skey;
 #pragma unroll
-        for (int step = N / 2; step >= 1; step >>= 1)
-          if (skey[pos + step - 1] < v[e]) pos += step;
-        rank = srank[pos];  // 1-based dense rank
-      }
-      cell0[c * (2 * TROW)] = (uint16_t)rank;
+      for (int step = 16; step >= 1; step >>= 1)
+        if (at[(E - 1) * 32 + step - 1] < v[e]) at += step;
+      const int holder = (int)(at - skey);
+#pragma unroll
+      for (int step = E / 2; step >= 1; step >>= 1)
+        if (at[(step - 1) * 32] < v[e]) at += step * 32;
+      const int place = (int)(at - skey) >> 5;
+      const uint32_t f = __shfl_sync(0xFFFFFFFFu, fresh, holder);
+      const uint32_t below = __shfl_sync(0xFFFFFFFFu, before_lane, holder);
+      // 1-based dense rank: fresh keys up to and including the place
+      const uint32_t rank = below + __popc(f & (0xFFFFFFFFu >> (31 - place)));
+      const int c = e * 32 + lane;
+      if (c < C) cell0[c * (2 * TROW)] = (uint16_t)(v[e] == kMissingKey ? 0u : rank);
     }
     __syncwarp();  // the buffer is rewritten for the next row
   }
@@ -217,7 +225,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) rank_wide_kernel(
   const int64_t word = (int64_t)blockIdx.x * 2;
   uint32_t* const slab = out + word / slab_high * pitch_words + word % slab_high;
   const int p = lane & 15, h = lane >> 4;
-  for (int c = warp; c < C; c += kWideWarps) {
+  for (int c = warp; c < C; c += kWideWarps<E>) {
     const uint32_t w = transpose32(tile[c * TROW + lane], rot, sel);
     if (p < planes) slab[((size_t)c * planes + p) * slab_high + h] = w;
   }
@@ -661,7 +669,7 @@ cudaError_t launch_rank_packed(const Layout& L, const float* dX, int64_t ld, int
 template <int E>
 cudaError_t launch_rank_wide(const Layout& L, const float* dX, int64_t ld, int exclude, float fill,
                              uint32_t* ranks, cudaStream_t s) {
-  const size_t smem = ((size_t)L.cols * 33 + (size_t)kWideWarps * 2 * 32 * E) * 4;
+  const size_t smem = ((size_t)L.cols * 33 + (size_t)kWideWarps<E> * 32 * E) * 4;
   if (smem > (size_t)kSmemDynMax) return cudaErrorInvalidConfiguration;
   const int64_t blocks = L.slabs * (L.slab_high / 2);
   if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
@@ -670,7 +678,7 @@ cudaError_t launch_rank_wide(const Layout& L, const float* dX, int64_t ld, int e
                                        (int)smem);
   if (e != cudaSuccess) return e;
   count_launch();
-  kern<<<(unsigned)blocks, kWideWarps * 32, smem, s>>>(dX, L.rows, L.cols, ld, exclude, fill,
+  kern<<<(unsigned)blocks, kWideWarps<E> * 32, smem, s>>>(dX, L.rows, L.cols, ld, exclude, fill,
                                                        ranks, L.planes, L.slab_high,
                                                        L.pitch_bytes / 4);
   return cudaGetLastError();
