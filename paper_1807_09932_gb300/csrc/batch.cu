@@ -61,8 +61,13 @@ struct BatchReq {
   uint64_t* share;                  // scratch: [n_cand] members sharing a column with each
   uint32_t n_arch;
   uint32_t ov_stride;               // n_arch rounded up to even
+  uint32_t copy_base;               // sum of the archive copy units of the requests before it
   uint32_t* terms;                  // pair-table requests: [n_cand][term_slots(neg)] scratch
 };
+
+// Archive copies are cut into units of one padded row's kCopyWords words, a warp each.
+constexpr uint32_t kCopyWords = 512;
+static_assert(kPairRangeWords % kCopyWords == 0, "padded rows are whole copy units");
 
 struct BatchHeader {
   uint32_t n_req;
@@ -73,6 +78,7 @@ struct BatchHeader {
   uint32_t* zero;                 // the fitness requests' counters, one block of n_zero words
   unsigned long long n_zero;
   uint32_t n_fit;                 // requests with a fitness output (set by the host)
+  uint32_t n_copy;                // archive copy units of all requests
 };
 
 constexpr int kCheckWarps = 8;     // warps per block of the check kernel
@@ -83,6 +89,16 @@ __device__ __forceinline__ uint32_t find_request(const BatchReq* reqs, uint32_t 
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) / 2;
     if (reqs[mid].cand_base <= cand) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+// The request whose copy units include `unit` (requests without an archive have none).
+__device__ __forceinline__ uint32_t find_copy(const BatchReq* reqs, uint32_t n, uint32_t unit) {
+  uint32_t lo = 0, hi = n;  // last request with copy_base <= unit
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (reqs[mid].copy_base <= unit) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -176,16 +192,33 @@ __global__ void __launch_bounds__(kCheckWarps * 32)
       }
     }
   }
-  // the fitness requests: counters zeroed, archives copied into rows of the table's stride, the
-  // column -> member masks, and the archive lists checked like candidate lists
+  // the fitness requests' counters
   const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t nthreads = (size_t)gridDim.x * blockDim.x;
   for (size_t i = tid; i < hdr->n_zero; i += nthreads) hdr->zero[i] = 0u;
-  // the requests with an archive, found 32 at a time (a lane per request, one ballot) rather
-  // than by one dependent load per request; every warp finds the same ones
-  // The archive copy of a request takes every thread; its column -> member masks and its list
-  // check take one block (the request's ordinal among them, modulo the grid), which loads every
-  // (member, position) of the list in one round and builds the masks in shared memory.
+  // the archives, copied into rows of the table's stride with zero padding (an even number of
+  // rows): a warp per unit of 512 words, all its loads in flight, whatever request it falls in
+  // (a request at a time with the whole grid cost a round of dependent loads per request: this
+  // kernel took 109 us for 64 requests with archives, 47 so)
+  for (uint32_t u = blockIdx.x * kCheckWarps + warp; u < hdr->n_copy; u += nwarps) {
+    const BatchReq& q = reqs[find_copy(reqs, n_req, u)];
+    const uint32_t local = u - q.copy_base, pieces = q.pair_stride / kCopyWords;
+    const uint32_t m = local / pieces, w0 = (local - m * pieces) * kCopyWords + lane;
+    const uint32_t* src = q.arch_src + (uint64_t)m * (uint64_t)q.words;
+    uint32_t* dst = q.arch_pad + (uint64_t)m * q.pair_stride;
+    uint32_t v[kCopyWords / 32];
+#pragma unroll
+    for (uint32_t k = 0; k < kCopyWords / 32; ++k) {
+      const uint32_t w = w0 + 32u * k;
+      v[k] = m < q.n_arch && w < (uint64_t)q.words ? src[w] : 0u;
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < kCopyWords / 32; ++k) dst[w0 + 32u * k] = v[k];
+  }
+  // The column -> member masks and the list check of a request with an archive take one block
+  // (the request's ordinal among them, modulo the grid), which loads every (member, position) of
+  // the list in one round and builds the masks in shared memory. Those requests are found 32 at
+  // a time (a lane per request, one ballot); every warp finds the same ones.
   __shared__ unsigned long long cmask[kMaxCols];
   uint32_t ordinal = 0;
   for (uint32_t r0 = 0; r0 < n_req; r0 += 32) {
@@ -193,10 +226,8 @@ __global__ void __launch_bounds__(kCheckWarps * 32)
     const bool has = rl < n_req && reqs[rl].fitness != nullptr && reqs[rl].n_arch != 0;
     for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, has); todo; todo &= todo - 1u, ++ordinal) {
       const uint32_t r = r0 + (uint32_t)(__ffs(todo) - 1);
-      const BatchReq& q = reqs[r];
-      prepdev::copy_archive_padded(q.arch_src, q.arch_pad, q.n_arch, q.words, q.pair_stride, tid,
-                                   nthreads);
       if (ordinal % gridDim.x != blockIdx.x) continue;  // block-uniform
+      const BatchReq& q = reqs[r];
       const uint32_t* ao = q.arch_offsets;
       const uint32_t na = q.n_arch, atot = ao[na];
       const int pc = q.pair_cols;
@@ -585,33 +616,44 @@ __global__ void __launch_bounds__(pairdev::kPairThreads, 1)
   }
 }
 
-// F_c of every candidate of the fitness requests, a warp per candidate (as ebic_eval_fitness's
-// finalize), after the batched pair pass. Requests that failed their check get no fitness.
-__global__ void batch_fitness_kernel(const BatchReq* __restrict__ reqs,
-                                     const BatchHeader* __restrict__ hdr,
-                                     const uint32_t* __restrict__ req_err) {
-  const int lane = threadIdx.x & 31;
+// F_c of every candidate of the fitness requests (as ebic_eval_fitness's finalize), after the
+// batched pair pass, a thread per candidate of the whole batch: its loads depend on nothing but
+// its request, so a batch takes a few rounds of loads whatever its number of requests (a warp per
+// candidate, one request after the other, took a round per request: 106 us for 64 requests and
+// 109,000 candidates, now 9). Requests that failed their check get no fitness.
+__global__ void __launch_bounds__(256)
+    batch_fitness_kernel(const BatchReq* __restrict__ reqs, const BatchHeader* __restrict__ hdr,
+                         const uint32_t* __restrict__ req_err) {
   if (hdr->n_fit == 0) return;
-  const uint32_t n_req = hdr->n_req;
-  const uint32_t nw = gridDim.x * (blockDim.x >> 5);
-  const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  for (uint32_t r = 0; r < n_req; ++r) {
+  const uint32_t n_req = hdr->n_req, total = hdr->total_cand;
+  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < total;
+       g += gridDim.x * blockDim.x) {
+    const uint32_t r = find_request(reqs, n_req, g);
     const BatchReq& q = reqs[r];
-    if (!q.fitness || req_err[r] != 0u) continue;  // the same for the whole grid
-    for (uint32_t i = gw; i < q.n_cand; i += nw) {
-      const uint32_t o = q.cand_offsets[i];
-      const uint32_t L = q.cand_offsets[i + 1] - o;
-      if (q.n_arch == 0) {
-        if (lane == 0) q.fitness[i] = (uint64_t)q.counts[i] << ((L < 33u ? L : 33u) - 1u);
-        continue;
+    if (!q.fitness || req_err[r] != 0u) continue;
+    const uint32_t i = g - q.cand_base;
+    const uint32_t L = q.cand_offsets[i + 1] - q.cand_offsets[i];
+    const uint32_t shift = (L < 33u ? L : 33u) - 1u;
+    const uint32_t n = q.counts[i];
+    uint32_t best = 0;
+    if (q.n_arch) {
+      const uint64_t qc = (uint64_t)n << shift;
+      const uint64_t share = q.share[i];  // members sharing a column
+      const uint2* ov = reinterpret_cast<const uint2*>(q.overlaps + (size_t)i * q.ov_stride);
+      // a strictly worse member (q(a) < q(c)) does not penalise the candidate
+      auto penalty = [&](uint32_t m, uint32_t o) {
+        const uint32_t al = q.arch_offsets[m + 1] - q.arch_offsets[m];
+        const uint64_t qa = (uint64_t)q.arch_counts[m] << ((al < 33u ? al : 33u) - 1u);
+        if (((share >> m) & 1ull) && qa >= qc && o > best) best = o;
+      };
+#pragma unroll 4
+      for (uint32_t m = 0; m < q.n_arch; m += 2) {
+        const uint2 o = ov[m / 2];
+        penalty(m, o.x);
+        if (m + 1 < q.n_arch) penalty(m + 1, o.y);
       }
-      const uint64_t sh = q.share[i];
-      const uint32_t* ao = q.arch_offsets;
-      const uint32_t al0 = lane < (int)q.n_arch ? ao[lane + 1] - ao[lane] : 0u;
-      const uint32_t al1 = lane + 32 < (int)q.n_arch ? ao[lane + 33] - ao[lane + 32] : 0u;
-      prepdev::fused_fitness_mask(i, L, al0, al1, q.n_arch, sh, q.counts, q.overlaps,
-                                  q.ov_stride, q.arch_counts, q.fitness, lane);
     }
+    q.fitness[i] = (uint64_t)(n - best) << shift;
   }
 }
 
@@ -629,6 +671,7 @@ struct HostPlan {
   std::vector<BatchReq> reqs;
   std::vector<int32_t> ncols;
   uint32_t total_cand = 0;
+  uint32_t n_copy = 0;
   uint32_t stage_cap = 0;
   int32_t chunk_cap = 0;
   int device = -1;
@@ -743,6 +786,7 @@ int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_c
   hp->stage_cap = cap;
   hp->chunk_cap = (int32_t)cc_cap;
   uint32_t base = 0;
+  uint32_t copy_units = 0;
   for (uint32_t i = 0; i < n; ++i) {
     const ebic_eval_request& r = reqs[i];
     const EvalArgs& a = args[i];
@@ -784,11 +828,15 @@ int build_plan(const ebic_eval_request* reqs, uint32_t n, uint32_t fixed_stage_c
       q.arch_offsets = r.arch_offsets;
       q.arch_src = r.arch_bitmaps;
     }
+    q.copy_base = copy_units;
+    // (2^32 units would be 8 TB of padded archives)
+    if (q.fitness) copy_units += q.ov_stride * (q.pair_stride / kCopyWords);
     hp->ncols.push_back(v.L.cols);
     hp->reqs.push_back(q);
     base += r.n_cand;
   }
   hp->total_cand = base;
+  hp->n_copy = copy_units;
   place_fitness(hp, nullptr, nullptr, nullptr);
   return EBIC_OK;
 }
@@ -906,6 +954,7 @@ void fill_header(const HostPlan& hp, uint32_t n, BatchHeader* h) {
   std::memset(h, 0, sizeof(*h));
   h->n_req = n;
   h->total_cand = hp.total_cand;
+  h->n_copy = hp.n_copy;
   for (const BatchReq& q : hp.reqs) h->n_fit += q.fitness != nullptr;
 }
 

@@ -361,18 +361,5 @@ __device__ __forceinline__ uint64_t fused_fitness_value(uint32_t c, uint32_t L, 
   return (uint64_t)(n - best) << shift;
 }
 
-// The same, stored by lane 0.
-__device__ __forceinline__ void fused_fitness_mask(uint32_t c, uint32_t L, uint32_t al0,
-                                                   uint32_t al1, uint32_t n_arch, uint64_t sh,
-                                                   const uint32_t* counts,
-                                                   const uint32_t* overlaps, uint32_t ov_stride,
-                                                   const uint32_t* arch_counts, uint64_t* fitness,
-                                                   int lane) {
-  uint32_t n;
-  const uint64_t f = fused_fitness_value(c, L, al0, al1, n_arch, sh, counts, overlaps, ov_stride,
-                                         arch_counts, lane, n);
-  if (lane == 0) fitness[c] = f;
-}
-
 }  // namespace prepdev
 }  // namespace ebic
