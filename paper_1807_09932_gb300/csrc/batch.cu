@@ -586,9 +586,11 @@ __global__ void __launch_bounds__(pairdev::kPairThreads, 1)
     if (m.cand >= q.n_cand) continue;  // warp-uniform
     const uint32_t cand = m.cand;
     uint4 x[pairdev::kParts];
-    pairdev::pair_chain<NEG>(t, q.pairs + rword + 4 * lane,
-                             pair_ones(q.pairs, (uint64_t)q.pair_cols, q.pair_stride), lane,
-                             x);
+    const uint32_t ones = (uint32_t)((uint64_t)q.pair_cols * q.pair_cols * q.pair_stride);
+    if (!pairdev::pair_chain<NEG, pairdev::kParts>(t, q.pairs, (uint32_t)rword + 4 * lane, ones,
+                                                   lane, x) &&
+        !q.bitmaps)
+      continue;  // no row of the item follows: nothing to add
     uint32_t pc = 0;
 #pragma unroll
     for (int k = 0; k < pairdev::kParts; ++k) pc += pairdev::popc4(x[k]);
@@ -605,13 +607,13 @@ __global__ void __launch_bounds__(pairdev::kPairThreads, 1)
       pa.ov_stride = q.ov_stride;
       const int n_pairs = (int)(q.n_arch + 1) >> 1;
       if (q.bitmaps)  // warp-uniform
-        pairdev::item_epilogue<true, true>(pa, cand, rword, x, c, stage[warp], lane, q.n_arch,
+        pairdev::item_epilogue<true, true, pairdev::kParts>(pa, cand, rword, x, c, stage[warp], lane, q.n_arch,
                                            n_pairs, sh);
       else
-        pairdev::item_epilogue<false, true>(pa, cand, rword, x, c, stage[warp], lane, q.n_arch,
+        pairdev::item_epilogue<false, true, pairdev::kParts>(pa, cand, rword, x, c, stage[warp], lane, q.n_arch,
                                             n_pairs, sh);
     } else if (q.bitmaps) {  // warp-uniform
-      pairdev::item_epilogue<true, false>(pa, cand, rword, x, c, stage[warp], lane, 0u, 0, 0ull);
+      pairdev::item_epilogue<true, false, pairdev::kParts>(pa, cand, rword, x, c, stage[warp], lane, 0u, 0, 0ull);
     }
   }
 }

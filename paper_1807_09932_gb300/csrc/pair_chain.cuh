@@ -12,11 +12,13 @@ namespace pairdev {
 
 constexpr int kPairThreads = 768;
 constexpr int kPairWarps = kPairThreads / 32;
-constexpr int kParts = 4;        // 128-word parts per item (four words per lane each)
-constexpr int kStepTerms = 2;    // terms per chain step (one with negative trends)
+constexpr int kParts = 4;        // 128-word parts per item (four words per lane each): 4, 2 or 1
 constexpr int kRangeWords = 128;             // words per part (4,096 rows)
 constexpr int kItemWords = kParts * kRangeWords;
 static_assert(kPairRangeWords % kItemWords == 0, "table stride must hold whole items");
+// 16-byte loads a lane keeps in flight in a chain step: the step's terms (half of them reversed
+// with negative trends) times the item's parts
+constexpr int kStepLoads = 8;
 constexpr int kFewWords = 12;  // at most this many non-zero words: a lane per archive member
 
 __device__ __forceinline__ uint4 and4(uint4 a, uint4 b) {
@@ -80,73 +82,78 @@ __device__ __forceinline__ void terms_from_list(const uint16_t* __restrict__ col
   terms_from_cols<NEG>(c_lo, c_hi, L, C, S, lane, t);
 }
 
-// L2 prefetch of the item segments (kParts parts of kRangeWords words: 2 KB, sixteen 128-byte
-// lines) of two table rows, at word offsets off_a and off_b from `item` (the item's first table
-// word): lanes 0-15 take row a's lines, lanes 16-31 row b's, one line per lane, only in the parts
-// whose bit is set in part_mask. A prefetch holds no register: the pass issues one for the next
-// candidate's first step before the current candidate's epilogue. (Prefetching each chain
-// step's next rows as well measured slower, most for long candidates.)
-__device__ __forceinline__ void prefetch_rows2(const uint32_t* item, uint32_t off_a, bool has_a,
-                                               uint32_t off_b, bool has_b, uint32_t part_mask,
-                                               int lane) {
-  const int line = lane & 15;
-  const bool b = lane >= 16;
-  if ((b ? has_b : has_a) && ((part_mask >> (line >> 2)) & 1u)) {
-    const uint32_t* ptr = item + (b ? off_b : off_a) + line * 32;
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
+// L2 prefetch of the table rows' segments that the first chain step of a term list reads, in the
+// item that starts `word` words into the rows: 128 bytes per lane, kStepLoads / PARTS rows of
+// 4 PARTS lines. A prefetch holds no register: the pass issues one for the next candidate's first
+// step before the current candidate's epilogue. (Prefetching each chain step's next rows as well
+// measured slower, most for long candidates.)
+template <bool NEG, int PARTS>
+__device__ __forceinline__ void prefetch_first_step(const uint32_t* table, uint32_t word,
+                                                    const Terms& t, int lane) {
+  constexpr int kLines = 4 * PARTS, kStep = kStepLoads / PARTS / (NEG ? 2 : 1);
+  const int L = (int)__shfl_sync(0xFFFFFFFFu, t.hi, 31);
+  const int n_terms = L == 1 ? 1 : L - 1;
+  const int row = lane / kLines;
+  const bool rev = NEG && row >= kStep;
+  const int term = rev ? row - kStep : row;
+  uint32_t off = __shfl_sync(0xFFFFFFFFu, t.lo, term);
+  if (NEG) {
+    const uint32_t back = __shfl_sync(0xFFFFFFFFu, t.blo, term);
+    off = rev ? back : off;
   }
+  if (term < n_terms && !(rev && L == 1))
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(table + (off + word + (lane % kLines) * 32u)));
 }
 
-// The candidate's bitmap words 4*lane .. 4*lane+3 of each 128-word part of the item whose first
-// table word is `base` (table + item*kItemWords): AND of its consecutive pairs' table rows, OR
-// the reversed pairs' AND with negative trends. Each step keeps the rows of several terms of
+// The candidate's bitmap words 4*lane .. 4*lane+3 of each 128-word part of the item, whose words
+// of this lane start `word` words into the table rows: AND of its consecutive pairs' table rows,
+// OR the reversed pairs' AND with negative trends. Each step keeps the rows of several terms of
 // every part in flight. A lane whose own words of a part are all zero (they stay zero) reads the
-// table's all-ones chunk `ones` instead of its segment: every lane doing so reads the same 16
-// bytes, so the step's requests shrink to the lanes that still match rows, with no branch. The
-// walk stops when no lane has a non-zero word left (long chains match no row of most ranges).
-template <bool NEG>
-__device__ __forceinline__ void pair_chain(const Terms& t, const uint32_t* base,
-                                           const uint32_t* ones, int lane,
-                                           uint4 (&out)[kParts]) {
-  constexpr int kStep = NEG ? kStepTerms / 2 : kStepTerms;
+// table's all-ones chunk (`ones` words into the table) instead of its segment: every lane doing so
+// reads the same 16 bytes, so the step's requests shrink to the lanes that still match rows, with
+// no branch. Places in the table are 32-bit word offsets up to the load (a select and one
+// multiply-add per load; 64-bit pointers took two selects and an add more). The walk stops when no
+// lane has a non-zero word left (long chains match no row of most ranges); false then.
+template <bool NEG, int PARTS>
+__device__ __forceinline__ bool pair_chain(const Terms& t, const uint32_t* table, uint32_t word,
+                                           uint32_t ones, int lane, uint4 (&out)[PARTS]) {
+  constexpr int kStep = kStepLoads / PARTS / (NEG ? 2 : 1);
   const int L = (int)__shfl_sync(0xFFFFFFFFu, t.hi, 31);
   const int n_terms = L == 1 ? 1 : L - 1;
   const bool two = NEG && L > 1;  // warp-uniform
   const uint4 all = make_uint4(~0u, ~0u, ~0u, ~0u);
-  uint4 x[kParts], y[kParts];
-  bool nzx[kParts], nzy[kParts];  // this lane's words of the part are not all zero
+  uint4 x[PARTS], y[PARTS];
+  bool nzx[PARTS], nzy[PARTS];  // this lane's words of the part are not all zero
 #pragma unroll
-  for (int q = 0; q < kParts; ++q) {
+  for (int q = 0; q < PARTS; ++q) {
     x[q] = y[q] = all;
     nzx[q] = nzy[q] = true;
   }
+  // part q of the row at `off`, or the all-ones chunk
+  auto load = [&](uint32_t off, bool live, int q) {
+    const uint32_t at = live ? off : ones - q * kRangeWords;
+    return __ldg(reinterpret_cast<const uint4*>(table + at) + q * (kRangeWords / 4));
+  };
   // terms [t0, t1) with t0 in {0, 32}: lane (i - t0) holds term i's offsets
   auto walk = [&](uint32_t offf, uint32_t offb, int t0, int t1) -> bool {
     for (int i0 = t0; i0 < t1; i0 += kStep) {
-      // the next step's rows, prefetched while this step's are loaded (the parts still alive
-      // after the previous step: at most one step's rows are fetched in vain)
-      uint4 v[kStep][kParts], u[kStep][kParts];
+      uint4 v[kStep][PARTS], u[kStep][PARTS];
 #pragma unroll
       for (int k = 0; k < kStep; ++k) {
         const int i = i0 + k;
         const bool has = i < t1;  // warp-uniform
-        const uint32_t* rf = base + __shfl_sync(0xFFFFFFFFu, offf, i & 31);
+        const uint32_t rf = word + __shfl_sync(0xFFFFFFFFu, offf, i & 31);
 #pragma unroll
-        for (int q = 0; q < kParts; ++q)
-          v[k][q] = __ldg(reinterpret_cast<const uint4*>(has && nzx[q] ? rf + q * kRangeWords
-                                                                       : ones));
+        for (int q = 0; q < PARTS; ++q) v[k][q] = load(rf, has && nzx[q], q);
         if (NEG) {
-          const uint32_t* rb = base + __shfl_sync(0xFFFFFFFFu, offb, i & 31);
+          const uint32_t rb = word + __shfl_sync(0xFFFFFFFFu, offb, i & 31);
 #pragma unroll
-          for (int q = 0; q < kParts; ++q)
-            u[k][q] = __ldg(reinterpret_cast<const uint4*>(two && has && nzy[q]
-                                                               ? rb + q * kRangeWords
-                                                               : ones));
+          for (int q = 0; q < PARTS; ++q) u[k][q] = load(rb, two && has && nzy[q], q);
         }
       }
       bool lane_any = false;
 #pragma unroll
-      for (int q = 0; q < kParts; ++q) {
+      for (int q = 0; q < PARTS; ++q) {
 #pragma unroll
         for (int k = 0; k < kStep; ++k) x[q] = and4(x[q], v[k][q]);
         nzx[q] = (x[q].x | x[q].y | x[q].z | x[q].w) != 0u;
@@ -162,12 +169,13 @@ __device__ __forceinline__ void pair_chain(const Terms& t, const uint32_t* base,
     }
     return true;
   };
-  if (walk(t.lo, t.blo, 0, n_terms < 32 ? n_terms : 32) && n_terms > 32)
-    walk(t.hi, t.bhi, 32, n_terms);
+  bool any = walk(t.lo, t.blo, 0, n_terms < 32 ? n_terms : 32);
+  if (any && n_terms > 32) any = walk(t.hi, t.bhi, 32, n_terms);
 #pragma unroll
-  for (int q = 0; q < kParts; ++q)
+  for (int q = 0; q < PARTS; ++q)
     out[q] = two ? make_uint4(x[q].x | y[q].x, x[q].y | y[q].y, x[q].z | y[q].z, x[q].w | y[q].w)
                  : x[q];
+  return any;
 }
 
 // An archive row segment: re-read by every warp of the CTA that scores a candidate of the same
@@ -199,15 +207,15 @@ __device__ __forceinline__ void add_pair(unsigned long long* ov2, int k, uint32_
 // x (lane holds words 4*lane .. 4*lane+3 of part q, i.e. item words 128q + 4*lane + j, in x[q])
 // and their warp total cnt.
 // `members`: the archive members whose overlaps are wanted (a bit per member below n_arch).
-template <bool BITMAPS, bool OVERLAP>
+template <bool BITMAPS, bool OVERLAP, int PARTS>
 __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, uint64_t rword,
-                                              const uint4 (&x)[kParts], uint32_t cnt, uint32_t* st,
+                                              const uint4 (&x)[PARTS], uint32_t cnt, uint32_t* st,
                                               int lane, uint32_t n_arch, int n_pairs,
                                               uint64_t members) {
   if constexpr (BITMAPS) {  // through shared memory, so each store instruction is coalesced
     uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.W;
 #pragma unroll
-    for (int h = 0; h < kParts; ++h) {
+    for (int h = 0; h < PARTS; ++h) {
       *reinterpret_cast<uint4*>(st + 4 * lane) = x[h];
       __syncwarp();
 #pragma unroll
@@ -224,18 +232,18 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
     const uint32_t* abase = p.arch + rword;
     uint32_t* ov = p.overlaps + (uint64_t)cand * p.ov_stride;
     // the lane's eight words and where they sit in the item
-    uint32_t xw[4 * kParts];
+    uint32_t xw[4 * PARTS];
 #pragma unroll
-    for (int q = 0; q < kParts; ++q) {
+    for (int q = 0; q < PARTS; ++q) {
       xw[4 * q] = x[q].x;
       xw[4 * q + 1] = x[q].y;
       xw[4 * q + 2] = x[q].z;
       xw[4 * q + 3] = x[q].w;
     }
-    uint32_t bal[4 * kParts];
+    uint32_t bal[4 * PARTS];
     int nz = 0;
 #pragma unroll
-    for (int j = 0; j < 4 * kParts; ++j) {
+    for (int j = 0; j < 4 * PARTS; ++j) {
       bal[j] = __ballot_sync(0xFFFFFFFFu, xw[j] != 0u);
       nz += __popc(bal[j]);
     }
@@ -246,7 +254,7 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
       const uint32_t lt = (1u << lane) - 1u;
       int base = 0;
 #pragma unroll
-      for (int j = 0; j < 4 * kParts; ++j) {
+      for (int j = 0; j < 4 * PARTS; ++j) {
         if (xw[j]) {
           const int q = base + __popc(bal[j] & lt);
           sv[q] = xw[j];
@@ -291,7 +299,7 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
       }
     } else {
       // dense: the wanted members two at a time (no unwanted partner), one packed reduction
-      // (each sum <= 128 * 4 * kParts * 32 / 4 < 2^16), lanes 0 and 1 add the two totals
+      // (each sum <= 128 * 4 * PARTS * 32 / 4 < 2^16), lanes 0 and 1 add the two totals
       const uint32_t* ab = abase + 4 * lane;
       uint64_t mm = members;
       while (mm) {  // warp-uniform
@@ -304,7 +312,7 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
         const uint32_t* pb = ab + (uint64_t)mb * astride;
         uint32_t sa = 0, sb = 0;
 #pragma unroll
-        for (int q = 0; q < kParts; ++q) {
+        for (int q = 0; q < PARTS; ++q) {
           sa += popc4(and4(x[q], ld_arch4(pa + q * kRangeWords)));
           sb += popc4(and4(x[q], ld_arch4(pb + q * kRangeWords)));
         }
@@ -327,18 +335,19 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
 // share meet in its L1.
 // `valid()` (warp-uniform) is asked after the warp's first term list is requested and before any
 // table row is read; false ends the pass.
-template <bool NEG, bool BITMAPS, bool OVERLAP, class Valid>
+template <bool NEG, bool BITMAPS, bool OVERLAP, int PARTS, class Valid>
 __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint32_t* next_unit,
                                            Valid valid) {
   const int lane = threadIdx.x & 31;
-  const uint32_t n_ranges = (uint32_t)((p.W + kItemWords - 1) / kItemWords);
+  constexpr uint32_t kWords = PARTS * kRangeWords;  // words per item
+  const uint32_t n_ranges = (uint32_t)((p.W + kWords - 1) / kWords);
   const uint32_t n_groups = (p.n_cand + kPairWarps - 1) / kPairWarps;
   const uint64_t n_items = (uint64_t)n_ranges * n_groups;
   const bool narrow = n_items <= 0xFFFFFFFFull;  // 32-bit item arithmetic suffices
   const uint32_t n_arch = OVERLAP ? p.n_arch : 0u;
   const int n_pairs = (int)(n_arch + 1) >> 1;
   const uint64_t all_members = n_arch >= 64 ? ~0ull : ((1ull << n_arch) - 1ull);
-  const uint32_t* ones = pair_ones(p.table, (uint64_t)p.C, p.stride);
+  const uint32_t ones = (uint32_t)((uint64_t)p.C * p.C * p.stride);  // below 2^32 (launch_pair_eval)
   struct Unit {
     uint64_t it;
     uint32_t range, grp, slot, cand;
@@ -369,7 +378,7 @@ __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint
   if (cur.it < n_items && cur.cand < p.n_cand) load_terms<NEG>(p, cur.cand, lane, next);
   if (!valid()) return;
   while (cur.it < n_items) {
-    const uint64_t rword = (uint64_t)cur.range * kItemWords;  // first word of the item
+    const uint32_t rword = cur.range * kWords;  // first word of the item
     const uint32_t cand = cur.cand;
     const Terms t = next;
     const bool arch_share = OVERLAP && cur.grp == 0;  // this range's archive counts, slot's share
@@ -382,30 +391,26 @@ __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint
         const uint32_t* ar = p.arch + (uint64_t)a * p.stride + rword + 4 * lane;
         uint32_t pa = 0;
 #pragma unroll
-        for (int q = 0; q < kParts; ++q) pa += popc4(ld_arch4(ar + q * kRangeWords));
+        for (int q = 0; q < PARTS; ++q) pa += popc4(ld_arch4(ar + q * kRangeWords));
         const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, pa);
         if (lane == 0 && n) atomicAdd(&p.arch_counts[a], n);
       }
     }
     if (cand >= p.n_cand) continue;  // warp-uniform
-    uint4 x[kParts];
-    pair_chain<NEG>(t, p.table + rword + 4 * lane, ones, lane, x);
+    uint4 x[PARTS];
+    const bool any = pair_chain<NEG, PARTS>(t, p.table, rword + 4 * lane, ones, lane, x);
     // the next unit's first step, prefetched while this unit's epilogue runs (its term list has
     // arrived during the walk)
-    if (!NEG && cur.it < n_items && cur.cand < p.n_cand) {
-      const int Ln = (int)__shfl_sync(0xFFFFFFFFu, next.hi, 31);
-      const uint32_t a0 = __shfl_sync(0xFFFFFFFFu, next.lo, 0);
-      const uint32_t a1 = __shfl_sync(0xFFFFFFFFu, next.lo, 1);
-      prefetch_rows2(p.table + (uint64_t)cur.range * kItemWords, a0, true, a1, Ln > 2,
-                     (1u << kParts) - 1u, lane);
-    }
+    if (cur.it < n_items && cur.cand < p.n_cand)
+      prefetch_first_step<NEG, PARTS>(p.table, cur.range * kWords, next, lane);
+    if (!BITMAPS && !any) continue;  // no row of the item follows: nothing to add
     uint32_t pc = 0;
 #pragma unroll
-    for (int q = 0; q < kParts; ++q) pc += popc4(x[q]);
+    for (int q = 0; q < PARTS; ++q) pc += popc4(x[q]);
     const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, pc);
     if (lane == 0 && c) atomicAdd(&p.counts[cand], c);
     const uint64_t members = OVERLAP && p.score ? p.score[cand] & all_members : all_members;
-    item_epilogue<BITMAPS, OVERLAP>(p, cand, rword, x, c, st, lane, n_arch, n_pairs, members);
+    item_epilogue<BITMAPS, OVERLAP, PARTS>(p, cand, rword, x, c, st, lane, n_arch, n_pairs, members);
   }
 }
 

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) pair_eval_kernel(const PairAr
     f = *reinterpret_cast<const volatile uint32_t*>(p.err);
   }
   __syncthreads();  // next_unit is set
-  pair_items<NEG, BITMAPS, OVERLAP>(p, stage[warp], &next_unit, [&]() {
+  pair_items<NEG, BITMAPS, OVERLAP, kParts>(p, stage[warp], &next_unit, [&]() {
     f = __reduce_or_sync(0xFFFFFFFFu, f);
     if (p.flags && blockIdx.x == 0 && threadIdx.x == 0) *p.err_out = f;  // CTA 0 records it
     return f == 0u;  // else invalid input: nothing is evaluated
