@@ -91,7 +91,10 @@ typedef struct ebic_matrix ebic_matrix;
 int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uint32_t flags,
                      float fill_value, void* stream, ebic_matrix** out);
 
-/* Free a matrix handle and its device memory. Synchronizes the device. NULL is a no-op. */
+/* Free a matrix handle and its device memory. Synchronizes the device. NULL is a no-op. Up to
+ * 2 GiB of freed device memory per device stays with the library's pool for the next matrix or
+ * search (mapping it again costs more than opening most data sets); what is above goes back to
+ * the system, and all of it when an allocation of the library finds no memory. */
 int ebic_free_matrix(ebic_matrix* m);
 
 /*

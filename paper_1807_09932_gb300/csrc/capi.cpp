@@ -561,17 +561,21 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
   m->fill = fill_value;
   m->total_rows = rows;
   auto cleanup = [&](int code) {
-    if (m->ranks) cudaFree(m->ranks);
-    if (m->status) cudaFree(m->status);
+    (void)device_free(m->ranks, s);
     delete m;
     return code;
   };
   cudaError_t e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
-  e = cudaMalloc(&m->ranks, m->L.rank_words() * 4);
-  if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc(rank matrix)"));
-  e = cudaMalloc(&m->status, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemsetAsync(m->status, 0, sizeof(uint32_t), s);
+  // the rank matrix, and the status word after it
+  const size_t rank_bytes = (m->L.rank_words() * 4 + 255) / 256 * 256;
+  e = device_alloc(reinterpret_cast<void**>(&m->ranks), rank_bytes + 256, dev, s);
+  if (e != cudaSuccess) {
+    m->ranks = nullptr;
+    return cleanup(cuda_fail(e, "allocation of the rank matrix"));
+  }
+  m->status = m->ranks + rank_bytes / 4;
+  e = cudaMemsetAsync(m->status, 0, sizeof(uint32_t), s);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "status word"));
 
   {
@@ -596,12 +600,13 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
     }
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "rank transform launch"));
   }
-  e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cleanup(cuda_fail(e, "rank transform"));
   {  // a bounded wait of the transform that expired leaves the matrix unusable
-    uint32_t bits = 0;
-    e = cudaMemcpy(&bits, m->status, sizeof(uint32_t), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "rank transform status"));
+    uint32_t pageable = 0;
+    uint32_t* const bits_at = t_err_word.get() ? t_err_word.host : &pageable;
+    e = cudaMemcpyAsync(bits_at, m->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cleanup(cuda_fail(e, "rank transform"));
+    const uint32_t bits = *static_cast<volatile uint32_t*>(bits_at);
     if (bits & kErrTimeout)
       return cleanup(fail(EBIC_ERR_DEVICE_TIMEOUT, "rank transform: a bounded device wait expired"));
   }
@@ -612,12 +617,12 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
 int ebic_free_matrix(ebic_matrix* m) {
   if (!m) return EBIC_OK;
   DeviceGuard g(m->device);
-  if (m->pairs) cudaFree(m->pairs);
-  cudaError_t e1 = cudaFree(m->ranks);
-  cudaError_t e2 = cudaFree(m->status);
+  // no stream uses the matrix once the device is synchronized
+  cudaError_t e = cudaDeviceSynchronize();
+  const cudaError_t e1 = device_free(m->pairs, nullptr), e2 = device_free(m->ranks, nullptr);
+  if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
   delete m;
-  if (e1 != cudaSuccess) return cuda_fail(e1, "cudaFree(rank matrix)");
-  if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFree(status)");
+  if (e != cudaSuccess) return cuda_fail(e, "freeing a matrix");
   return EBIC_OK;
 }
 
@@ -1129,7 +1134,7 @@ int ebic_matrix_build_pairs(ebic_matrix* m, uint64_t max_bytes, void* stream, ui
   if (m->pairs) return EBIC_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* table = nullptr;
-  cudaError_t e = cudaMalloc(&table, need);
+  cudaError_t e = device_alloc(reinterpret_cast<void**>(&table), need, m->device, s);
   if (e != cudaSuccess) return cuda_fail(e, "pair table allocation");
   {
     Timed t(EBIC_TIMING_EVALUATE, s);
@@ -1137,7 +1142,7 @@ int ebic_matrix_build_pairs(ebic_matrix* m, uint64_t max_bytes, void* stream, ui
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
-    cudaFree(table);
+    (void)device_free(table, s);
     return cuda_fail(e, "pair table build");
   }
   m->pairs = table;
@@ -1150,7 +1155,8 @@ int ebic_matrix_drop_pairs(ebic_matrix* m) {
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
   if (m->pairs) {
     DeviceGuard g(m->device);
-    EBIC_CUDA(cudaFree(m->pairs));
+    EBIC_CUDA(cudaDeviceSynchronize());  // no stream reads the table any more
+    EBIC_CUDA(device_free(m->pairs, nullptr));
     m->pairs = nullptr;
     m->pair_stride = 0;
     m->pair_bytes = 0;

@@ -55,7 +55,13 @@ struct Layout {
 void count_launch();
 void count_launches(int64_t n);  // n kernels at once (a negative n takes back counted ones)
 
-// Choose width and VEC for a column count (host).
+// Device memory that lives as long as a matrix, a pair table or a search, from the device's pool
+// (devmem.cpp), stream-ordered on s: other streams may use it once s has reached the allocation.
+// Freed memory must no longer be in use by any stream but s.
+cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s);
+cudaError_t device_free(void* p, cudaStream_t s);
+
+// The layout for a matrix shape (host).
 Layout make_layout(int64_t rows, int32_t cols);
 
 // ---- rank transform ------------------------------------------------------------------------

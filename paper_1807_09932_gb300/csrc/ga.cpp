@@ -802,6 +802,8 @@ struct GpuEvaluator : Evaluator {
   // the offers' lists, staged in pinned memory and sent in one copy to a device block of the
   // same layout: gather indices [T], columns [T * max_len], offsets [T + 1], counts [T]
   char *hstage = nullptr, *dstage = nullptr;
+  char* pinned = nullptr;  // hstage, hpov, hcnt, hfit and hov
+  int device = 0;
   size_t st_cols = 0, st_offs = 0, st_cnt = 0, st_bytes = 0;
   uint32_t* hpov = nullptr;  // pinned [T][T]: the pair overlaps' copy-back
   uint32_t pending_t = 0;
@@ -820,22 +822,19 @@ struct GpuEvaluator : Evaluator {
         T(2 * p.archive_size), max_len(p.max_len), W(words) {}
   ~GpuEvaluator() override {
     cudaStreamSynchronize(s);
-    for (void* a : allocs) cudaFree(a);
-    if (hpov) cudaFreeHost(hpov);
-    if (hstage) cudaFreeHost(hstage);
-    if (hcnt) cudaFreeHost(hcnt);
-    if (hfit) cudaFreeHost(hfit);
-    if (hov) cudaFreeHost(hov);
+    for (void* a : allocs) (void)device_free(a, s);
+    if (pinned) cudaFreeHost(pinned);
   }
   template <class X>
   cudaError_t alloc(X** p, size_t n) {
     void* v = nullptr;
-    cudaError_t e = cudaMalloc(&v, (n ? n : 1) * sizeof(X));
+    cudaError_t e = device_alloc(&v, (n ? n : 1) * sizeof(X), device, s);
     if (e == cudaSuccess) allocs.push_back(v);
     *p = static_cast<X*>(v);
     return e;
   }
   int init() {
+    GA_CUDA(cudaGetDevice(&device));
     GA_CUDA(alloc(&dcols, (size_t)P * max_len));
     GA_CUDA(alloc(&doffs, (size_t)P + 1));
     GA_CUDA(alloc(&dcounts, P));
@@ -852,7 +851,6 @@ struct GpuEvaluator : Evaluator {
     st_cnt = st_offs + up16(((size_t)T + 1) * 4);
     st_bytes = st_cnt + up16((size_t)T * 4);
     GA_CUDA(alloc(&dstage, st_bytes));
-    GA_CUDA(cudaMallocHost(&hstage, st_bytes));
     pcols = reinterpret_cast<uint16_t*>(dstage + st_cols);
     poffs = reinterpret_cast<uint32_t*>(dstage + st_offs);
     pcounts = reinterpret_cast<uint32_t*>(dstage + st_cnt);
@@ -860,10 +858,15 @@ struct GpuEvaluator : Evaluator {
     GA_CUDA(alloc(&pfit, T));
     GA_CUDA(alloc(&pov, (size_t)T * T));
     GA_CUDA(alloc(&didx, (size_t)std::max(T, K)));
-    GA_CUDA(cudaMallocHost(&hpov, (size_t)std::max(T, 1u) * std::max(T, 1u) * 4));
-    GA_CUDA(cudaMallocHost(&hcnt, (size_t)P * 4));
-    GA_CUDA(cudaMallocHost(&hfit, (size_t)P * 8));
-    GA_CUDA(cudaMallocHost(&hov, (size_t)P * std::max(K, 1u) * 4));
+    // the pinned blocks, in one allocation
+    const size_t pov_bytes = up16((size_t)T * T * 4), cnt_bytes = up16((size_t)P * 4),
+                 fit_bytes = up16((size_t)P * 8), ov_bytes = up16((size_t)P * K * 4);
+    GA_CUDA(cudaMallocHost(&pinned, st_bytes + pov_bytes + cnt_bytes + fit_bytes + ov_bytes + 16));
+    hstage = pinned;
+    hpov = reinterpret_cast<uint32_t*>(pinned + st_bytes);
+    hcnt = reinterpret_cast<uint32_t*>(pinned + st_bytes + pov_bytes);
+    hfit = reinterpret_cast<uint64_t*>(pinned + st_bytes + pov_bytes + cnt_bytes);
+    hov = reinterpret_cast<uint32_t*>(pinned + st_bytes + pov_bytes + cnt_bytes + fit_bytes);
     return EBIC_OK;
   }
   int evaluate(const std::vector<uint16_t>& cols, const std::vector<uint32_t>& offs, uint32_t n,

@@ -1140,15 +1140,18 @@ namespace {
     }                                                                                      \
   } while (0)
 
+// The loop's device buffers, allocated on its stream; freed once its streams are drained.
 struct DeviceBuffers {
   std::vector<void*> all;
+  int device = 0;
+  cudaStream_t s = nullptr;
   ~DeviceBuffers() {
-    for (void* p : all) cudaFree(p);
+    for (void* p : all) (void)device_free(p, nullptr);
   }
   template <class X>
   cudaError_t get(X** p, size_t n) {
     void* v = nullptr;
-    cudaError_t e = cudaMalloc(&v, (n ? n : 1) * sizeof(X));
+    cudaError_t e = device_alloc(&v, (n ? n : 1) * sizeof(X), device, s);
     if (e == cudaSuccess) all.push_back(v);
     *p = static_cast<X*>(v);
     return e;
@@ -1164,6 +1167,41 @@ uint64_t pow2_at_least(uint64_t x) {
 }  // namespace
 
 namespace {
+// An archive's lists in one block, on the device and (the same layout) on the host, so that each
+// archive goes up, and the result comes back, in one copy.
+struct ArchiveImage {
+  uint32_t K;
+  size_t c, n, count, offs, size, cols, bytes;
+  explicit ArchiveImage(uint32_t k) : K(k) {
+    auto up16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    c = up16((size_t)K * 8);  // (the qualities come first)
+    n = c + up16((size_t)K * kMaxLen * 2);
+    count = n + up16((size_t)K * 4);
+    offs = count + up16((size_t)K * 4);
+    size = offs + up16(((size_t)K + 1) * 4);
+    cols = size + 16;
+    bytes = cols + up16((size_t)K * kMaxLen * 2);
+  }
+  gadev::Archive at(uint8_t* base) const {
+    gadev::Archive a;
+    a.q = reinterpret_cast<uint64_t*>(base);
+    a.c = reinterpret_cast<uint16_t*>(base + c);
+    a.n = reinterpret_cast<uint32_t*>(base + n);
+    a.count = reinterpret_cast<uint32_t*>(base + count);
+    a.csr_offs = reinterpret_cast<uint32_t*>(base + offs);
+    a.size = reinterpret_cast<uint32_t*>(base + size);
+    a.csr_cols = reinterpret_cast<uint16_t*>(base + cols);
+    return a;
+  }
+};
+
+struct GraphExec {
+  cudaGraphExec_t exec = nullptr;
+  ~GraphExec() {
+    if (exec) (void)cudaGraphExecDestroy(exec);
+  }
+};
+
 // The loop's own stream (it can be captured into a graph, which the legacy default stream cannot),
 // started after the caller's stream's pending work; released when the run returns.
 struct RunStream {
@@ -1190,6 +1228,8 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   RunStream rs;
   GD_CUDA(cudaStreamCreateWithFlags(&rs.s, cudaStreamNonBlocking));
   GD_CUDA(cudaStreamCreateWithFlags(&rs.s2, cudaStreamNonBlocking));
+  GD_CUDA(cudaGetDevice(&b.device));
+  b.s = rs.s;
   for (cudaEvent_t* x : {&rs.e, &rs.fork0, &rs.tabu_done, &rs.fork1, &rs.archive_done})
     GD_CUDA(cudaEventCreateWithFlags(x, cudaEventDisableTiming));
   GD_CUDA(cudaEventRecord(rs.e, caller));
@@ -1204,11 +1244,7 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   if (cap_e >= 0xFFFFFFFFull)
     return set_last_error(EBIC_ERR_UNSUPPORTED, "population x generations too large for the device loop");
   int num_sms = 0;
-  {
-    int dev = 0;
-    GD_CUDA(cudaGetDevice(&dev));
-    GD_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
-  }
+  GD_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, b.device));
   Pop pop, nxt;
   GD_CUDA(b.get(&pop.c, (size_t)P * kMaxLen));
   GD_CUDA(b.get(&pop.n, P));
@@ -1257,16 +1293,14 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   GD_CUDA(b.get(&tabu.ent_n, cap_e));
   GD_CUDA(b.get(&tabu.arena, cap_e * kMaxLen));
   GD_CUDA(b.get(&tabu.n_ent, 1));
+  // the archives: an image of each one's lists (see ArchiveImage) and its bitmap rows
   Archive arch[2];
   uint32_t* abm[2];
+  uint8_t* images[2];
+  const ArchiveImage img(K);
   for (int k = 0; k < 2; ++k) {
-    GD_CUDA(b.get(&arch[k].c, (size_t)K * kMaxLen));
-    GD_CUDA(b.get(&arch[k].n, K));
-    GD_CUDA(b.get(&arch[k].count, K));
-    GD_CUDA(b.get(&arch[k].q, K));
-    GD_CUDA(b.get(&arch[k].size, 1));
-    GD_CUDA(b.get(&arch[k].csr_cols, (size_t)K * kMaxLen));
-    GD_CUDA(b.get(&arch[k].csr_offs, (size_t)K + 1));
+    GD_CUDA(b.get(&images[k], img.bytes));
+    arch[k] = img.at(images[k]);
     GD_CUDA(b.get(&abm[k], (size_t)(K + 1) * W));  // row K stays zero: the empty members' row
     GD_CUDA(cudaMemsetAsync(abm[k], 0, (size_t)(K + 1) * W * 4, s));
   }
@@ -1277,23 +1311,12 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   GD_CUDA(cudaMemcpyAsync(pop.c, init_cols, (size_t)P * kMaxLen * 2, cudaMemcpyHostToDevice, s));
   GD_CUDA(cudaMemcpyAsync(pop.n, init_n, (size_t)P * 4, cudaMemcpyHostToDevice, s));
   GD_CUDA(cudaMemcpyAsync(pop.h, init_h, (size_t)P * 8, cudaMemcpyHostToDevice, s));
-  {
-    std::vector<uint16_t> c((size_t)K * kMaxLen, 0);
-    std::vector<uint32_t> n(K, 1u), zeros(K, 0u), offs(K + 1);
-    std::vector<uint64_t> q(K, 0ull);
-    for (uint32_t r = 0; r <= K; ++r) offs[r] = r;
-    const uint32_t size0 = 0;
-    for (int k = 0; k < 2; ++k) {
-      // synchronous copies: the host vectors go out of scope
-      GD_CUDA(cudaMemcpy(arch[k].c, c.data(), c.size() * 2, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].n, n.data(), K * 4, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].count, zeros.data(), K * 4, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].q, q.data(), K * 8, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].size, &size0, 4, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].csr_cols, c.data(), (size_t)K * 2, cudaMemcpyHostToDevice));
-      GD_CUDA(cudaMemcpy(arch[k].csr_offs, offs.data(), (K + 1) * 4, cudaMemcpyHostToDevice));
-    }
-  }
+  std::vector<uint64_t> host_image(img.bytes / 8, 0);
+  const Archive host = img.at(reinterpret_cast<uint8_t*>(host_image.data()));
+  std::fill(host.n, host.n + K, 1u);
+  for (uint32_t r = 0; r <= K; ++r) host.csr_offs[r] = r;
+  for (int k = 0; k < 2; ++k)  // (a pageable source has been read when the call returns)
+    GD_CUDA(cudaMemcpyAsync(images[k], host_image.data(), img.bytes, cudaMemcpyHostToDevice, s));
   Ops o;
   o.P = P;
   o.min_len = p.min_len;
@@ -1375,12 +1398,18 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   };
   pack_kernel<<<1, 1024, 0, s>>>(pops[0], P, dcols, doffs);
   GD_CUDA(cudaGetLastError());
-  // the breeding generations 0 .. G-2 (two at a time from a captured graph when the stream can be
-  // captured), then the last one without breeding
+  // the breeding generations 0 .. G-2, then the last one without breeding. Two at a time from a
+  // captured graph where there are enough: the first two are launched directly, and run while the
+  // graph is captured and instantiated. The graph is destroyed after the run (destroying it waits
+  // for its launches).
   uint32_t gen = 0;
-  cudaGraphExec_t exec = nullptr;
+  GraphExec graph_exec;
   int64_t graph_launches = 0;  // kernels in the two-generation graph
   if (G >= 5) {
+    for (; gen < 2; ++gen) {
+      const int rc = issue((int)gen, true);
+      if (rc != EBIC_OK) return rc;
+    }
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
       const int64_t c0 = ebic_launch_count();
@@ -1390,23 +1419,17 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
       count_launches(-graph_launches);  // nothing ran while capturing
       const cudaError_t ec = cudaStreamEndCapture(s, &graph);
       if (rc1 == EBIC_OK && ec == cudaSuccess && graph &&
-          cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
-        exec = nullptr;
+          cudaGraphInstantiate(&graph_exec.exec, graph, 0) != cudaSuccess)
+        graph_exec.exec = nullptr;
       if (graph) cudaGraphDestroy(graph);
     }
     (void)cudaGetLastError();  // a failed capture leaves the direct launches below
   }
-  if (exec) {
+  if (graph_exec.exec)
     for (; gen + 2 <= G - 1; gen += 2) {
-      cudaError_t e = cudaGraphLaunch(exec, s);
-      if (e != cudaSuccess) {
-        cudaGraphExecDestroy(exec);
-        GD_CUDA(e);
-      }
+      GD_CUDA(cudaGraphLaunch(graph_exec.exec, s));
       count_launches(graph_launches);
     }
-    cudaGraphExecDestroy(exec);
-  }
   for (; gen + 1 < G; ++gen) {
     const int rc = issue((int)(gen & 1u), true);
     if (rc != EBIC_OK) return rc;
@@ -1418,19 +1441,14 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   }
   const int cur = (int)(gen & 1u);  // the archive the last generation wrote
   const uint64_t evaluated = (uint64_t)P * gen;
-  GD_CUDA(cudaStreamSynchronize(s));
-  int st = ebic_matrix_status(const_cast<ebic_matrix*>(m), s);
-  if (st != EBIC_OK) return st;
   // the archive, best first
-  uint32_t n = 0;
-  GD_CUDA(cudaMemcpy(&n, arch[cur].size, 4, cudaMemcpyDeviceToHost));
-  std::vector<uint16_t> c((size_t)K * kMaxLen);
-  std::vector<uint32_t> len(K), cnt(K);
-  std::vector<uint64_t> q(K);
-  GD_CUDA(cudaMemcpy(c.data(), arch[cur].c, c.size() * 2, cudaMemcpyDeviceToHost));
-  GD_CUDA(cudaMemcpy(len.data(), arch[cur].n, K * 4, cudaMemcpyDeviceToHost));
-  GD_CUDA(cudaMemcpy(cnt.data(), arch[cur].count, K * 4, cudaMemcpyDeviceToHost));
-  GD_CUDA(cudaMemcpy(q.data(), arch[cur].q, K * 8, cudaMemcpyDeviceToHost));
+  GD_CUDA(cudaMemcpyAsync(host_image.data(), images[cur], img.bytes, cudaMemcpyDeviceToHost, s));
+  int st = ebic_matrix_status(const_cast<ebic_matrix*>(m), s);  // (synchronizes s)
+  if (st != EBIC_OK) return st;
+  const uint32_t n = *host.size;
+  const uint16_t* c = host.c;
+  const uint32_t *len = host.n, *cnt = host.count;
+  const uint64_t* q = host.q;
   ebic_result* r = new ebic_result();
   std::memset(r, 0, sizeof(*r));
   r->n = n;
@@ -1447,8 +1465,7 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
   r->offsets[0] = 0;
   size_t pos = 0;
   for (uint32_t i = 0; i < n; ++i) {
-    std::copy(c.begin() + (size_t)i * kMaxLen, c.begin() + (size_t)i * kMaxLen + len[i],
-              r->cols + pos);
+    std::copy(c + (size_t)i * kMaxLen, c + (size_t)i * kMaxLen + len[i], r->cols + pos);
     pos += len[i];
     r->offsets[i + 1] = (uint32_t)pos;
     r->counts[i] = cnt[i];
