@@ -996,31 +996,42 @@ static int eval_fitness_impl(const ebic_matrix* cm, const uint16_t* cols, const 
     pa.table = m->pairs;
     EBIC_CUDA(launch_fused_prepare(pa, prep_blocks, s));
   }
-  {
+  PairArgs p;
+  p.table = m->pairs;
+  p.stride = stride;
+  p.C = L.cols;
+  p.W = L.words;
+  p.terms = dterms;
+  p.n_cand = n_cand;
+  p.counts = dcounts;
+  p.bitmaps = dbm;
+  p.arch = n_arch > 0 ? dpad : nullptr;
+  p.n_arch = n_arch;
+  // all members only when the caller reads all their overlaps
+  p.score = overlaps && !sharing_only ? nullptr : dshare;
+  p.overlaps = dov;
+  p.ov_stride = ov_stride;
+  p.arch_counts = darch_counts;
+  p.flags = dflags;
+  p.n_flags = prep_blocks;
+  p.err_out = err;  // the OR of the flags, for the finalize and the host
+  p.status = m->status;
+  // (a shard's archive counts come from the pass)
+  if (!arch_counts_out && pair_score_fits(L.words, n_cand, neg)) {
     Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
-    PairArgs p;
-    p.table = m->pairs;
-    p.stride = stride;
-    p.C = L.cols;
-    p.W = L.words;
-    p.terms = dterms;
-    p.n_cand = n_cand;
-    p.counts = dcounts;
-    p.bitmaps = dbm;
-    p.arch = n_arch > 0 ? dpad : nullptr;
-    p.n_arch = n_arch;
-    // all members only when the caller reads all their overlaps
-    p.score = overlaps && !sharing_only ? nullptr : dshare;
-    p.overlaps = dov;
-    p.ov_stride = ov_stride;
-    p.arch_counts = darch_counts;
-    p.flags = dflags;
-    p.n_flags = prep_blocks;
-    p.err_out = err;  // CTA 0 stores the OR of the flags here for the finalize and the host
-    p.status = m->status;
-    EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !timing_on(), s));
-  }
-  {
+    ScoreArgs f;
+    f.offsets = doffs;
+    f.arch_offsets = daoffs;
+    f.share = dshare;
+    f.fitness = dfit;
+    f.counts_mirror = counts_mirror;
+    f.err_mirror = err_mirror;
+    EBIC_CUDA(launch_pair_score(p, f, neg, !timing_on(), s));
+  } else {
+    {
+      Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
+      EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !timing_on(), s));
+    }
     Timed t(EBIC_TIMING_FITNESS, s);
     EBIC_CUDA(launch_fused_finalize(doffs, n_cand, dcounts, daoffs, n_arch, dov, ov_stride,
                                     darch_counts, dshare, dfit, err, counts_mirror, err_mirror,

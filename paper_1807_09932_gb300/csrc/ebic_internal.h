@@ -183,6 +183,22 @@ struct PairArgs {
 cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pdl,
                              cudaStream_t s);
 
+// The scores of a small call in one launch: the candidates' rows, overlaps and fitness after the
+// fused preparation (which has zeroed the overlaps). p as for launch_pair_eval with flags.
+constexpr int kScoreWarps = 8;  // most warps per block, and so the most 128-word parts of a bitmap
+struct ScoreArgs {
+  const uint32_t* offsets = nullptr;       // the population's
+  const uint32_t* arch_offsets = nullptr;
+  const uint64_t* share = nullptr;         // members sharing a column with each candidate
+  uint64_t* fitness = nullptr;             // device, or pinned host memory
+  uint32_t* counts_mirror = nullptr;       // pinned host copy of the counts, or null
+  uint32_t* err_mirror = nullptr;          // pinned host copy of the error word, or null
+};
+// Whether launch_pair_score is the faster one for n_cand candidates of W-word bitmaps.
+bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative);
+cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,
+                              cudaStream_t s);
+
 // Builds the pair table (rows of `stride` words and the all-ones row after them) from a matrix's
 // bit planes.
 cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,

@@ -78,6 +78,121 @@ __global__ void __launch_bounds__(kPairThreads, 1) pair_eval_kernel(const PairAr
   });
 }
 
+// A generation's scores in one launch after the preparation, for matrices and populations that a
+// wave or two of warps covers: a warp per 128-word part of a candidate, all of a candidate's warps
+// in one block, which therefore has its whole count and overlaps in shared memory and computes
+// its fitness itself. Against the pass above and its finalize launch there are no global
+// counters, one launch less, and the chain of a short walk is not cut into steps of two terms:
+// a warp keeps eight terms of its one part in flight (four of each direction with negative
+// trends), so a chain of up to nine columns waits for memory once. Bound by those round trips:
+// list, rows, archive rows.
+// A member's own row count is taken along with the overlap, from the same words, and only where
+// the candidate has rows at all.
+constexpr int kScoreMembers = 4;   // archive members whose words are in flight together
+constexpr int kScoreCands = 8;     // most candidates per block
+
+template <bool NEG>
+__global__ void __launch_bounds__(kScoreWarps * 32)
+    pair_score_kernel(const PairArgs p, const ScoreArgs f, int parts) {
+  __shared__ uint32_t count_s[kScoreCands];
+  __shared__ uint32_t over_s[kScoreCands][kPairMaxArch];  // overlap with each member
+  __shared__ uint32_t rows_s[kScoreCands][kPairMaxArch];  // the member's own rows
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / parts, part = warp - team * parts;
+  const uint32_t cand = blockIdx.x * (blockDim.x / (32u * parts)) + team;
+  const bool live = cand < p.n_cand;
+  for (int i = threadIdx.x; i < kScoreCands * kPairMaxArch; i += blockDim.x) {
+    (&over_s[0][0])[i] = 0u;
+    (&rows_s[0][0])[i] = 0u;
+  }
+  if (threadIdx.x < kScoreCands) count_s[threadIdx.x] = 0u;
+  // (inputs of the call, complete before the preparation started)
+  const uint32_t L = live ? f.offsets[cand + 1] - f.offsets[cand] : 1u;
+  dev::pdl_wait();  // the preparation is complete and visible
+  uint32_t bad = 0;
+  for (uint32_t i = lane; i < p.n_flags; i += 32) bad |= p.flags[i];
+  Terms t;
+  uint64_t members = 0;
+  if (live) {
+    load_terms<NEG>(p, cand, lane, t);
+    if (p.n_arch)
+      members = p.score ? p.score[cand] : p.n_arch >= 64 ? ~0ull : (1ull << p.n_arch) - 1ull;
+  }
+  bad = __reduce_or_sync(0xFFFFFFFFu, bad);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *p.err_out = bad;
+    if (f.err_mirror) *f.err_mirror = bad;
+  }
+  if (bad) return;  // the whole grid: invalid input, nothing is evaluated
+  __syncthreads();  // the shared sums are zero
+  const uint32_t word = (uint32_t)part * kRangeWords + 4u * lane;
+  uint4 x[1] = {make_uint4(0u, 0u, 0u, 0u)};
+  if (live) {
+    const uint32_t ones = (uint32_t)((uint64_t)p.C * p.C * p.stride);
+    const bool any = pair_chain<NEG, 1>(t, p.table, word, ones, lane, x);
+    if (any) {
+      const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, popc4(x[0]));
+      if (lane == 0) atomicAdd(&count_s[team], c);
+    }
+    if (p.bitmaps) {
+      uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.W + word;
+      const uint32_t v[4] = {x[0].x, x[0].y, x[0].z, x[0].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (word + j < (uint64_t)p.W) out[j] = v[j];
+    }
+  }
+  __syncthreads();
+  const uint32_t n = count_s[team];
+  if (n) {
+    const uint32_t* arch = p.arch + word;
+    for (uint64_t left = members; left;) {  // warp-uniform
+      int m[kScoreMembers];
+      uint4 v[kScoreMembers];
+#pragma unroll
+      for (int k = 0; k < kScoreMembers; ++k) {
+        m[k] = left ? __ffsll((long long)left) - 1 : -1;
+        left &= left - 1ull;
+        v[k] = m[k] >= 0 ? __ldg(reinterpret_cast<const uint4*>(arch + (uint64_t)m[k] * p.stride))
+                         : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int k = 0; k < kScoreMembers; ++k) {
+        // both sums are at most 4,096
+        const uint32_t r = __reduce_add_sync(
+            0xFFFFFFFFu, popc4(and4(x[0], v[k])) | (popc4(v[k]) << 16));
+        if (lane == 0 && r) {
+          atomicAdd(&over_s[team][m[k]], r & 0xFFFFu);
+          atomicAdd(&rows_s[team][m[k]], r >> 16);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (part != 0 || !live) return;
+  // q(a) >= q(c) of the members sharing a column decides which overlaps count
+  const uint32_t shift = (L < 33u ? L : 33u) - 1u;
+  const uint64_t qc = (uint64_t)n << shift;
+  const uint64_t share = p.n_arch ? f.share[cand] : 0ull;
+  uint32_t best = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t a = lane + 32u * h;
+    if (a >= p.n_arch) continue;
+    const uint32_t o = over_s[team][a];
+    const uint32_t al = f.arch_offsets[a + 1] - f.arch_offsets[a];
+    const uint64_t qa = (uint64_t)rows_s[team][a] << ((al < 33u ? al : 33u) - 1u);
+    if (((share >> a) & 1ull) && qa >= qc && o > best) best = o;
+    if (o) p.overlaps[(uint64_t)cand * p.ov_stride + a] = o;  // (zeroed by the preparation)
+  }
+  best = __reduce_max_sync(0xFFFFFFFFu, best);
+  if (lane == 0) {
+    p.counts[cand] = n;
+    if (f.counts_mirror) f.counts_mirror[cand] = n;
+    f.fitness[cand] = (uint64_t)(n - best) << shift;
+  }
+}
+
 // The pair table from the bit planes: a lane has two neighbouring bitmap words, a warp kBuildA
 // columns a, whose planes it keeps in registers; columns b pass through shared memory, kBuildB at
 // a time and two buffers deep (cp.async), and each serves all of the block's columns a. A table
@@ -200,6 +315,30 @@ cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pd
               : launch_variant<true, false>(p, grid, pdl, s);
   return bm ? launch_variant<false, true>(p, grid, pdl, s)
             : launch_variant<false, false>(p, grid, pdl, s);
+}
+
+// One-part bitmaps (up to 4,096 rows): the pass reads four parts whatever the rows, and its
+// finalize launch costs more than the work (200 candidates on 1,000 rows 17.3 -> 14.2 us a call
+// queued among others, 12,800 on 4,000 rows 36.5 -> 29.5). Up to eight parts with both trends,
+// where the pass takes one term a step: while the warps come to a few waves (20,000 x 200, 800
+// candidates 20.3 -> 14.9 us, 1,600 24.6 -> 21.2, 3,200 32.5 -> 30.5, 6,400 48.3 -> 49.6: there
+// the pass's order, which keeps a range's rows in L2 and L1 for all candidates, counts for more).
+// Increasing trends over several parts stay with the pass: 1,600 candidates on 20,000 rows 18.9
+// against 19.2 us.
+bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative) {
+  const int64_t parts = (W + kRangeWords - 1) / kRangeWords;
+  return parts == 1 || (negative && parts <= kScoreWarps && (int64_t)n_cand * parts <= 16000);
+}
+
+cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,
+                              cudaStream_t s) {
+  const int parts = (int)((p.W + kRangeWords - 1) / kRangeWords);
+  // several candidates per block while their warps are few
+  const int cands = parts >= kScoreCands ? 1 : kScoreCands / parts;
+  const unsigned blocks = (unsigned)(((uint64_t)p.n_cand + cands - 1) / cands);
+  count_launch();
+  return launch_maybe_pdl(pdl, negative ? pair_score_kernel<true> : pair_score_kernel<false>,
+                          dim3(blocks), dim3(32 * parts * cands), 0, s, p, f, parts);
 }
 
 cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,
