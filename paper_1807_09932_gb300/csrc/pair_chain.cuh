@@ -326,22 +326,22 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
 }
 
 // The pass over all (range, candidate group) items of one population, by a persistent grid of
-// kPairThreads-thread CTAs (see pairs.cu for the work order); `st` is the warp's kRangeWords-word
+// CTAs of WARPS warps (see pairs.cu for the work order); `st` is the warp's kRangeWords-word
 // shared staging buffer. CTA b owns items b, b + G, b + 2G, ... (G = gridDim.x); an item's
-// kPairWarps candidates are its units, and the CTA's warps take units in that order from the
+// WARPS candidates are its units, and the CTA's warps take units in that order from the
 // CTA's shared counter `next_unit` (zero at entry) as each becomes free, so a warp that drew
 // short candidates takes more of them and the CTA ends when its work ends, not when its unluckiest
 // warp does. The units of one item still run side by side on one SM, so the table rows they
 // share meet in its L1.
 // `valid()` (warp-uniform) is asked after the warp's first term list is requested and before any
 // table row is read; false ends the pass.
-template <bool NEG, bool BITMAPS, bool OVERLAP, int PARTS, class Valid>
+template <bool NEG, bool BITMAPS, bool OVERLAP, int PARTS, int WARPS, class Valid>
 __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint32_t* next_unit,
                                            Valid valid) {
   const int lane = threadIdx.x & 31;
   constexpr uint32_t kWords = PARTS * kRangeWords;  // words per item
   const uint32_t n_ranges = (uint32_t)((p.W + kWords - 1) / kWords);
-  const uint32_t n_groups = (p.n_cand + kPairWarps - 1) / kPairWarps;
+  const uint32_t n_groups = (p.n_cand + WARPS - 1) / WARPS;
   const uint64_t n_items = (uint64_t)n_ranges * n_groups;
   const bool narrow = n_items <= 0xFFFFFFFFull;  // 32-bit item arithmetic suffices
   const uint32_t n_arch = OVERLAP ? p.n_arch : 0u;
@@ -358,8 +358,8 @@ __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint
     if (lane == 0) u = atomicAdd(next_unit, 1u);
     u = __shfl_sync(0xFFFFFFFFu, u, 0);
     Unit x;
-    x.slot = u % kPairWarps;
-    x.it = blockIdx.x + (uint64_t)(u / kPairWarps) * gridDim.x;
+    x.slot = u % WARPS;
+    x.it = blockIdx.x + (uint64_t)(u / WARPS) * gridDim.x;
     x.range = x.grp = x.cand = 0;
     if (x.it < n_items) {
       if (narrow) {
@@ -369,7 +369,7 @@ __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint
         x.range = (uint32_t)(x.it / n_groups);
         x.grp = (uint32_t)(x.it - (uint64_t)x.range * n_groups);
       }
-      x.cand = x.grp * kPairWarps + x.slot;
+      x.cand = x.grp * WARPS + x.slot;
     }
     return x;
   };
@@ -387,7 +387,7 @@ __device__ __forceinline__ void pair_items(const PairArgs& p, uint32_t* st, uint
     cur = take();
     if (cur.it < n_items && cur.cand < p.n_cand) load_terms<NEG>(p, cur.cand, lane, next);
     if (arch_share) {  // the archive members' own row counts, once per range
-      for (uint32_t a = slot; a < n_arch; a += kPairWarps) {
+      for (uint32_t a = slot; a < n_arch; a += WARPS) {
         const uint32_t* ar = p.arch + (uint64_t)a * p.stride + rword + 4 * lane;
         uint32_t pa = 0;
 #pragma unroll
