@@ -120,6 +120,9 @@ int ebic_matrix_ranks(const ebic_matrix* m, uint16_t* out, void* stream);
  *   counts         out: uint32[n_cand], the matched-row count of each candidate
  *   bitmaps        out: uint32[n_cand][W] row bitmaps, or NULL for counts only
  * Results are exact integers. They do not depend on the launch configuration.
+ * On a matrix without a pair table, a population that is large against cols * cols is scored
+ * through a pair table built for the call in scratch (at most 256 MB, stream-ordered, freed with the
+ * call; not with EBIC_EVAL_DIRECT, and not when that memory is not to be had).
  */
 int ebic_eval_population(const ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                          uint32_t n_cand, uint32_t flags, uint32_t* counts, uint32_t* bitmaps,

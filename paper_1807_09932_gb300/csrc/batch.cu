@@ -599,6 +599,7 @@ __global__ void __launch_bounds__(pairdev::kPairThreads, 1)
     PairArgs pa;
     pa.bitmaps = q.bitmaps;
     pa.W = q.words;
+    pa.bitmap_stride = q.words;
     if constexpr (FIT) {
       pa.arch = q.arch_pad;
       pa.stride = q.pair_stride;

@@ -405,6 +405,23 @@ const char* check_candidates_host_c(const uint16_t* cols, const uint32_t* offset
 
 }  // namespace ebic
 
+// Words per row (a multiple of the table's) of the pair table that a call on a matrix without one
+// builds for itself in scratch, or 0 where the evaluator is the faster way. A table costs C * C
+// comparisons of every row; through it a candidate costs a quarter of what it costs the
+// evaluator. So it pays from C * C / 3 candidates on, and only where the evaluator takes some 40
+// us (candidates times words), since it adds launches. Counts and bitmaps, evaluator against
+// table: 436,444 x 64, 1,600 candidates of 2-16 columns 191 against 130 us, of 2-6 columns 162
+// against 124, 6,400 candidates 827 against 222; 100,000 x 64, 1,600 candidates 54 against 44, 400
+// (C * C / 10) 23 against 37; 436,444 x 32, 400 candidates 51 against 42; 30,000 x 50, 1,600 24
+// against 26. The table is at most kCallTable bytes; more rows are taken in ranges.
+constexpr int64_t kCallTable = 256ll << 20;
+static int64_t call_table_words(const Layout& L, uint32_t n_cand) {
+  const int64_t cc = (int64_t)L.cols * L.cols;
+  if (3ll * n_cand < cc || (int64_t)n_cand * L.words < 4000000) return 0;
+  const int64_t most = kCallTable / (cc * 4) / kPairRangeWords * kPairRangeWords;
+  return std::min(most, pair_stride(L.words));
+}
+
 static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                                 uint32_t n_cand, uint32_t flags, uint32_t* counts,
                                 uint32_t* bitmaps, void* stream) {
@@ -460,8 +477,21 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     EBIC_CUDA(out_buffer(bitmaps, (size_t)n_cand * L.words, dev, sc, &dbitmaps,
                          &bitmaps_host));
 
-  const bool use_pairs = m->pairs && !(flags & EBIC_EVAL_DIRECT);
   const bool neg = (flags & EBIC_NEGATIVE_TRENDS) != 0;
+  // the matrix's pair table, or one for the call
+  const uint32_t* pairs = flags & EBIC_EVAL_DIRECT ? nullptr : m->pairs;
+  int64_t stride = m->pair_stride;
+  uint32_t* call_table = nullptr;
+  if (!pairs && !(flags & EBIC_EVAL_DIRECT)) {
+    stride = call_table_words(L, n_cand);
+    if (stride > 0 && sc.alloc(reinterpret_cast<void**>(&call_table),
+                               ((size_t)L.cols * L.cols * stride + kOnesWords) * 4) != cudaSuccess) {
+      (void)cudaGetLastError();  // no room: the evaluator needs none
+      call_table = nullptr;
+    }
+    pairs = call_table;
+  }
+  const bool use_pairs = pairs != nullptr;
   uint32_t* dterms = nullptr;  // the pair-table term lists, built by the preparation kernel
   if (use_pairs)
     EBIC_CUDA(sc.alloc(reinterpret_cast<void**>(&dterms),
@@ -480,25 +510,33 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     pa.terms = dterms;
     pa.n_terms_cand = use_pairs ? n_cand : 0;
     pa.pair_cols = L.cols;
-    pa.pair_stride = m->pair_stride;
+    pa.pair_stride = (uint32_t)stride;
     pa.negative = neg;
     EBIC_CUDA(launch_prepare(pa, s));
   }
   if (use_pairs) {
-    Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
     PairArgs p;
-    p.table = m->pairs;
-    p.stride = m->pair_stride;
+    p.table = pairs;
+    p.stride = (uint32_t)stride;
     p.C = L.cols;
-    p.W = L.words;
     p.terms = dterms;
     p.n_cand = n_cand;
     p.counts = dcounts;
-    p.bitmaps = dbitmaps;
+    p.bitmap_stride = L.words;
     p.err = err;
     p.err_out = err;
     p.status = m->status;
-    EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !timing_on(), s));
+    // the matrix's table in one pass; a call's table one range of rows after the other
+    for (int64_t w0 = 0; w0 < L.words; w0 += stride) {
+      p.W = std::min(stride, L.words - w0);
+      p.bitmaps = dbitmaps ? dbitmaps + w0 : nullptr;
+      if (call_table) {
+        Timed t(EBIC_TIMING_EVALUATE, s);
+        EBIC_CUDA(launch_pair_build(L, m->ranks, call_table, (uint32_t)stride, w0, m->num_sms, s));
+      }
+      Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
+      EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !call_table && !timing_on(), s));
+    }
   } else {
     a.n_cand = n_cand;
     a.cand_cols = dcols;
@@ -1005,6 +1043,7 @@ static int eval_fitness_impl(const ebic_matrix* cm, const uint16_t* cols, const 
   p.n_cand = n_cand;
   p.counts = dcounts;
   p.bitmaps = dbm;
+  p.bitmap_stride = L.words;
   p.arch = n_arch > 0 ? dpad : nullptr;
   p.n_arch = n_arch;
   // all members only when the caller reads all their overlaps
@@ -1149,7 +1188,7 @@ int ebic_matrix_build_pairs(ebic_matrix* m, uint64_t max_bytes, void* stream, ui
   if (e != cudaSuccess) return cuda_fail(e, "pair table allocation");
   {
     Timed t(EBIC_TIMING_EVALUATE, s);
-    e = launch_pair_build(L, m->ranks, table, (uint32_t)stride, m->num_sms, s);
+    e = launch_pair_build(L, m->ranks, table, (uint32_t)stride, 0, m->num_sms, s);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {

@@ -163,7 +163,8 @@ struct PairArgs {
   const uint32_t* terms = nullptr;   // [n_cand][term_slots(negative)] term lists
   uint32_t n_cand = 0;
   uint32_t* counts = nullptr;        // [n_cand], zeroed before the launch
-  uint32_t* bitmaps = nullptr;       // [n_cand][W] or null
+  uint32_t* bitmaps = nullptr;       // [n_cand][bitmap_stride], W words each, or null
+  int64_t bitmap_stride = 0;
   // fused overlaps: null arch = evaluation only
   const uint32_t* arch = nullptr;    // [n_arch rounded up to even][stride], padding words zero
   uint32_t n_arch = 0;               // <= kPairMaxArch
@@ -199,10 +200,10 @@ bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative);
 cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,
                               cudaStream_t s);
 
-// Builds the pair table (rows of `stride` words and the all-ones row after them) from a matrix's
-// bit planes.
+// Builds the pair table of bitmap words word0 .. word0 + stride - 1 (rows of `stride` words and the
+// all-ones row after them) from a matrix's bit planes.
 cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,
-                              uint32_t stride, int num_sms, cudaStream_t s);
+                              uint32_t stride, int64_t word0, int num_sms, cudaStream_t s);
 
 // Preparation of the fused pass, one launch: checks the candidate list and (check_arch) the
 // archive list, zeroes counts, overlaps and archive counts, writes for every candidate the mask

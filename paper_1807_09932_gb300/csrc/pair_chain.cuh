@@ -213,7 +213,7 @@ __device__ __forceinline__ void item_epilogue(const PairArgs& p, uint32_t cand, 
                                               int lane, uint32_t n_arch, int n_pairs,
                                               uint64_t members) {
   if constexpr (BITMAPS) {  // through shared memory, so each store instruction is coalesced
-    uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.W;
+    uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.bitmap_stride;
 #pragma unroll
     for (int h = 0; h < PARTS; ++h) {
       *reinterpret_cast<uint4*>(st + 4 * lane) = x[h];

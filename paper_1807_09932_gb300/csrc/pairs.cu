@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kScoreWarps * 32)
       if (lane == 0) atomicAdd(&count_s[team], c);
     }
     if (p.bitmaps) {
-      uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.W + word;
+      uint32_t* out = p.bitmaps + (uint64_t)cand * (uint64_t)p.bitmap_stride + word;
       const uint32_t v[4] = {x[0].x, x[0].y, x[0].z, x[0].w};
 #pragma unroll
       for (int j = 0; j < 4; ++j)
@@ -217,7 +217,7 @@ constexpr int kBuildWords = 64;                    // words of a block's range
 template <int NB>
 __global__ void __launch_bounds__(kBuildWarps * 32, 2)
     pair_build_kernel(const uint32_t* __restrict__ ranks, int C, int T, uint32_t pitch_words,
-                      int64_t slabs, uint32_t* __restrict__ table, uint32_t stride,
+                      int64_t slabs, int64_t word0, uint32_t* __restrict__ table, uint32_t stride,
                       uint32_t groups_a, uint32_t groups_b, int b_per_block) {
   extern __shared__ __align__(16) uint2 bs[];  // [2][kBuildB][NB][32]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -227,9 +227,9 @@ __global__ void __launch_bounds__(kBuildWarps * 32, 2)
   const int b0 = (int)gb * b_per_block, b1 = min(C, b0 + b_per_block);
   const uint32_t word = rest / groups_a * (uint32_t)kBuildWords + 2u * lane;
   // (slabs are 2, 4, 8 or 16 words high: both of the lane's words lie in one)
-  const int64_t q = word / (uint32_t)T;
+  const int64_t q = (word0 + word) / T;
   const bool in = q < slabs;
-  const uint32_t* const src = ranks + (in ? (size_t)q * pitch_words + word % (uint32_t)T : 0);
+  const uint32_t* const src = ranks + (in ? (size_t)q * pitch_words + (word0 + word) % T : 0);
   // columns b of one buffer; past the matrix (rows or columns) zeros are written instead
   auto stage = [&](int b, int buf) {
     for (int i = warp; i < kBuildB * NB; i += kBuildWarps) {
@@ -345,7 +345,7 @@ cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negati
 }
 
 cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,
-                              uint32_t stride, int num_sms, cudaStream_t s) {
+                              uint32_t stride, int64_t word0, int num_sms, cudaStream_t s) {
   const uint32_t ga = (L.cols + kBuildCols - 1) / kBuildCols;
   const uint64_t outer = (uint64_t)(stride / kBuildWords) * ga;
   // all columns b in one block where that fills the GPU several times over, else fewer
@@ -362,7 +362,7 @@ cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* 
     if (e != cudaSuccess) return e;
     count_launch();
     pair_build_kernel<nb()><<<(unsigned)blocks, kBuildWarps * 32, smem, s>>>(
-        ranks, L.cols, L.slab_high, L.pitch_bytes / 4, L.slabs, table, stride, ga, gb, per);
+        ranks, L.cols, L.slab_high, L.pitch_bytes / 4, L.slabs, word0, table, stride, ga, gb, per);
     return cudaGetLastError();
   };
   switch (L.planes) {
