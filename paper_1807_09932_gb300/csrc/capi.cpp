@@ -798,12 +798,12 @@ static int fitness_impl(const ebic_matrix* cm, const uint16_t* cols, const uint3
   {
     Timed t(EBIC_TIMING_OVERLAP, s);
     EBIC_CUDA(launch_overlap(dbm, n_cand, dabm, n_arch, L.words, dov, darch_counts, err,
-                             m->num_sms, s));
+                             m->num_sms, !timing_on(), s));
   }
   {
     Timed t(EBIC_TIMING_FITNESS, s);
     EBIC_CUDA(launch_fitness_finalize(dcols, doffs, n_cand, dcounts, dacols, daoffs, n_arch, dov,
-                                      darch_counts, dfit, err, s));
+                                      darch_counts, dfit, err, !timing_on(), s));
   }
   const bool ac_host = arch_counts_out && n_arch > 0 && !on_device(arch_counts_out, dev);
   if (arch_counts_out && n_arch > 0)
@@ -1357,7 +1357,7 @@ int ebic_fitness_reduced(const ebic_matrix* cm, const uint16_t* cols, const uint
   {
     Timed t(EBIC_TIMING_FITNESS, s);
     EBIC_CUDA(launch_fitness_finalize(dcols, doffs, n_cand, dcounts, dacols, daoffs, n_arch, dov,
-                                      dacnt, dfit, err, s));
+                                      dacnt, dfit, err, !timing_on(), s));
   }
   if (fit_host) {
     EBIC_CUDA(cudaMemcpyAsync(fitness, dfit, (size_t)n_cand * 8, cudaMemcpyDeviceToHost, s));

@@ -270,13 +270,14 @@ cudaError_t launch_maybe_pdl(bool pdl, void (*kernel)(Params...), dim3 grid, dim
 // ---- fitness -------------------------------------------------------------------------------
 cudaError_t launch_overlap(const uint32_t* bitmaps, uint32_t n_cand, const uint32_t* arch_bitmaps,
                            uint32_t n_arch, int64_t words, uint32_t* overlaps,
-                           uint32_t* arch_counts, const uint32_t* err, int num_sms,
+                           uint32_t* arch_counts, const uint32_t* err, int num_sms, bool pdl,
                            cudaStream_t s);
 cudaError_t launch_fitness_finalize(const uint16_t* cols, const uint32_t* offsets, uint32_t n_cand,
                                     const uint32_t* counts, const uint16_t* arch_cols,
                                     const uint32_t* arch_offsets, uint32_t n_arch,
                                     const uint32_t* overlaps, const uint32_t* arch_counts,
-                                    uint64_t* fitness, const uint32_t* err, cudaStream_t s);
+                                    uint64_t* fitness, const uint32_t* err, bool pdl,
+                                    cudaStream_t s);
 
 // Row gather for the host GA: dst row k = a's row idx[k] when idx[k] >= 0, else b's row
 // -idx[k]-1 (rows of W words; idx in device memory). One launch instead of a copy per row.

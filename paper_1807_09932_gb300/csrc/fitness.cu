@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kOverlapWarps * 32, 5)
                    const uint32_t* err, uint32_t cand_blocks, uint32_t segments) {
   __shared__ uint32_t arch_s[kOvArch * kOvRow];
   __shared__ uint2 list_s[kOverlapWarps][kOvList];
-  if (*reinterpret_cast<const volatile uint32_t*>(err) != 0) return;
+  dev::pdl_trigger();  // the finalize may be scheduled; it waits for this grid
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // block = (member group, segment, candidate group), the candidates fastest: neighbours share
   // the segment's archive words in L2
@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(kOverlapWarps * 32, 5)
   const int nw = W - ws < kOvSeg ? (int)(W - ws) : kOvSeg;  // words of this segment
   const uint32_t a0 = rest / segments * kOvArch;
   const int na = n_arch - a0 < (uint32_t)kOvArch ? (int)(n_arch - a0) : kOvArch;
-  // the candidates' words are requested before the archive's are staged
+  // the candidates' words (an input of the call, complete before the preparation started) are
+  // requested while the preparation ends
   uint32_t cw[CPW][kOvNPL];
 #pragma unroll
   for (int c = 0; c < CPW; ++c)
@@ -178,6 +179,8 @@ __global__ void __launch_bounds__(kOverlapWarps * 32, 5)
       cw[c][t] = c0 + c < n_cand && w < nw
                      ? __ldg(bitmaps + (size_t)(c0 + c) * (size_t)W + ws + w) : 0u;
     }
+  dev::pdl_wait();  // the preparation (list checks, zeroed sums) is complete and visible
+  if (*reinterpret_cast<const volatile uint32_t*>(err) != 0) return;
   for (int a = warp; a < na; a += kOverlapWarps) {
     const uint32_t* src = arch + (size_t)(a0 + a) * (size_t)W + ws;
     uint32_t v[kOvNPL];
@@ -262,6 +265,7 @@ __global__ void __launch_bounds__(kFinalizeWarps * 32)
                             const uint32_t* __restrict__ arch_counts,
                             uint64_t* __restrict__ fitness, const uint32_t* err) {
   __shared__ uint32_t colset[kFinalizeWarps][(kMaxCols + 31) / 32];
+  dev::pdl_wait();  // the kernel before (overlaps, or the preparation) is complete and visible
   if (*reinterpret_cast<const volatile uint32_t*>(err) != 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t c = blockIdx.x * kFinalizeWarps + warp;
@@ -376,7 +380,7 @@ cudaError_t launch_fused_finalize(const uint32_t* offsets, uint32_t n_cand, cons
 
 cudaError_t launch_overlap(const uint32_t* bitmaps, uint32_t n_cand, const uint32_t* arch_bitmaps,
                            uint32_t n_arch, int64_t words, uint32_t* overlaps,
-                           uint32_t* arch_counts, const uint32_t* err, int num_sms,
+                           uint32_t* arch_counts, const uint32_t* err, int num_sms, bool pdl,
                            cudaStream_t s) {
   if (n_cand == 0 || n_arch == 0) return cudaSuccess;
   const uint64_t segments = (uint64_t)(words + kOvSeg - 1) / kOvSeg;
@@ -392,24 +396,23 @@ cudaError_t launch_overlap(const uint32_t* bitmaps, uint32_t n_cand, const uint3
   if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
   auto kern = one ? overlap_kernel<1> : overlap_kernel<2>;
   count_launch();
-  kern<<<(unsigned)blocks, kOverlapWarps * 32, 0, s>>>(bitmaps, n_cand, arch_bitmaps, n_arch,
-                                                       words, overlaps, arch_counts, err,
-                                                       (uint32_t)cb, (uint32_t)segments);
-  return cudaGetLastError();
+  return launch_maybe_pdl(pdl, kern, dim3((unsigned)blocks), dim3(kOverlapWarps * 32), 0, s, bitmaps,
+                          n_cand, arch_bitmaps, n_arch, words, overlaps, arch_counts, err,
+                          (uint32_t)cb, (uint32_t)segments);
 }
 
 cudaError_t launch_fitness_finalize(const uint16_t* cols, const uint32_t* offsets, uint32_t n_cand,
                                     const uint32_t* counts, const uint16_t* arch_cols,
                                     const uint32_t* arch_offsets, uint32_t n_arch,
                                     const uint32_t* overlaps, const uint32_t* arch_counts,
-                                    uint64_t* fitness, const uint32_t* err, cudaStream_t s) {
+                                    uint64_t* fitness, const uint32_t* err, bool pdl,
+                                    cudaStream_t s) {
   if (n_cand == 0) return cudaSuccess;
   const unsigned grid = (n_cand + kFinalizeWarps - 1) / kFinalizeWarps;
   count_launch();
-  fitness_finalize_kernel<<<grid, kFinalizeWarps * 32, 0, s>>>(
-      cols, offsets, n_cand, counts, arch_cols, arch_offsets, n_arch, overlaps, arch_counts,
-      fitness, err);
-  return cudaGetLastError();
+  return launch_maybe_pdl(pdl, fitness_finalize_kernel, dim3(grid), dim3(kFinalizeWarps * 32), 0, s,
+                          cols, offsets, n_cand, counts, arch_cols, arch_offsets, n_arch, overlaps,
+                          arch_counts, fitness, err);
 }
 
 }  // namespace ebic
