@@ -320,17 +320,22 @@ cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pd
             : launch_variant<false, false, 28>(p, grid, pdl, s);
 }
 
-// One-part bitmaps (up to 4,096 rows): the pass reads four parts whatever the rows, and its
-// finalize launch costs more than the work (200 candidates on 1,000 rows 17.3 -> 14.2 us a call
-// queued among others, 12,800 on 4,000 rows 36.5 -> 29.5). Up to eight parts with both trends,
-// where the pass takes one term a step: while the warps come to a few waves (20,000 x 200, 800
-// candidates 20.3 -> 14.9 us, 1,600 24.6 -> 21.2, 3,200 32.5 -> 30.5, 6,400 48.3 -> 49.6: there
-// the pass's order, which keeps a range's rows in L2 and L1 for all candidates, counts for more).
-// Increasing trends over several parts stay with the pass: 1,600 candidates on 20,000 rows 18.9
-// against 19.2 us.
+// Where the pass's items of four parts are mostly empty and its finalize launch costs more than the
+// work, up to some waves of warps; beyond, its order, which keeps a range's rows in L1 and L2 for
+// all candidates, counts for more. Measured, a call queued among others, the pass against one
+// launch (us):
+//   one part (up to 4,096 rows): 200 candidates on 1,000 rows 17.3 and 14.2; on 2,000 rows with 20
+//     members 8,000 candidates 29.3 and 25.9, 20,000 46 and 40, with 64 members 20,000 65.1 and
+//     63.4, 60,000 131 and 139;
+//   two parts: 4,756 rows 1,600 candidates 22.5 and 18.9, 3,500 23.3 and 22.7, 8,000 36 and 40;
+//   both trends, where the pass takes one term a step, up to eight parts: 20,000 x 200, 800
+//     candidates 20.3 and 14.9, 1,600 24.6 and 21.2, 3,200 32.5 and 30.5, 6,400 48.3 and 49.6;
+//   one trend over more parts stays with the pass: 20,000 rows, 1,600 candidates 18.9 and 19.2.
 bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative) {
-  const int64_t parts = (W + kRangeWords - 1) / kRangeWords;
-  return parts == 1 || (negative && parts <= kScoreWarps && (int64_t)n_cand * parts <= 16000);
+  const int64_t parts = (W + kRangeWords - 1) / kRangeWords, warps = (int64_t)n_cand * parts;
+  if (parts == 1) return warps <= 32000;
+  if (negative) return parts <= kScoreWarps && warps <= 16000;
+  return parts == 2 && warps <= 7000;
 }
 
 cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,

@@ -226,8 +226,10 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
   __syncthreads();
 
   // (B) the first candidate's columns are requested first, then every block builds the
-  // members' column sets, one (member, position) per thread; a member whose offsets fail
-  // contributes none (the list is rejected below, and the pass that follows does nothing)
+  // members' column sets, one list entry per thread (loads coalesced, the member found in the
+  // shared offsets; a thread per possible position took four rounds of loads for 64 members); of
+  // a list whose offsets fail the sets are arbitrary (it is rejected, and the pass that follows
+  // does nothing)
   const bool first_sane = gw < a.n_cand && offsets_sane(lo0, hi0, tot0, gw == 0);
   uint32_t c_lo = 0, c_hi = 0;
   if (first_sane) load_cols_regs(a.cols, lo0, hi0, lane, c_lo, c_hi);
@@ -240,35 +242,32 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
       const uint32_t lo = sh.aoff[m], hi = sh.aoff[m + 1];
       abad |= !offsets_sane(lo, hi, atotal, m == 0);
     }
-  for (uint32_t t0 = threadIdx.x; t0 < na * (uint32_t)kMaxLen; t0 += 4 * blockDim.x) {
-    uint32_t c[4], m[4];
-    bool ok[4];
+  // (a list whose total exceeds 64 columns a member is rejected above; none of it is read)
+  const uint32_t n_entries = atotal <= na * (uint32_t)kMaxLen ? atotal : 0u;
+  for (uint32_t t0 = threadIdx.x; t0 < n_entries; t0 += 4 * blockDim.x) {
+    uint32_t c[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t t = t0 + k * blockDim.x;
-      m[k] = t / kMaxLen;
-      const uint32_t j = t % kMaxLen;
-      ok[k] = false;
-      c[k] = 0u;
-      if (m[k] < na) {
-        const uint32_t lo = sh.aoff[m[k]], hi = sh.aoff[m[k] + 1];
-        const bool sane = !(m[k] == 0 && lo != 0u) && hi > lo && hi - lo <= (uint32_t)kMaxLen &&
-                          hi <= atotal;
-        ok[k] = sane && j < hi - lo;
-        if (ok[k]) c[k] = a.acols[lo + j];
-      }
+      c[k] = t < n_entries ? a.acols[t] : 0u;
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (ok[k]) {
-        if (c[k] < (uint32_t)a.ncols) {
-          const uint32_t bit = 1u << (c[k] & 31u);
-          const bool seen = (atomicOr(&sh.msets[m[k]][c[k] >> 5], bit) & bit) != 0u;
-          abad |= a.check_arch && seen;
-        } else {
-          abad |= a.check_arch;
-        }
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t t = t0 + k * blockDim.x;
+      if (t >= n_entries) continue;
+      uint32_t m = 0, hi = na;  // the last member whose columns start at or before t
+      while (hi - m > 1) {
+        const uint32_t mid = (m + hi) / 2;
+        if (sh.aoff[mid] <= t) m = mid; else hi = mid;
       }
+      if (c[k] < (uint32_t)a.ncols) {
+        const uint32_t bit = 1u << (c[k] & 31u);
+        const bool seen = (atomicOr(&sh.msets[m][c[k] >> 5], bit) & bit) != 0u;
+        abad |= a.check_arch && seen;
+      } else {
+        abad |= a.check_arch;
+      }
+    }
   }
   bool bad = false;
   if (gw < a.n_cand) {
