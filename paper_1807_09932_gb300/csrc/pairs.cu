@@ -201,20 +201,23 @@ __global__ void __launch_bounds__(kScoreWarps * 32)
 // a is present; for b = a that leaves "a present". Rows past the matrix read as code 0, so the
 // padding words come out zero, and every word of the table is written by one store, 256 bytes a
 // warp.
-// Bound by those stores (C * C rows of the padded width) with the logic pipe close behind (NB + 1
+// Bound by those stores (C * C rows of the padded width) with the logic pipe close behind (NB
 // operations per word: for NB = 9, 5 cycles of an SM per 128 bytes, 6 of its share of HBM), so
 // everything else per word is kept small: two words per lane halve the address arithmetic, four
-// columns a per warp the shared reads. Measured at 72 % of the logic pipe: 50,021 x 457 (1.7 GB)
-// 475 us, 436,444 x 64 (226 MB) 65 us; run through the evaluator as a population of all pairs
-// (with the table zeroed first) 3,670 and 355 us; one word per lane and eight columns a 559 and
-// 69 us.
+// columns a per warp the shared reads. Measured (library events, which add some 5 us): 50,021 x 457
+// (1.7 GB) 450 us, 436,444 x 64 (226 MB) 70 us, 20,000 x 200 51 us; without FOLD 485, 76 and 58;
+// one word per lane and eight columns a 566 and 76; run through the evaluator as a population of
+// all pairs (with the table zeroed first) 3,670 and 355.
 constexpr int kBuildWarps = 8;
 constexpr int kBuildA = 4;                         // columns a per warp
 constexpr int kBuildB = 16;                        // columns b per buffer
 constexpr int kBuildCols = kBuildWarps * kBuildA;  // columns a per block
 constexpr int kBuildWords = 64;                    // words of a block's range
 
-template <int NB>
+// FOLD (columns < 2^NB - 1, so that no code has every bit set): a row where a is missing is given
+// the code with every bit set in a, which no b reaches, instead of a mask at the end: one operation
+// of NB + 1 less.
+template <int NB, bool FOLD>
 __global__ void __launch_bounds__(kBuildWarps * 32, 2)
     pair_build_kernel(const uint32_t* __restrict__ ranks, int C, int T, uint32_t pitch_words,
                       int64_t slabs, int64_t word0, uint32_t* __restrict__ table, uint32_t stride,
@@ -259,6 +262,12 @@ __global__ void __launch_bounds__(kBuildWarps * 32, 2)
       here[k].x |= v.x;
       here[k].y |= v.y;
     }
+    if (FOLD)
+#pragma unroll
+      for (int p = 0; p < NB; ++p) {
+        na[k][p].x &= here[k].x;
+        na[k][p].y &= here[k].y;
+      }
   }
   uint32_t* out = table + ((uint64_t)a0 * C + b0) * stride + word;
   const uint64_t next_a = (uint64_t)C * stride;
@@ -281,8 +290,10 @@ __global__ void __launch_bounds__(kBuildWarps * 32, 2)
           g.x = (v[p].x & na[k][p].x) | (g.x & (v[p].x | na[k][p].x));
           g.y = (v[p].y & na[k][p].y) | (g.y & (v[p].y | na[k][p].y));
         }
-        g.x &= here[k].x;
-        g.y &= here[k].y;
+        if (!FOLD) {
+          g.x &= here[k].x;
+          g.y &= here[k].y;
+        }
         if (a0 + k < C) *reinterpret_cast<uint2*>(out + k * next_a) = g;
       }
     }
@@ -362,11 +373,13 @@ cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* 
   if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
   auto go = [&](auto nb) {
     const size_t smem = (size_t)2 * kBuildB * nb() * 32 * sizeof(uint2);
-    cudaError_t e = cudaFuncSetAttribute(pair_build_kernel<nb()>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = L.cols < (1 << nb()) - 1 ? pair_build_kernel<nb(), true>
+                                         : pair_build_kernel<nb(), false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
     count_launch();
-    pair_build_kernel<nb()><<<(unsigned)blocks, kBuildWarps * 32, smem, s>>>(
+    kern<<<(unsigned)blocks, kBuildWarps * 32, smem, s>>>(
         ranks, L.cols, L.slab_high, L.pitch_bytes / 4, L.slabs, word0, table, stride, ga, gb, per);
     return cudaGetLastError();
   };
