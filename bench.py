@@ -777,7 +777,9 @@ def roofline_overlap(pops, K, m, launch_ms, sms, clk):
     """The overlap kernel: P x K x W AND+popcount of 32-bit words. Its roof is the popcount
     pipe (16 per SM per clock) for the plain formulation; the carry-save tree trades half of
     the popcounts for ALU work, so the ALU pipe (64 lanes/clk/SM, ~26 ops per 8 words) is the
-    roof of the kernel as written. Both are reported; the larger minimum time binds."""
+    roof of the kernel's dense form. Both are reported; the larger minimum time binds. Segments
+    without a match are skipped and those with few matching words are walked word by word, so the
+    fractions count work that the kernel leaves out and can pass 1."""
     P = 1600
     W = m.words
     units = float(P) * K * W
@@ -797,25 +799,25 @@ def roofline_overlap(pops, K, m, launch_ms, sms, clk):
 def roofline_eval(pops, R, m, launch_ms, sms, clk, peaks):
     """The evaluator against the roof that binds it.
 
-    Algorithmic work per launch (one population): every candidate column must be read for every
-    row, sum_c L_c * R ranks of rank_bits/8 bytes each, out of shared memory (the row tile is
-    staged there by TMA); and each is one packed-field compare, 32/rank_bits rows per 32-bit
-    lane-op. Peaks from the recipe's unit counts and the median SM clock sampled during the
-    timed region: shared memory 128 B/clk/SM, INT32 ALU 64 lanes/clk/SM. The shared-memory time
-    is the larger of the two minimum times, so it is the binding roof ("bound"); the ALU and HBM
-    roofs are reported beside it. HBM: rank matrix + bitmaps against the measured copy
-    bandwidth (MEASURED_PEAKS.json).
+    Algorithmic work per launch (one population): every candidate column is read for every row,
+    sum_c L_c * R codes of NB bits each (NB = the bits of the column count), out of shared memory
+    (the row tile is staged there by bulk copies); and each is one three-input logic operation
+    per bit and 32 rows. The walk ends where no row follows any more, so long candidates read
+    less than that and the fraction can pass 1 for them. Peaks from the recipe's unit counts and
+    the median SM clock sampled during the timed region: shared memory 128 B/clk/SM, ALU 64
+    lanes/clk/SM. Shared memory is the binding roof ("bound"); the ALU and HBM roofs are
+    reported beside it. HBM: rank matrix + bitmaps against the measured copy bandwidth
+    (MEASURED_PEAKS.json).
     """
     sum_l = float(np.mean([int(o[-1]) for _, o in pops]))
-    bytes_per_rank = m.rank_bits / 8
-    fields_per_word = 32 // m.rank_bits
+    planes = int(m.cols).bit_length()
     clock_hz = (clk.get("sm_mhz") or peaks.get("sm_max_mhz") or 2070.0) * 1e6
     t = launch_ms / 1000.0
-    smem_bytes = sum_l * R * bytes_per_rank
+    smem_bytes = sum_l * R * planes / 8
     smem_peak = 128 * sms * clock_hz
-    lane_ops = sum_l * R / fields_per_word
+    lane_ops = sum_l * R / 32 * planes
     alu_peak = 64 * sms * clock_hz
-    hbm_bytes = m.cols * R * bytes_per_rank + 1600 * m.words * 4
+    hbm_bytes = m.cols * R * planes / 8 + 1600 * m.words * 4
     return {"bound": "smem", "achieved": smem_bytes / t / 1e9, "peak": smem_peak / 1e9,
             "unit": "GB/s", "frac": (smem_bytes / t) / smem_peak,
             "traffic": traffic_record("eval_population"),
@@ -827,7 +829,7 @@ def roofline_eval(pops, R, m, launch_ms, sms, clk, peaks):
             "peak_basis": "shared memory 128 B/clk/SM x SMs x median SM clock in the timed region",
             "alu": {"achieved_gops": lane_ops / t / 1e9, "peak_gops": alu_peak / 1e9,
                     "frac": (lane_ops / t) / alu_peak,
-                    "basis": "one 32-bit compare per column per 32/rank_bits rows; 64 INT32 lanes/clk/SM"},
+                    "basis": "one logic operation per plane, column and 32 rows; 64 lanes/clk/SM"},
             "hbm": {"algorithmic_bytes": hbm_bytes, "achieved_gbs": hbm_bytes / t / 1e9,
                     "peak_gbs": peaks.get("hbm_gbs"),
                     "frac": (hbm_bytes / t / 1e9) / peaks["hbm_gbs"] if "hbm_gbs" in peaks

@@ -1093,6 +1093,15 @@ static int eval_fitness_impl(const ebic_matrix* cm, const uint16_t* cols, const 
                         w_ov.dev, sync, err_mirror ? t_err_word.host : nullptr, s);
 }
 
+int ebic::eval_fitness_sharing(const ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
+                               uint32_t n_cand, uint32_t flags, const uint16_t* arch_cols,
+                               const uint32_t* arch_offsets, const uint32_t* arch_bitmaps,
+                               uint32_t n_arch, uint32_t* counts, uint32_t* bitmaps,
+                               uint64_t* fitness, uint32_t* overlaps, void* stream) {
+  return eval_fitness_impl(m, cols, offsets, n_cand, flags, arch_cols, arch_offsets, arch_bitmaps,
+                           n_arch, counts, bitmaps, fitness, overlaps, nullptr, true, stream);
+}
+
 extern "C" {
 
 int ebic_eval_fitness(const ebic_matrix* cm, const uint16_t* cols, const uint32_t* offsets,

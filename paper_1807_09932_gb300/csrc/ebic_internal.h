@@ -317,6 +317,13 @@ int set_last_error(int code, const char* msg);
 int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t W,
                      const ebic_params& p, cudaStream_t s, const uint16_t* init_cols,
                      const uint32_t* init_n, const uint64_t* init_h, ebic_result** out);
+// ebic_eval_fitness for the generation loops: the overlaps of a candidate with members that share no
+// column with it may be left 0 (admission reads none of them).
+int eval_fitness_sharing(const ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
+                         uint32_t n_cand, uint32_t flags, const uint16_t* arch_cols,
+                         const uint32_t* arch_offsets, const uint32_t* arch_bitmaps,
+                         uint32_t n_arch, uint32_t* counts, uint32_t* bitmaps, uint64_t* fitness,
+                         uint32_t* overlaps, void* stream);
 // Host-side check of a CSR candidate list; empty string when valid.
 const char* check_candidates_host_c(const uint16_t* cols, const uint32_t* offsets, uint32_t n,
                                     int32_t ncols);

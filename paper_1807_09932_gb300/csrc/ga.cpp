@@ -893,8 +893,8 @@ struct GpuEvaluator : Evaluator {
     // one generation's scoring in one call: with a pair table on the matrix, the evaluation and
     // the archive overlaps run as one pass (the bitmaps are still written: the archive update
     // needs the offered candidates' rows)
-    int rc = ebic_eval_fitness(m, dcols, doffs, n, flags, acols, aoffs, abm, n_arch, dcounts, dbm,
-                               dfit, n_arch ? dov : nullptr, s);
+    int rc = eval_fitness_sharing(m, dcols, doffs, n, flags, acols, aoffs, abm, n_arch, dcounts,
+                                  dbm, dfit, n_arch ? dov : nullptr, s);
     if (rc != EBIC_OK) return rc;
     GA_CUDA(cudaMemcpyAsync(hcnt, dcounts, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
     GA_CUDA(cudaMemcpyAsync(hfit, dfit, (size_t)n * 8, cudaMemcpyDeviceToHost, s));

@@ -1347,8 +1347,8 @@ int run_ga_on_device(const ebic_matrix* m, int64_t rows, int32_t ncols, int64_t 
     count_launch();
     tabu_insert_kernel<<<(P + 255) / 256, 256, 0, s2>>>(tabu, cp, P);
     GD_CUDA(cudaEventRecord(rs.tabu_done, s2));
-    int rc = ebic_eval_fitness(m, dcols, doffs, P, eflags, arch[par].csr_cols, arch[par].csr_offs,
-                               abm[par], K, dcounts, dbm, dfit, dov, s);
+    int rc = eval_fitness_sharing(m, dcols, doffs, P, eflags, arch[par].csr_cols,
+                                  arch[par].csr_offs, abm[par], K, dcounts, dbm, dfit, dov, s);
     if (rc != EBIC_OK) return rc;
     GD_CUDA(cudaMemsetAsync(n_offerable, 0, 4, s));
     OrderArgs oa{cp, P, p.elite, dfit, dcounts, rank, elites, offer_sorted, n_offerable};
