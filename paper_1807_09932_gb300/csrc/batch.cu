@@ -587,8 +587,8 @@ __global__ void __launch_bounds__(pairdev::kPairThreads, 1)
     const uint32_t cand = m.cand;
     uint4 x[pairdev::kParts];
     const uint32_t ones = (uint32_t)((uint64_t)q.pair_cols * q.pair_cols * q.pair_stride);
-    if (!pairdev::pair_chain<NEG, pairdev::kParts>(t, q.pairs, (uint32_t)rword + 4 * lane, ones,
-                                                   lane, x) &&
+    if (!pairdev::pair_chain<NEG, pairdev::kParts, FIT && !NEG>(
+            t, q.pairs, (uint32_t)rword + 4 * lane, ones, lane, x) &&
         !q.bitmaps)
       continue;  // no row of the item follows: nothing to add
     uint32_t pc = 0;
