@@ -478,24 +478,26 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
                          &bitmaps_host));
 
   const bool neg = (flags & EBIC_NEGATIVE_TRENDS) != 0;
-  // the matrix's pair table, or one for the call
+  // the matrix's pair table, or one for the call, and the term lists that the preparation kernel
+  // builds for it
   const uint32_t* pairs = flags & EBIC_EVAL_DIRECT ? nullptr : m->pairs;
+  const size_t term_bytes = (size_t)n_cand * term_slots(neg) * sizeof(uint32_t);
   int64_t stride = m->pair_stride;
-  uint32_t* call_table = nullptr;
-  if (!pairs && !(flags & EBIC_EVAL_DIRECT)) {
+  uint32_t *call_table = nullptr, *dterms = nullptr;
+  if (pairs) {
+    EBIC_CUDA(sc.alloc(reinterpret_cast<void**>(&dterms), term_bytes));
+  } else if (!(flags & EBIC_EVAL_DIRECT) && term_bytes <= (size_t)kCallTable) {
     stride = call_table_words(L, n_cand);
-    if (stride > 0 && sc.alloc(reinterpret_cast<void**>(&call_table),
-                               ((size_t)L.cols * L.cols * stride + kOnesWords) * 4) != cudaSuccess) {
-      (void)cudaGetLastError();  // no room: the evaluator needs none
-      call_table = nullptr;
+    if (stride > 0) {
+      const size_t bytes = ((size_t)L.cols * L.cols * stride + kOnesWords) * 4;
+      if (sc.alloc(reinterpret_cast<void**>(&call_table), bytes) == cudaSuccess &&
+          sc.alloc(reinterpret_cast<void**>(&dterms), term_bytes) == cudaSuccess)
+        pairs = call_table;
+      else
+        (void)cudaGetLastError();  // no room: the evaluator needs none
     }
-    pairs = call_table;
   }
   const bool use_pairs = pairs != nullptr;
-  uint32_t* dterms = nullptr;  // the pair-table term lists, built by the preparation kernel
-  if (use_pairs)
-    EBIC_CUDA(sc.alloc(reinterpret_cast<void**>(&dterms),
-                       (size_t)n_cand * term_slots(neg) * sizeof(uint32_t)));
   {
     Timed t(EBIC_TIMING_PREPARE, s);
     PrepareArgs pa;
@@ -507,7 +509,7 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     pa.n_zero = n_cand;
     pa.err = err;
     pa.status = m->status;
-    pa.terms = dterms;
+    pa.terms = use_pairs ? dterms : nullptr;
     pa.n_terms_cand = use_pairs ? n_cand : 0;
     pa.pair_cols = L.cols;
     pa.pair_stride = (uint32_t)stride;
@@ -530,12 +532,12 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     for (int64_t w0 = 0; w0 < L.words; w0 += stride) {
       p.W = std::min(stride, L.words - w0);
       p.bitmaps = dbitmaps ? dbitmaps + w0 : nullptr;
-      if (call_table) {
+      if (pairs == call_table) {
         Timed t(EBIC_TIMING_EVALUATE, s);
         EBIC_CUDA(launch_pair_build(L, m->ranks, call_table, (uint32_t)stride, w0, m->num_sms, s));
       }
       Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
-      EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, !call_table && !timing_on(), s));
+      EBIC_CUDA(launch_pair_eval(p, neg, m->num_sms, pairs != call_table && !timing_on(), s));
     }
   } else {
     a.n_cand = n_cand;
