@@ -212,7 +212,12 @@ __global__ void __launch_bounds__(kEvalThreads, 1) eval_population_kernel(const 
   const uint64_t per = units / gridDim.x, rem = units % gridDim.x;
   const uint64_t u0 = per * blockIdx.x + (blockIdx.x < rem ? blockIdx.x : rem);
   const uint64_t u1 = u0 + per + (blockIdx.x < rem ? 1u : 0u);
-  if (u0 >= u1) return;
+  if (u0 >= u1) {
+    // (waits all the same: with a total of 0, in a rejected list, no CTA has work, and the grid must
+    // not end before the preparation, whose outputs the next operation in the stream reads)
+    dev::pdl_wait();
+    return;
+  }
   const uint64_t i0 = u0 / kItemUnits, i1 = (u1 + kItemUnits - 1) / kItemUnits;
   __syncthreads();  // the barriers are set up
   if (tid == 0) {  // the first tiles are on their way while the preparation ends
