@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kCheckWarps * 32)
         lo[t] = __shfl_sync(0xFFFFFFFFu, lok, src);
         hi[t] = __shfl_sync(0xFFFFFFFFu, hik, src);
         const uint32_t tot = __shfl_sync(0xFFFFFFFFu, totk, src);
-        sane[t] = has[t] && prepdev::offsets_sane(lo[t], hi[t], tot, ia[t] == 0);
+        sane[t] = has[t] && offsets_sane(lo[t], hi[t], tot, ia[t] == 0);
         ca_lo[t] = ca_hi[t] = 0u;
         if (sane[t])
           prepdev::load_cols_regs(reqs[ra[t]].cand_cols, lo[t], hi[t], lane, ca_lo[t], ca_hi[t]);
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kCheckWarps * 32)
       for (uint32_t t = threadIdx.x; t < na * (uint32_t)kMaxLen; t += blockDim.x) {
         const uint32_t m = t / kMaxLen, j = t % kMaxLen;
         const uint32_t lo = ao[m], hi = ao[m + 1];
-        if (!prepdev::offsets_sane(lo, hi, atot, m == 0)) {
+        if (!offsets_sane(lo, hi, atot, m == 0)) {
           bad |= j == 0;  // once per member
           continue;
         }

@@ -69,11 +69,6 @@ __device__ inline void build_terms_warp(const uint16_t* __restrict__ cols, uint3
   }
 }
 
-__device__ __forceinline__ bool offsets_sane(uint32_t lo, uint32_t hi, uint32_t total,
-                                             bool first) {
-  return !(first && lo != 0u) && hi > lo && hi - lo <= (uint32_t)kMaxLen && hi <= total;
-}
-
 __device__ __forceinline__ void report_invalid(bool bad, uint32_t* err, uint32_t* status) {
   if (bad) {
     atomicOr(err, kErrInvalid);
@@ -227,9 +222,10 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
 
   // (B) the first candidate's columns are requested first, then every block builds the
   // members' column sets, one list entry per thread (loads coalesced, the member found in the
-  // shared offsets; a thread per possible position took four rounds of loads for 64 members); of
-  // a list whose offsets fail the sets are arbitrary (it is rejected, and the pass that follows
-  // does nothing)
+  // shared offsets; a thread per possible position took four rounds of loads for 64 members). Of
+  // a list whose offsets fail, only entries of members whose own offsets hold are read: the list's
+  // total may be one of the wrong ones, and its columns end before it. The sets are then
+  // arbitrary (the list is rejected, and the pass that follows does nothing)
   const bool first_sane = gw < a.n_cand && offsets_sane(lo0, hi0, tot0, gw == 0);
   uint32_t c_lo = 0, c_hi = 0;
   if (first_sane) load_cols_regs(a.cols, lo0, hi0, lane, c_lo, c_hi);
@@ -245,24 +241,19 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
   // (a list whose total exceeds 64 columns a member is rejected above; none of it is read)
   const uint32_t n_entries = atotal <= na * (uint32_t)kMaxLen ? atotal : 0u;
   for (uint32_t t0 = threadIdx.x; t0 < n_entries; t0 += 4 * blockDim.x) {
-    uint32_t c[4];
+    uint32_t c[4], m[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t t = t0 + k * blockDim.x;
-      c[k] = t < n_entries ? a.acols[t] : 0u;
+      m[k] = t < n_entries ? entry_member(sh.aoff, na, t) : na;
+      c[k] = m[k] < na ? a.acols[t] : 0u;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const uint32_t t = t0 + k * blockDim.x;
-      if (t >= n_entries) continue;
-      uint32_t m = 0, hi = na;  // the last member whose columns start at or before t
-      while (hi - m > 1) {
-        const uint32_t mid = (m + hi) / 2;
-        if (sh.aoff[mid] <= t) m = mid; else hi = mid;
-      }
+      if (m[k] >= na) continue;
       if (c[k] < (uint32_t)a.ncols) {
         const uint32_t bit = 1u << (c[k] & 31u);
-        const bool seen = (atomicOr(&sh.msets[m][c[k] >> 5], bit) & bit) != 0u;
+        const bool seen = (atomicOr(&sh.msets[m[k]][c[k] >> 5], bit) & bit) != 0u;
         abad |= a.check_arch && seen;
       } else {
         abad |= a.check_arch;
