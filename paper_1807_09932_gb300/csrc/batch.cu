@@ -994,7 +994,7 @@ int ebic_eval_batch(const ebic_eval_request* reqs, uint32_t n_req, void* stream)
   if (prev != hp.device) B_CUDA(cudaSetDevice(hp.device));
   void* mem = nullptr;
   const size_t bb = round_up(batch_bytes(n_req), 256);
-  B_CUDA(cudaMallocAsync(&mem, bb + hp.fit_bytes, s));
+  B_CUDA(scratch_alloc(&mem, bb + hp.fit_bytes, s));
   DeviceBatch d;
   carve(static_cast<uint8_t*>(mem), n_req, &d);
   BatchHeader h;
@@ -1037,7 +1037,7 @@ int ebic_batch_create(uint32_t max_requests, ebic_batch** out) {
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
   const size_t bytes = batch_bytes(max_requests);
-  if (e == cudaSuccess) e = cudaMalloc(&b->dmem, bytes);
+  if (e == cudaSuccess) e = fixed_alloc(reinterpret_cast<void**>(&b->dmem), bytes);
   if (e == cudaSuccess) e = cudaMallocHost(&b->hmem, bytes);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming);
   if (e != cudaSuccess) return fail_free(cerr(e, "ebic_batch_create"));
@@ -1099,7 +1099,7 @@ int ebic_batch_run(ebic_batch* b, const ebic_eval_request* reqs, uint32_t n_req,
     if (b->fmem) B_CUDA(cudaFree(b->fmem));
     b->fmem = nullptr;
     b->fbytes = 0;
-    B_CUDA(cudaMalloc(&b->fmem, hp.fit_bytes));
+    B_CUDA(fixed_alloc(reinterpret_cast<void**>(&b->fmem), hp.fit_bytes));
     b->fbytes = hp.fit_bytes;
   }
   fill_header(hp, n_req, b->h.hdr);

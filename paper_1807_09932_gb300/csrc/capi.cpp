@@ -75,7 +75,7 @@ struct Scratch {
   std::vector<void*> ptrs;
   explicit Scratch(cudaStream_t st) : s(st) {}
   cudaError_t alloc(void** p, size_t bytes) {
-    cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, s);
+    cudaError_t e = scratch_alloc(p, bytes, s);
     if (e == cudaSuccess) ptrs.push_back(*p);
     return e;
   }

@@ -1,11 +1,14 @@
-// Device memory of matrices, pair tables and searches: one stream-ordered pool per device.
+// Device memory. Matrices, pair tables and searches take theirs from one stream-ordered pool per
+// device; the calls' scratch comes from the device's default pool, and what a captured graph holds
+// the address of from cudaMalloc.
 //
 // Opening a data set takes its rank matrix and its pair table (25 MB and 226 MB for 436,444 x 64)
 // and a search some fifty buffers; cudaMalloc and cudaFree map and unmap that memory every time
 // (0.6 ms to open and close that data set, against 0.2 ms of kernels; 1.7 ms for a table of 1.7
 // GB; 0.9 ms per search). The pool keeps up to kPoolKeep bytes of what has been freed mapped for
-// the next matrix or search; anything above goes back to the system at the next synchronisation,
-// and all of it when an allocation of the library finds no memory. The pool is the driver's, so
+// the next matrix or search; anything above goes back to the system at the next synchronisation.
+// An allocation of any of the three kinds that finds no memory has both pools give back what they
+// hold unused, and is tried once more. The pool is the driver's, so
 // threads and streams may use it side by side; memory is handed from one user to the next only
 // after the first one's free is reached by its stream.
 #include <mutex>
@@ -43,6 +46,33 @@ cudaError_t pool_of(int device, cudaMemPool_t* out) {
   return cudaSuccess;
 }
 
+// What the two pools of `device` hold unused goes back to the system.
+void trim(int device) {
+  cudaMemPool_t pool = nullptr;
+  if (device >= 0 && device < kMaxDevices) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    pool = g_pool[device];
+  }
+  if (pool) (void)cudaMemPoolTrimTo(pool, 0);
+  if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) (void)cudaMemPoolTrimTo(pool, 0);
+  (void)cudaGetLastError();
+}
+
+// After an allocation on s found no memory: whether to try it again. Memory freed on s is unused
+// once s has run; a capture can neither wait for that nor be left with an error, and its
+// allocations take no memory before the graph runs.
+bool give_back(int device, cudaStream_t s) {
+  (void)cudaGetLastError();
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (cudaStreamSynchronize(s) != cudaSuccess) return false;
+  trim(device);
+  return true;
+}
+
 }  // namespace
 
 cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
@@ -50,20 +80,31 @@ cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
   cudaError_t e = pool_of(device, &pool);
   if (e != cudaSuccess) return e;
   e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
-  if (e != cudaErrorMemoryAllocation) return e;
-  // out of memory: freed memory that the pools still hold goes back first
-  (void)cudaGetLastError();
-  (void)cudaStreamSynchronize(s);
-  (void)cudaMemPoolTrimTo(pool, 0);
-  cudaMemPool_t scratch = nullptr;
-  if (cudaDeviceGetDefaultMemPool(&scratch, device) == cudaSuccess)
-    (void)cudaMemPoolTrimTo(scratch, 0);
-  (void)cudaGetLastError();
-  return cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
+  if (e == cudaErrorMemoryAllocation && give_back(device, s))
+    e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
+  return e;
 }
 
 cudaError_t device_free(void* p, cudaStream_t s) {
   return p ? cudaFreeAsync(p, s) : cudaSuccess;
+}
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, s);
+  int device = 0;
+  if (e == cudaErrorMemoryAllocation && cudaGetDevice(&device) == cudaSuccess &&
+      give_back(device, s))
+    e = cudaMallocAsync(p, bytes ? bytes : 16, s);
+  return e;
+}
+
+cudaError_t fixed_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
+  int device = 0;
+  if (e == cudaErrorMemoryAllocation && cudaGetDevice(&device) == cudaSuccess &&
+      give_back(device, nullptr))
+    e = cudaMalloc(p, bytes ? bytes : 16);
+  return e;
 }
 
 }  // namespace ebic

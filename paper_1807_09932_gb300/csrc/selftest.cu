@@ -34,7 +34,7 @@ extern "C" int ebic_selftest_wait_timeout(uint64_t timeout_ns, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* d = nullptr;
   uint32_t h = 0;
-  cudaError_t e = cudaMallocAsync(&d, sizeof(uint32_t), s);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&d), sizeof(uint32_t), s);
   if (e == cudaSuccess) {
     count_launch();
     wait_timeout_kernel<<<1, 32, 0, s>>>(timeout_ns, d);

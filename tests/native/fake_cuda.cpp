@@ -1,0 +1,234 @@
+// The CUDA runtime calls and kernel launches that the library's host code makes, on host memory: for
+// tests of what the host code does when memory runs out or a stream is captured, without a GPU.
+// Every trim, synchronisation and launch is written to a log; allocations can be made to fail.
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+
+#include "ebic.h"
+#include "ebic_internal.h"
+
+namespace {
+
+enum Kind { kPool, kAsync, kMalloc, kKinds };  // the library's pool, the default pool, cudaMalloc
+
+std::string g_log;
+int g_seen[kKinds], g_fail_from[kKinds], g_fail_count[kKinds];
+bool g_capturing;
+struct Block {
+  size_t bytes;
+  Kind kind;
+};
+std::map<char*, Block> g_live;
+
+void note(const std::string& what) { g_log += what + "\n"; }
+
+cudaError_t take(void** p, size_t bytes, Kind kind) {
+  const int n = g_seen[kind]++;
+  if (n >= g_fail_from[kind] && n < g_fail_from[kind] + g_fail_count[kind])
+    return cudaErrorMemoryAllocation;
+  char* m = static_cast<char*>(std::malloc(bytes));  // (untouched pages cost nothing)
+  g_live[m] = {bytes, kind};
+  *p = m;
+  return cudaSuccess;
+}
+
+cudaError_t drop(void* p) {
+  auto it = g_live.find(static_cast<char*>(p));
+  if (it == g_live.end()) return cudaErrorInvalidValue;
+  std::free(p);
+  g_live.erase(it);
+  return cudaSuccess;
+}
+
+const cudaMemPool_t kLibraryPool = reinterpret_cast<cudaMemPool_t>(0x10);
+const cudaMemPool_t kDefaultPool = reinterpret_cast<cudaMemPool_t>(0x20);
+
+}  // namespace
+
+extern "C" {
+
+// ---- the test's side -------------------------------------------------------------------------
+void fake_reset() {
+  g_log.clear();
+  for (int k = 0; k < kKinds; ++k) g_seen[k] = g_fail_from[k] = g_fail_count[k] = 0;
+  g_capturing = false;
+}
+// allocations `from` .. `from + count` of a kind, counted from the last reset, find no memory
+void fake_fail(int kind, int from, int count) {
+  g_fail_from[kind] = from;
+  g_fail_count[kind] = count;
+}
+void fake_capture(int on) { g_capturing = on != 0; }
+const char* fake_log() { return g_log.c_str(); }
+int fake_seen(int kind) { return g_seen[kind]; }
+size_t fake_live(int kind) {
+  size_t n = 0;
+  for (const auto& b : g_live)
+    if (b.second.kind == kind) n += b.second.bytes;
+  return n;
+}
+
+// ---- the runtime's side ------------------------------------------------------------------------
+cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
+  return take(p, n, kPool);
+}
+cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return take(p, n, kAsync); }
+cudaError_t cudaMalloc(void** p, size_t n) { return take(p, n, kMalloc); }
+cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return drop(p); }
+cudaError_t cudaFree(void* p) { return drop(p); }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
+  *p = std::calloc(1, n);
+  return cudaSuccess;
+}
+cudaError_t cudaFreeHost(void* p) {
+  std::free(p);
+  return cudaSuccess;
+}
+cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) {
+  *d = h;
+  return cudaSuccess;
+}
+cudaError_t cudaMemPoolCreate(cudaMemPool_t* pool, const cudaMemPoolProps*) {
+  *pool = kLibraryPool;
+  return cudaSuccess;
+}
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { return cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t pool, size_t keep) {
+  note((pool == kLibraryPool ? "trim library " : "trim default ") + std::to_string(keep));
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t* pool, int) {
+  *pool = kDefaultPool;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) {
+  *st = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+  note("sync");
+  return g_capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
+cudaError_t cudaDeviceSynchronize() {
+  note("sync");
+  return g_capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
+cudaError_t cudaGetDevice(int* d) {
+  *d = 0;
+  return cudaSuccess;
+}
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetDeviceCount(int* n) {
+  *n = 1;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) {
+  *v = 152;
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* at, const void* p) {
+  std::memset(at, 0, sizeof(*at));
+  const char* c = static_cast<const char*>(p);
+  for (const auto& b : g_live)
+    if (c >= b.first && c < b.first + b.second.bytes) at->type = cudaMemoryTypeDevice;
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+  std::memcpy(d, s, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  std::memcpy(d, s, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpy2DAsync(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h,
+                              cudaMemcpyKind, cudaStream_t) {
+  for (size_t i = 0; i < h; ++i)
+    std::memcpy(static_cast<char*>(d) + i * dp, static_cast<const char*>(s) + i * sp, w);
+  return cudaSuccess;
+}
+cudaError_t cudaMemset(void* p, int v, size_t n) {
+  std::memset(p, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
+  std::memset(p, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float*, cudaEvent_t, cudaEvent_t) { return cudaSuccess; }
+
+}  // extern "C"
+
+// ---- the kernels' side ----------------------------------------------------------------------------
+namespace ebic {
+
+cudaError_t launch_rank_transform(const Layout&, const float*, int64_t, int, float, uint32_t*,
+                                  uint32_t*, int, cudaStream_t) {
+  note("rank");
+  return cudaSuccess;
+}
+cudaError_t launch_prepare(const PrepareArgs&, cudaStream_t) {
+  note("prepare");
+  return cudaSuccess;
+}
+cudaError_t launch_eval(const EvalArgs&, bool, int, bool, cudaStream_t) {
+  note("evaluate");
+  return cudaSuccess;
+}
+cudaError_t launch_pair_build(const Layout&, const uint32_t*, uint32_t*, uint32_t, int64_t, int,
+                              cudaStream_t) {
+  note("pair build");
+  return cudaSuccess;
+}
+cudaError_t launch_pair_eval(const PairArgs&, bool, int, bool, cudaStream_t) {
+  note("pair evaluate");
+  return cudaSuccess;
+}
+bool pair_score_fits(int64_t, uint32_t, bool) { return false; }
+cudaError_t launch_pair_score(const PairArgs&, const ScoreArgs&, bool, bool, cudaStream_t) {
+  return cudaSuccess;
+}
+uint32_t fused_prepare_blocks(uint32_t, uint32_t, uint32_t, int) { return 1; }
+cudaError_t launch_fused_prepare(const FusedPrepareArgs&, uint32_t, cudaStream_t) {
+  return cudaSuccess;
+}
+cudaError_t launch_fused_finalize(const uint32_t*, uint32_t, const uint32_t*, const uint32_t*,
+                                  uint32_t, const uint32_t*, uint32_t, const uint32_t*,
+                                  const uint64_t*, uint64_t*, const uint32_t*, uint32_t*,
+                                  uint32_t*, bool, cudaStream_t) {
+  return cudaSuccess;
+}
+cudaError_t launch_overlap(const uint32_t*, uint32_t, const uint32_t*, uint32_t, int64_t,
+                           uint32_t*, uint32_t*, const uint32_t*, int, bool, cudaStream_t) {
+  return cudaSuccess;
+}
+cudaError_t launch_fitness_finalize(const uint16_t*, const uint32_t*, uint32_t, const uint32_t*,
+                                    const uint16_t*, const uint32_t*, uint32_t, const uint32_t*,
+                                    const uint32_t*, uint64_t*, const uint32_t*, bool,
+                                    cudaStream_t) {
+  return cudaSuccess;
+}
+
+}  // namespace ebic
+
+// the library's other allocation calls, which no entry point built here makes
+extern "C" int fake_scratch(size_t bytes) {
+  void* p = nullptr;
+  const cudaError_t e = ebic::scratch_alloc(&p, bytes, nullptr);
+  if (e == cudaSuccess) (void)cudaFreeAsync(p, nullptr);
+  return e;
+}
+extern "C" int fake_fixed(size_t bytes) {
+  void* p = nullptr;
+  const cudaError_t e = ebic::fixed_alloc(&p, bytes);
+  if (e == cudaSuccess) (void)cudaFree(p);
+  return e;
+}

@@ -1,0 +1,111 @@
+"""What the host code does when device memory runs out, on a fake CUDA runtime: every allocation of
+the library has both pools give back what they hold and is tried once more."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import native_build
+
+POOL, ASYNC, MALLOC = 0, 1, 2   # the library's pool, the default pool, cudaMalloc
+OK, OOM = 0, -2
+CUDA_OOM = 2                     # cudaErrorMemoryAllocation
+GIVEN_BACK = ["sync", "trim library 0", "trim default 0"]
+P = ctypes.c_void_p
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    lib = native_build.load(tmp_path_factory.mktemp("native"), "fake_cuda",
+                            ["capi.cpp", "devmem.cpp"])
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_live.restype = ctypes.c_size_t
+    lib.fake_scratch.argtypes = lib.fake_fixed.argtypes = [ctypes.c_size_t]
+    lib.ebic_load_matrix.argtypes = [P, ctypes.c_int64, ctypes.c_int32, ctypes.c_int64,
+                                     ctypes.c_uint32, ctypes.c_float, P, ctypes.POINTER(P)]
+    lib.ebic_eval_population.argtypes = [P, P, P, ctypes.c_uint32, ctypes.c_uint32, P, P, P]
+    lib.ebic_matrix_build_pairs.argtypes = [P, ctypes.c_uint64, P, P]
+    lib.ebic_free_matrix.argtypes = [P]
+    lib.ebic_matrix_drop_pairs.argtypes = [P]
+    lib.fake_reset()
+    return lib
+
+
+def log(lib):
+    return lib.fake_log().decode().splitlines()
+
+
+def load(lib, rows, cols):
+    x = np.zeros((rows, cols), np.float32)
+    h = P()
+    rc = lib.ebic_load_matrix(x.ctypes.data, rows, cols, cols, 1, 0.0, None, ctypes.byref(h))
+    return rc, h
+
+
+class Population:
+    def __init__(self, n):
+        self.n = n
+        self.cols = np.tile(np.array([0, 1], np.uint16), n)
+        self.offs = np.arange(0, 2 * n + 1, 2, dtype=np.uint32)
+        self.counts = np.zeros(n, np.uint32)
+
+    def score(self, lib, h, flags=0):
+        return lib.ebic_eval_population(h, self.cols.ctypes.data, self.offs.ctypes.data, self.n,
+                                        flags, self.counts.ctypes.data, None, None)
+
+
+def test_matrix_and_table_tried_again(lib):
+    rc, h = load(lib, 3000, 20)
+    assert rc == OK
+    lib.fake_reset()
+    lib.fake_fail(POOL, 0, 1)
+    rc, h2 = load(lib, 3000, 20)
+    assert rc == OK and log(lib)[:3] == GIVEN_BACK
+    lib.fake_reset()
+    lib.fake_fail(POOL, 0, 1)
+    assert lib.ebic_matrix_build_pairs(h, 1 << 40, None, None) == OK
+    assert log(lib)[:3] == GIVEN_BACK
+    lib.fake_reset()
+    lib.fake_fail(POOL, 0, 2)
+    assert lib.ebic_matrix_build_pairs(h2, 1 << 40, None, None) == OOM
+    assert load(lib, 3000, 20)[0] == OK
+    for m in (h, h2):
+        lib.ebic_free_matrix(m)
+
+
+def test_scratch_tried_again(lib):
+    rc, h = load(lib, 3000, 20)
+    pop = Population(10)
+    lib.fake_reset()
+    assert pop.score(lib, h) == OK
+    held, calls = lib.fake_live(ASYNC), lib.fake_seen(ASYNC)
+    assert held == 0 and calls >= 3 and "trim library 0" not in log(lib)
+    for k in range(calls):  # each of the call's allocations in turn
+        lib.fake_reset()
+        lib.fake_fail(ASYNC, k, 1)
+        assert pop.score(lib, h) == OK
+        assert [x for x in log(lib) if x.startswith("trim")] == GIVEN_BACK[1:]
+        lib.fake_reset()
+        lib.fake_fail(ASYNC, k, 2)
+        assert pop.score(lib, h) == OOM
+        assert lib.fake_live(ASYNC) == 0  # nothing stays behind
+    lib.ebic_free_matrix(h)
+
+
+@pytest.mark.parametrize("kind,call", [(ASYNC, "fake_scratch"), (MALLOC, "fake_fixed")])
+def test_the_batch_allocations_tried_again(lib, kind, call):
+    lib.fake_reset()
+    lib.fake_fail(kind, 0, 1)
+    assert getattr(lib, call)(1 << 20) == OK and log(lib) == GIVEN_BACK
+    lib.fake_reset()
+    lib.fake_fail(kind, 0, 2)
+    assert getattr(lib, call)(1 << 20) == CUDA_OOM
+
+
+def test_a_capture_is_left_alone(lib):
+    lib.fake_reset()
+    lib.fake_capture(1)
+    lib.fake_fail(ASYNC, 0, 1)
+    assert lib.fake_scratch(1 << 20) == CUDA_OOM
+    assert log(lib) == []
+    lib.fake_reset()
