@@ -91,10 +91,11 @@ typedef struct ebic_matrix ebic_matrix;
 int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uint32_t flags,
                      float fill_value, void* stream, ebic_matrix** out);
 
-/* Free a matrix handle and its device memory. Synchronizes the device. NULL is a no-op. Up to
- * 2 GiB of freed device memory per device stays with the library's pool for the next matrix or
- * search (mapping it again costs more than opening most data sets); what is above goes back to
- * the system, and all of it when an allocation of the library finds no memory. */
+/* Free a matrix handle and its device memory. Synchronizes the device. NULL is a no-op. Freed
+ * device memory stays with the library's pool for the next matrix or search (mapping it again costs
+ * more than opening most data sets) while that pool holds at most 2 GiB per device, in use and
+ * not; beyond that it goes back to the system, and all that is unused does when an allocation that
+ * a call of the library needs finds no memory. */
 int ebic_free_matrix(ebic_matrix* m);
 
 /*
@@ -121,8 +122,9 @@ int ebic_matrix_ranks(const ebic_matrix* m, uint16_t* out, void* stream);
  *   bitmaps        out: uint32[n_cand][W] row bitmaps, or NULL for counts only
  * Results are exact integers. They do not depend on the launch configuration.
  * On a matrix without a pair table, a population that is large against cols * cols is scored
- * through a pair table built for the call in scratch (at most 256 MB, stream-ordered, freed with the
- * call; not with EBIC_EVAL_DIRECT, and not when that memory is not to be had).
+ * through a pair table built for the call (at most 256 MB, and as much again for term lists,
+ * stream-ordered and freed with the call, from a pool like the one that ebic_free_matrix describes
+ * with a limit of 512 MiB; not with EBIC_EVAL_DIRECT, and not when that memory is not to be had).
  */
 int ebic_eval_population(const ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                          uint32_t n_cand, uint32_t flags, uint32_t* counts, uint32_t* bitmaps,

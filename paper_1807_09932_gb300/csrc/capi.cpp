@@ -79,6 +79,12 @@ struct Scratch {
     if (e == cudaSuccess) ptrs.push_back(*p);
     return e;
   }
+  // From a pool that keeps a bounded amount (the default pool keeps all that it ever held).
+  cudaError_t alloc_table(void** p, size_t bytes, int device) {
+    cudaError_t e = call_table_alloc(p, bytes, device, s);
+    if (e == cudaSuccess) ptrs.push_back(*p);
+    return e;
+  }
   ~Scratch() {
     for (void* p : ptrs) (void)cudaFreeAsync(p, s);
   }
@@ -490,8 +496,8 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     stride = call_table_words(L, n_cand);
     if (stride > 0) {
       const size_t bytes = ((size_t)L.cols * L.cols * stride + kOnesWords) * 4;
-      if (sc.alloc(reinterpret_cast<void**>(&call_table), bytes) == cudaSuccess &&
-          sc.alloc(reinterpret_cast<void**>(&dterms), term_bytes) == cudaSuccess)
+      if (sc.alloc_table(reinterpret_cast<void**>(&call_table), bytes, dev) == cudaSuccess &&
+          sc.alloc_table(reinterpret_cast<void**>(&dterms), term_bytes, dev) == cudaSuccess)
         pairs = call_table;
       else
         (void)cudaGetLastError();  // no room: the evaluator needs none

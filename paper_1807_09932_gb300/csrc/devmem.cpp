@@ -1,15 +1,16 @@
 // Device memory. Matrices, pair tables and searches take theirs from one stream-ordered pool per
-// device; the calls' scratch comes from the device's default pool, and what a captured graph holds
-// the address of from cudaMalloc.
+// device, the pair table of a single call from another; the calls' other scratch comes from the
+// device's default pool, and what a captured graph holds the address of from cudaMalloc.
 //
 // Opening a data set takes its rank matrix and its pair table (25 MB and 226 MB for 436,444 x 64)
 // and a search some fifty buffers; cudaMalloc and cudaFree map and unmap that memory every time
 // (0.6 ms to open and close that data set, against 0.2 ms of kernels; 1.7 ms for a table of 1.7
-// GB; 0.9 ms per search). The pool keeps up to kPoolKeep bytes of what has been freed mapped for
-// the next matrix or search; anything above goes back to the system at the next synchronisation.
-// An allocation of any of the three kinds that finds no memory has both pools give back what they
-// hold unused, and is tried once more. The pool is the driver's, so
-// threads and streams may use it side by side; memory is handed from one user to the next only
+// GB; 0.9 ms per search). A pool keeps freed memory mapped for the next user while it holds, used
+// and unused, no more than its limit; beyond that, freed memory goes back to the system at the
+// next synchronisation. An allocation that finds no memory has all the pools give back what they hold
+// unused, and is tried once more (not a call's pair table: the call does without one, and need not
+// wait for its stream). The pools are the driver's, so
+// threads and streams may use them side by side; memory is handed from one user to the next only
 // after the first one's free is reached by its stream.
 #include <mutex>
 
@@ -18,15 +19,18 @@
 namespace ebic {
 namespace {
 
-constexpr uint64_t kPoolKeep = 2ull << 30;  // under 1 % of the device's memory
+enum Pool { kLasting, kCall, kPools };
+// Together under 1 % of the device's memory. The second is what one call takes at most, and a pool of
+// its own so that the matrices loaded beside it don't count against its limit.
+constexpr uint64_t kPoolKeep[kPools] = {2ull << 30, 512ull << 20};
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-cudaMemPool_t g_pool[kMaxDevices] = {};
+cudaMemPool_t g_pool[kMaxDevices][kPools] = {};
 
-cudaError_t pool_of(int device, cudaMemPool_t* out) {
+cudaError_t pool_of(int device, Pool which, cudaMemPool_t* out) {
   if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_pool[device]) {
+  if (!g_pool[device][which]) {
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -34,27 +38,28 @@ cudaError_t pool_of(int device, cudaMemPool_t* out) {
     cudaMemPool_t pool = nullptr;
     cudaError_t e = cudaMemPoolCreate(&pool, &props);
     if (e != cudaSuccess) return e;
-    uint64_t keep = kPoolKeep;
+    uint64_t keep = kPoolKeep[which];
     e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     if (e != cudaSuccess) {
       (void)cudaMemPoolDestroy(pool);
       return e;
     }
-    g_pool[device] = pool;
+    g_pool[device][which] = pool;
   }
-  *out = g_pool[device];
+  *out = g_pool[device][which];
   return cudaSuccess;
 }
 
-// What the two pools of `device` hold unused goes back to the system.
+// What the pools of `device` hold unused goes back to the system.
 void trim(int device) {
-  cudaMemPool_t pool = nullptr;
   if (device >= 0 && device < kMaxDevices) {
     std::lock_guard<std::mutex> lk(g_mu);
-    pool = g_pool[device];
+    for (cudaMemPool_t pool : g_pool[device])
+      if (pool) (void)cudaMemPoolTrimTo(pool, 0);
   }
-  if (pool) (void)cudaMemPoolTrimTo(pool, 0);
-  if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) (void)cudaMemPoolTrimTo(pool, 0);
+  cudaMemPool_t scratch = nullptr;
+  if (cudaDeviceGetDefaultMemPool(&scratch, device) == cudaSuccess)
+    (void)cudaMemPoolTrimTo(scratch, 0);
   (void)cudaGetLastError();
 }
 
@@ -77,12 +82,18 @@ bool give_back(int device, cudaStream_t s) {
 
 cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
   cudaMemPool_t pool = nullptr;
-  cudaError_t e = pool_of(device, &pool);
+  cudaError_t e = pool_of(device, kLasting, &pool);
   if (e != cudaSuccess) return e;
   e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
   if (e == cudaErrorMemoryAllocation && give_back(device, s))
     e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
   return e;
+}
+
+cudaError_t call_table_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
+  cudaMemPool_t pool = nullptr;
+  const cudaError_t e = pool_of(device, kCall, &pool);
+  return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s) : e;
 }
 
 cudaError_t device_free(void* p, cudaStream_t s) {

@@ -78,7 +78,10 @@ void count_launches(int64_t n);  // n kernels at once (a negative n takes back c
 // Freed memory must no longer be in use by any stream but s.
 cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s);
 cudaError_t device_free(void* p, cudaStream_t s);
-// A call's scratch on the current device, stream-ordered on s; freed with cudaFreeAsync.
+// A single call's pair table and term lists, from a pool of their own; freed with cudaFreeAsync. Not
+// tried again when there is no memory.
+cudaError_t call_table_alloc(void** p, size_t bytes, int device, cudaStream_t s);
+// A call's other scratch on the current device, stream-ordered on s; freed with cudaFreeAsync.
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 // Memory of the current device that is no stream's (a captured graph holds its address); freed with
 // cudaFree.

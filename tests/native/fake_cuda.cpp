@@ -11,7 +11,8 @@
 
 namespace {
 
-enum Kind { kPool, kAsync, kMalloc, kKinds };  // the library's pool, the default pool, cudaMalloc
+// the pool of matrices and tables, the default pool, cudaMalloc, the pool of calls' tables
+enum Kind { kPool, kAsync, kMalloc, kCallPool, kKinds };
 
 std::string g_log;
 int g_seen[kKinds], g_fail_from[kKinds], g_fail_count[kKinds];
@@ -42,8 +43,15 @@ cudaError_t drop(void* p) {
   return cudaSuccess;
 }
 
-const cudaMemPool_t kLibraryPool = reinterpret_cast<cudaMemPool_t>(0x10);
-const cudaMemPool_t kDefaultPool = reinterpret_cast<cudaMemPool_t>(0x20);
+// pools by their handles: the library's, told apart by their limits, then the default one
+char g_handles[3];
+const cudaMemPool_t kDefaultPool = reinterpret_cast<cudaMemPool_t>(&g_handles[2]);
+int g_pools;
+uint64_t g_limit[2];
+Kind kind_of(cudaMemPool_t pool) {
+  const int i = (int)(reinterpret_cast<char*>(pool) - g_handles);
+  return i == 2 ? kAsync : g_limit[i] == (2ull << 30) ? kPool : kCallPool;
+}
 
 }  // namespace
 
@@ -63,6 +71,11 @@ void fake_fail(int kind, int from, int count) {
 void fake_capture(int on) { g_capturing = on != 0; }
 const char* fake_log() { return g_log.c_str(); }
 int fake_seen(int kind) { return g_seen[kind]; }
+uint64_t fake_limit(int kind) {
+  for (int i = 0; i < g_pools; ++i)
+    if (kind_of(reinterpret_cast<cudaMemPool_t>(&g_handles[i])) == kind) return g_limit[i];
+  return 0;
+}
 size_t fake_live(int kind) {
   size_t n = 0;
   for (const auto& b : g_live)
@@ -71,8 +84,8 @@ size_t fake_live(int kind) {
 }
 
 // ---- the runtime's side ------------------------------------------------------------------------
-cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
-  return take(p, n, kPool);
+cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t pool, cudaStream_t) {
+  return take(p, n, kind_of(pool));
 }
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return take(p, n, kAsync); }
 cudaError_t cudaMalloc(void** p, size_t n) { return take(p, n, kMalloc); }
@@ -91,13 +104,20 @@ cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) {
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* pool, const cudaMemPoolProps*) {
-  *pool = kLibraryPool;
+  if (g_pools == 2) return cudaErrorUnknown;
+  *pool = reinterpret_cast<cudaMemPool_t>(&g_handles[g_pools++]);
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { return cudaSuccess; }
-cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t pool, cudaMemPoolAttr, void* v) {
+  if (pool != kDefaultPool)
+    g_limit[reinterpret_cast<char*>(pool) - g_handles] = *static_cast<uint64_t*>(v);
+  return cudaSuccess;
+}
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t pool, size_t keep) {
-  note((pool == kLibraryPool ? "trim library " : "trim default ") + std::to_string(keep));
+  const Kind k = kind_of(pool);
+  note((k == kPool ? "trim library " : k == kAsync ? "trim default " : "trim tables ") +
+       std::to_string(keep));
   return cudaSuccess;
 }
 cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t* pool, int) {
