@@ -124,7 +124,8 @@ int ebic_matrix_ranks(const ebic_matrix* m, uint16_t* out, void* stream);
  * On a matrix without a pair table, a population that is large against cols * cols is scored
  * through a pair table built for the call (at most 256 MB, and as much again for term lists,
  * stream-ordered and freed with the call, from a pool like the one that ebic_free_matrix describes
- * with a limit of 512 MiB; not with EBIC_EVAL_DIRECT, and not when that memory is not to be had).
+ * with a limit of 512 MiB; not with EBIC_EVAL_DIRECT, not in a stream capture, and not when that
+ * memory is not to be had).
  */
 int ebic_eval_population(const ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                          uint32_t n_cand, uint32_t flags, uint32_t* counts, uint32_t* bitmaps,

@@ -428,6 +428,15 @@ static int64_t call_table_words(const Layout& L, uint32_t n_cand) {
   return std::min(most, pair_stride(L.words));
 }
 
+// A captured call takes no table: its graph would hold the table's memory for as long as it exists, and
+// could not fall back to the evaluator when a replay finds none.
+static bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();
+  return true;
+}
+
 static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                                 uint32_t n_cand, uint32_t flags, uint32_t* counts,
                                 uint32_t* bitmaps, void* stream) {
@@ -494,7 +503,7 @@ static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint
     EBIC_CUDA(sc.alloc(reinterpret_cast<void**>(&dterms), term_bytes));
   } else if (!(flags & EBIC_EVAL_DIRECT) && term_bytes <= (size_t)kCallTable) {
     stride = call_table_words(L, n_cand);
-    if (stride > 0) {
+    if (stride > 0 && !is_capturing(s)) {
       const size_t bytes = ((size_t)L.cols * L.cols * stride + kOnesWords) * 4;
       if (sc.alloc_table(reinterpret_cast<void**>(&call_table), bytes, dev) == cudaSuccess &&
           sc.alloc_table(reinterpret_cast<void**>(&dterms), term_bytes, dev) == cudaSuccess)

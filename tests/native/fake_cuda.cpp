@@ -83,6 +83,13 @@ size_t fake_live(int kind) {
   return n;
 }
 
+void* fake_device(size_t bytes) {
+  void* p = nullptr;
+  (void)take(&p, bytes, kMalloc);
+  return p;
+}
+void fake_device_free(void* p) { (void)drop(p); }
+
 // ---- the runtime's side ------------------------------------------------------------------------
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t pool, cudaStream_t) {
   return take(p, n, kind_of(pool));

@@ -21,6 +21,9 @@ def lib(tmp_path_factory):
     lib.fake_log.restype = ctypes.c_char_p
     lib.fake_live.restype = ctypes.c_size_t
     lib.fake_limit.restype = ctypes.c_uint64
+    lib.fake_device.restype = P
+    lib.fake_device.argtypes = [ctypes.c_size_t]
+    lib.fake_device_free.argtypes = [P]
     lib.fake_scratch.argtypes = lib.fake_fixed.argtypes = [ctypes.c_size_t]
     lib.ebic_load_matrix.argtypes = [P, ctypes.c_int64, ctypes.c_int32, ctypes.c_int64,
                                      ctypes.c_uint32, ctypes.c_float, P, ctypes.POINTER(P)]
@@ -151,4 +154,24 @@ def test_call_table_without_memory_falls_back(lib, which):
     assert not any(x.startswith("trim") for x in log(lib))   # nor does the call wait for memory
     assert [x for x in log(lib) if x in ("pair build", "pair evaluate", "evaluate")] == ["evaluate"]
     assert lib.fake_live(TABLE) == 0
+    lib.ebic_free_matrix(h)
+
+
+def test_captured_call_takes_no_table(lib):
+    rows, cols, n = BIG
+    rc, h = load(lib, rows, cols)
+    dev = {}
+    for name, a in (("cols", Population(n).cols), ("offs", Population(n).offs),
+                    ("counts", np.zeros(n, np.uint32))):
+        dev[name] = lib.fake_device(a.nbytes)
+        ctypes.memmove(dev[name], a.ctypes.data, a.nbytes)
+    lib.fake_reset()
+    lib.fake_capture(1)
+    rc = lib.ebic_eval_population(h, dev["cols"], dev["offs"], n, 0, dev["counts"], None, None)
+    assert rc == OK and log(lib) == ["prepare", "evaluate"] and lib.fake_seen(TABLE) == 0
+    lib.fake_reset()
+    rc = lib.ebic_eval_population(h, dev["cols"], dev["offs"], n, 0, dev["counts"], None, None)
+    assert rc == OK and log(lib) == ["prepare", "pair build", "pair evaluate"]
+    for d in dev.values():
+        lib.fake_device_free(d)
     lib.ebic_free_matrix(h)
