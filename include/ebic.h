@@ -98,6 +98,11 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
  * a call of the library needs finds no memory. */
 int ebic_free_matrix(ebic_matrix* m);
 
+/* Give the memory that the library's pools and the device's default pool hold unused back to the
+ * system, for another allocator of the process to take. Synchronizes the device. device: its index,
+ * or -1 for the current one. */
+int ebic_release_memory(int32_t device);
+
 /*
  * Shape of a loaded matrix. Any output pointer may be NULL.
  *   words      W = ceil(rows/32), the bitmap length per candidate

@@ -681,6 +681,16 @@ int ebic_free_matrix(ebic_matrix* m) {
   return EBIC_OK;
 }
 
+int ebic_release_memory(int32_t device) {
+  int n = 0, dev = device;
+  EBIC_CUDA(cudaGetDeviceCount(&n));
+  if (device == -1) EBIC_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= n) return fail(EBIC_ERR_INVALID_ARG, "no such device");
+  DeviceGuard g(dev);
+  EBIC_CUDA(release_memory(dev));
+  return EBIC_OK;
+}
+
 int ebic_matrix_info(const ebic_matrix* m, int64_t* rows, int32_t* cols, int64_t* words,
                      int32_t* rank_bits) {
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");

@@ -109,6 +109,12 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
+cudaError_t release_memory(int device) {
+  const cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) trim(device);
+  return e;
+}
+
 cudaError_t fixed_alloc(void** p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
   int device = 0;

@@ -78,6 +78,8 @@ void count_launches(int64_t n);  // n kernels at once (a negative n takes back c
 // Freed memory must no longer be in use by any stream but s.
 cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s);
 cudaError_t device_free(void* p, cudaStream_t s);
+// What the pools of `device`, the current one, hold unused goes back to the system, once it is idle.
+cudaError_t release_memory(int device);
 // A single call's pair table and term lists, from a pool of their own; freed with cudaFreeAsync. Not
 // tried again when there is no memory.
 cudaError_t call_table_alloc(void** p, size_t bytes, int device, cudaStream_t s);

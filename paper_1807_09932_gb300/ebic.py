@@ -68,6 +68,7 @@ def _sig(name, args, res=ctypes.c_int):
 _lib_load = _sig("ebic_load_matrix", [_P, _I64, _I32, _I64, _U32, ctypes.c_float, _P,
                                       ctypes.POINTER(_P)])
 _lib_free = _sig("ebic_free_matrix", [_P])
+_lib_release = _sig("ebic_release_memory", [_I32])
 _lib_info = _sig("ebic_matrix_info", [_P, ctypes.POINTER(_I64), ctypes.POINTER(_I32),
                                       ctypes.POINTER(_I64), ctypes.POINTER(_I32)])
 _lib_ranks = _sig("ebic_matrix_ranks", [_P, _P, _P])
@@ -334,6 +335,12 @@ def ebic_matrix_build_pairs(h, max_bytes, stream=None):
     _check(_lib_build_pairs(h, max_bytes, _stream(stream), ctypes.byref(n)),
            "ebic_matrix_build_pairs")
     return n.value
+
+
+def ebic_release_memory(device=-1):
+    """Give the memory that the library keeps mapped for the next matrix or search back to the
+    system (and to other allocators of the process). Synchronizes the device (-1: the current)."""
+    _check(_lib_release(int(device)), "ebic_release_memory")
 
 
 def ebic_matrix_drop_pairs(h):

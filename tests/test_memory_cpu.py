@@ -175,3 +175,15 @@ def test_captured_call_takes_no_table(lib):
     for d in dev.values():
         lib.fake_device_free(d)
     lib.ebic_free_matrix(h)
+
+
+def test_release(lib):
+    rows, cols, n = BIG
+    rc, h = load(lib, rows, cols)
+    assert Population(n).score(lib, h) == OK
+    lib.ebic_free_matrix(h)
+    lib.fake_reset()
+    assert lib.ebic_release_memory(ctypes.c_int32(-1)) == OK
+    assert log(lib)[0] == "sync"
+    assert set(log(lib)[1:]) == {"trim library 0", "trim tables 0", "trim default 0"}
+    assert lib.ebic_release_memory(ctypes.c_int32(7)) == -1
