@@ -98,6 +98,10 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
  * a call of the library needs finds no memory. */
 int ebic_free_matrix(ebic_matrix* m);
 
+/* Device bytes that a loaded matrix of this shape takes, and those of its pair table
+ * (ebic_matrix_build_pairs). Either output may be NULL. */
+int ebic_matrix_bytes(int64_t rows, int32_t cols, uint64_t* matrix, uint64_t* pairs);
+
 /* Give the memory that the library's pools and the device's default pool hold unused back to the
  * system, for another allocator of the process to take. Synchronizes the device. device: its index,
  * or -1 for the current one. */

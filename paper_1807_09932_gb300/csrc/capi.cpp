@@ -437,6 +437,13 @@ static bool is_capturing(cudaStream_t s) {
   return true;
 }
 
+// A matrix's device memory: its bit planes, then the status word in kStatusBytes of its own.
+constexpr size_t kStatusBytes = 256;
+static size_t rank_bytes(const Layout& L) { return (L.rank_words() * 4 + 255) / 256 * 256; }
+static uint64_t pair_table_bytes(const Layout& L) {
+  return (uint64_t)L.cols * L.cols * pair_stride(L.words) * 4 + kOnesWords * 4;
+}
+
 static int eval_population_impl(ebic_matrix* m, const uint16_t* cols, const uint32_t* offsets,
                                 uint32_t n_cand, uint32_t flags, uint32_t* counts,
                                 uint32_t* bitmaps, void* stream) {
@@ -623,13 +630,13 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
   cudaError_t e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
   // the rank matrix, and the status word after it
-  const size_t rank_bytes = (m->L.rank_words() * 4 + 255) / 256 * 256;
-  e = device_alloc(reinterpret_cast<void**>(&m->ranks), rank_bytes + 256, dev, s);
+  const size_t ranks = rank_bytes(m->L);
+  e = device_alloc(reinterpret_cast<void**>(&m->ranks), ranks + kStatusBytes, dev, s);
   if (e != cudaSuccess) {
     m->ranks = nullptr;
     return cleanup(cuda_fail(e, "allocation of the rank matrix"));
   }
-  m->status = m->ranks + rank_bytes / 4;
+  m->status = m->ranks + ranks / 4;
   e = cudaMemsetAsync(m->status, 0, sizeof(uint32_t), s);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "status word"));
 
@@ -678,6 +685,15 @@ int ebic_free_matrix(ebic_matrix* m) {
   if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
   delete m;
   if (e != cudaSuccess) return cuda_fail(e, "freeing a matrix");
+  return EBIC_OK;
+}
+
+int ebic_matrix_bytes(int64_t rows, int32_t cols, uint64_t* matrix, uint64_t* pairs) {
+  if (rows < 1 || rows > INT32_MAX || cols < 1 || cols > kMaxCols)
+    return fail(EBIC_ERR_INVALID_ARG, "no matrix has this shape");
+  const Layout L = make_layout(rows, cols);
+  if (matrix) *matrix = rank_bytes(L) + kStatusBytes;
+  if (pairs) *pairs = pair_table_bytes(L);
   return EBIC_OK;
 }
 
@@ -1208,13 +1224,12 @@ int ebic_matrix_build_pairs(ebic_matrix* m, uint64_t max_bytes, void* stream, ui
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
   const Layout& L = m->L;
   const int64_t stride = pair_stride(L.words);
-  const uint64_t rows = (uint64_t)L.cols * (uint64_t)L.cols * (uint64_t)stride * 4ull;
-  const uint64_t need = rows + (uint64_t)kOnesWords * 4ull;
+  const uint64_t need = pair_table_bytes(L);
   if (bytes) *bytes = need;
   if (need > max_bytes)
     return fail(EBIC_ERR_UNSUPPORTED, "the pair table needs " + std::to_string(need) +
                                           " bytes, more than max_bytes");
-  if (rows / 4ull > 0xFFFFFFFFull)  // table rows are addressed with 32-bit word offsets
+  if (need / 4ull - kOnesWords > 0xFFFFFFFFull)  // table rows are addressed with 32-bit word offsets
     return fail(EBIC_ERR_UNSUPPORTED, "the pair table would exceed 2^32 words");
   DeviceGuard g(m->device);
   if (m->pairs) return EBIC_OK;

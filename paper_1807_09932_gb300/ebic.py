@@ -68,6 +68,8 @@ def _sig(name, args, res=ctypes.c_int):
 _lib_load = _sig("ebic_load_matrix", [_P, _I64, _I32, _I64, _U32, ctypes.c_float, _P,
                                       ctypes.POINTER(_P)])
 _lib_free = _sig("ebic_free_matrix", [_P])
+_lib_bytes = _sig("ebic_matrix_bytes", [_I64, _I32, ctypes.POINTER(ctypes.c_uint64),
+                                          ctypes.POINTER(ctypes.c_uint64)])
 _lib_release = _sig("ebic_release_memory", [_I32])
 _lib_info = _sig("ebic_matrix_info", [_P, ctypes.POINTER(_I64), ctypes.POINTER(_I32),
                                       ctypes.POINTER(_I64), ctypes.POINTER(_I32)])
@@ -335,6 +337,13 @@ def ebic_matrix_build_pairs(h, max_bytes, stream=None):
     _check(_lib_build_pairs(h, max_bytes, _stream(stream), ctypes.byref(n)),
            "ebic_matrix_build_pairs")
     return n.value
+
+
+def ebic_matrix_bytes(rows, cols):
+    """Device bytes of a loaded matrix of this shape, and of its pair table."""
+    a, b = ctypes.c_uint64(), ctypes.c_uint64()
+    _check(_lib_bytes(int(rows), int(cols), ctypes.byref(a), ctypes.byref(b)), "ebic_matrix_bytes")
+    return a.value, b.value
 
 
 def ebic_release_memory(device=-1):

@@ -306,7 +306,7 @@ class GpuBackend:
     def footprint(self, spec: RunSpec):
         R, C = spec.X.shape
         W = (R + 31) // 32
-        rank_bytes = R * C * (1 if C <= 127 else 2) * 1.02 + 4096
+        rank_bytes, _ = self.ebic.ebic_matrix_bytes(R, C)
         pb = self.pair_bytes(spec)
         if 0 < pb <= self.pair_budget:
             rank_bytes += pb
@@ -335,7 +335,8 @@ class GpuBackend:
         # resident archive: its members scored once on this matrix
         if spec.archive_offsets is not None and len(spec.archive_offsets) > 1:
             ac, ao = spec.archive_cols, spec.archive_offsets
-            _, abm = self.ebic.eval_population(m, ac, ao)
+            # (without a pair table: not through one for the call, which no footprint counts)
+            _, abm = self.ebic.eval_population(m, ac, ao, direct=not pairs)
             run["acols"] = torch.from_numpy(np.ascontiguousarray(ac).view(np.int16)).to(self.dev)
             run["aoffs"] = torch.from_numpy(np.ascontiguousarray(ao).view(np.int32)).to(self.dev)
             run["abm"] = torch.from_numpy(abm.view(np.int32)).to(self.dev)
@@ -357,6 +358,9 @@ class GpuBackend:
         run = self.runs.pop(run_id)
         self.torch.cuda.synchronize(self.dev)
         run["m"].close()
+        # the next run's tensors come from another allocator than its matrix: what the library would
+        # keep for the next matrix is free for both
+        self.ebic.ebic_release_memory(self.dev.index)
 
     def launch(self, reqs):
         slot = next(s for s in self.slots if not s["busy"])

@@ -187,3 +187,44 @@ def test_release(lib):
     assert log(lib)[0] == "sync"
     assert set(log(lib)[1:]) == {"trim library 0", "trim tables 0", "trim default 0"}
     assert lib.ebic_release_memory(ctypes.c_int32(7)) == -1
+
+
+SHAPES = [(1, 1), (1000, 20), (4097, 33), (300, 52), (5000, 64), (70001, 127), (513, 128),
+          (9000, 208), (9000, 209), (3000, 457), (100, 666), (65, 832)]
+
+
+@pytest.mark.parametrize("rows,cols", SHAPES)
+def test_admission_counts_what_a_run_allocates(lib, rows, cols):
+    """The server's footprint of a run without an archive is its matrix, its pair table (within the
+    budget) or else its population's bitmaps, and 4 KB; the matrix and table as the library
+    allocates them."""
+    from paper_1807_09932_gb300 import ebic, serve
+    lib.fake_reset()
+    before = lib.fake_live(POOL)
+    rc, h = load(lib, rows, cols)
+    matrix = lib.fake_live(POOL) - before
+    assert rc == OK and lib.ebic_matrix_build_pairs(h, 1 << 60, None, None) == OK
+    table = lib.fake_live(POOL) - before - matrix
+    lib.ebic_free_matrix(h)
+    assert ebic.ebic_matrix_bytes(rows, cols) == (matrix, table)
+    spec = serve.RunSpec(run_id=0, X=np.empty((rows, cols), np.float32), max_cand=10)
+    be = object.__new__(serve.GpuBackend)
+    be.ebic = ebic
+    be.pair_budget = 0
+    assert be.footprint(spec) == matrix + 10 * ((rows + 31) // 32) * 4 + 4096
+    be.pair_budget = table
+    assert be.footprint(spec) == matrix + table + 4096
+
+
+def test_a_closed_run_leaves_its_memory_to_every_allocator():
+    from types import SimpleNamespace as NS
+
+    from paper_1807_09932_gb300 import serve
+    calls = []
+    be = object.__new__(serve.GpuBackend)
+    be.dev = NS(index=0)
+    be.torch = NS(cuda=NS(synchronize=lambda d: calls.append("sync")))
+    be.ebic = NS(ebic_release_memory=lambda d: calls.append(("release", d)))
+    be.runs = {3: {"m": NS(close=lambda: calls.append("close"))}}
+    be.close_run(3)
+    assert calls == ["sync", "close", ("release", 0)]
