@@ -28,9 +28,14 @@ def default_cache_path():
                                        "autotune.json"))
 
 
+# What the evaluator that a cached winner was timed on reads: its name is part of every key, and
+# changes with the stored layout or the kernel, so that another form's winners are not taken over.
+EVALUATOR = "planes1"
+
+
 def shape_key(rank_bits, cols, rows, n_cand, mean_len, negative):
     """The shape class a tuning result is valid for."""
-    return (f"w{rank_bits}-c{cols}-r{int(round(math.log2(max(rows, 1))))}"
+    return (f"{EVALUATOR}-w{rank_bits}-c{cols}-r{int(round(math.log2(max(rows, 1))))}"
             f"-p{int(round(math.log2(max(n_cand, 1))))}-l{int(round(mean_len))}"
             f"-n{int(bool(negative))}")
 
@@ -101,12 +106,13 @@ def allowed_tiles(m):
 
 def gpu_measure(m, dcols, doffs, n_cand, counts, bitmaps, negative=False, iters=5):
     """measure(tile, chunk) over ebic_eval_population on device buffers, timed with CUDA events
-    on the current stream (median of ``iters`` after one warm-up)."""
+    on the current stream (median of ``iters`` after one warm-up). The evaluator itself is timed: a
+    pair table, the matrix's or one for the call, has no tiles."""
     import torch
 
     from . import ebic
     stream = torch.cuda.current_stream()
-    flags = ebic.EBIC_NEGATIVE_TRENDS if negative else 0
+    flags = ebic.EBIC_EVAL_DIRECT | (ebic.EBIC_NEGATIVE_TRENDS if negative else 0)
 
     def measure(tile, chunk):
         m.set_tile(tile)
