@@ -57,6 +57,13 @@ CLOCK_QUERY = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.ac
                "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 
 
+def route_flags(no_pairs):
+    """Flags of the timed scoring calls: without pair tables the rank-code evaluator is asked for (a
+    plain call would build a table for itself where the population is large)."""
+    from paper_1807_09932_gb300 import ebic
+    return ebic.EBIC_EVAL_DIRECT if no_pairs else 0
+
+
 def parse_args():
     p = argparse.ArgumentParser()
     p.add_argument("--gpus", type=int, default=1)
@@ -305,8 +312,8 @@ def main():
         view = {np.dtype(np.uint16): np.int16, np.dtype(np.uint32): np.int32}[a.dtype]
         return torch.from_numpy(np.ascontiguousarray(a).view(view)).to(dev)
 
-    # load: rank transform, timed by the library's own events; then the pair table, built by the
-    # evaluator on the population of all column pairs (once per matrix, like the transform)
+    # load: rank transform, timed by the library's own events; then the pair table (once per
+    # matrix, like the transform; its build is among the events of EBIC_TIMING_EVALUATE)
     Xd = torch.from_numpy(X).to(dev)
     # one transform of a small slice first, so that the timed one does not include the
     # kernel's first-launch module load
@@ -342,11 +349,12 @@ def main():
     flush = torch.empty(FLUSH_BYTES, dtype=torch.uint8, device=dev)
     h = m.handle
     sp = stream.cuda_stream
+    route = route_flags(args.no_pairs)
 
     def step(i):
         dc, do, n = dpops[i % N_POPS]
         if args.unfused:
-            rc = ebic.ebic_eval_population(h, dc, do, n, 0, counts, bitmaps, sp)
+            rc = ebic.ebic_eval_population(h, dc, do, n, route, counts, bitmaps, sp)
             if rc:
                 raise ebic.EbicError(rc, "ebic_eval_population")
             rc = ebic.ebic_fitness(h, dc, do, n, counts, bitmaps, dacols, daoffs, dabm, K, 0,
@@ -354,8 +362,8 @@ def main():
             if rc:
                 raise ebic.EbicError(rc, "ebic_fitness")
             return
-        rc = ebic.ebic_eval_fitness(h, dc, do, n, 0, dacols, daoffs, dabm, K, counts, None, fit,
-                                    None, sp)
+        rc = ebic.ebic_eval_fitness(h, dc, do, n, route, dacols, daoffs, dabm, K, counts, None,
+                                    fit, None, sp)
         if rc:
             raise ebic.EbicError(rc, "ebic_eval_fitness")
 
@@ -432,7 +440,7 @@ def main():
         def e2e_step(i):
             hc, ho, n = hpops[i % N_POPS]
             if args.unfused:
-                rc = ebic.ebic_eval_population(h, hc, ho, n, 0, counts, bitmaps, sp)
+                rc = ebic.ebic_eval_population(h, hc, ho, n, route, counts, bitmaps, sp)
                 if rc:
                     raise ebic.EbicError(rc, "ebic_eval_population")
                 rc = ebic.ebic_fitness(h, hc, ho, n, counts, bitmaps, dacols, daoffs, dabm, K,
@@ -440,8 +448,8 @@ def main():
                 if rc:
                     raise ebic.EbicError(rc, "ebic_fitness")
                 return
-            rc = ebic.ebic_eval_fitness(h, hc, ho, n, 0, dacols, daoffs, dabm, K, counts, None,
-                                        hfit, None, sp)   # host output: synchronizes
+            rc = ebic.ebic_eval_fitness(h, hc, ho, n, route, dacols, daoffs, dabm, K, counts,
+                                        None, hfit, None, sp)   # host output: synchronizes
             if rc:
                 raise ebic.EbicError(rc, "ebic_eval_fitness")
 
@@ -540,6 +548,7 @@ def main():
             "config": {"workload": WORKLOAD, "rows": R, "cols": C, "population": P,
                        "archive": K, "populations_cycled": N_POPS,
                        "step": ("ebic_eval_population + ebic_fitness" if args.unfused
+                                else "ebic_eval_fitness" if args.no_pairs
                                 else "ebic_eval_fitness (evaluation and archive overlaps fused)"),
                        "l2": "flushed between timed steps (512 MB write, outside the events)",
                        "parallelism": "replicas" if ws > 1 else "single GPU",
@@ -942,9 +951,9 @@ def batched_measure(args, steps):
     evals_per_step = float(sum(p["n"] * p["R"] for p in pops))
     flush = torch.empty(FLUSH_BYTES, dtype=torch.uint8, device=dev)
 
-    def plain_step():
+    def plain_step(flags=route_flags(args.no_pairs)):
         for p in pops:
-            rc = ebic.ebic_eval_population(p["m"].handle, p["dc"], p["do"], p["n"], 0, p["cnt"],
+            rc = ebic.ebic_eval_population(p["m"].handle, p["dc"], p["do"], p["n"], flags, p["cnt"],
                                            p["bm"], stream.cuda_stream)
             if rc:
                 raise ebic.EbicError(rc, "ebic_eval_population")
@@ -991,8 +1000,11 @@ def batched_measure(args, steps):
         for m in mats:
             m.drop_pairs()
         ms_rank = timed(batched_step, steps)
-        ms_rank_plain = timed(plain_step, steps)
+        ms_rank_plain = timed(lambda: plain_step(ebic.EBIC_EVAL_DIRECT), steps)
+        # (plain calls left to the library build a table for the call where it pays)
+        ms_call_table = timed(lambda: plain_step(0), steps)
         rank_code = {"batched_ms_per_step": ms_rank, "plain_ms_per_step": ms_rank_plain,
+                     "plain_call_tables_ms_per_step": ms_call_table,
                      "batched_value": evals_per_step / (ms_rank / 1000)}
     ebic.ebic_batch_free(batch)
     line = {"metric": "candidate-row evals/s", "value": evals_per_step / (ms_batched / 1000),

@@ -519,7 +519,8 @@ int64_t ebic_launch_count(void);
  * library's own kernel launches. Kinds: */
 #define EBIC_TIMING_RANK_TRANSFORM 0
 #define EBIC_TIMING_PREPARE        1  /* device-side argument checks and output zeroing */
-#define EBIC_TIMING_EVALUATE       2  /* the population evaluator */
+#define EBIC_TIMING_EVALUATE       2  /* the population evaluator; also each build of a pair table,
+                                         * the matrix's or one for a call */
 #define EBIC_TIMING_OVERLAP        3  /* bitmap overlaps against the archive */
 #define EBIC_TIMING_FITNESS        4  /* penalised fitness */
 #define EBIC_TIMING_PAIR_EVALUATE  5  /* the pair-table evaluator */
