@@ -524,14 +524,14 @@ def main():
         kernels["pair_evaluate"] = roofline_pairs(pops, R, m, pev_ms / pev_n, clk, peaks,
                                                   not args.unfused, K)
     if eval_n:
-        kernels["evaluate"] = roofline_eval(pops, R, m, eval_launch_ms, sms, clk, peaks)
+        kernels["evaluate"] = roofline_eval(X, pops, R, m, eval_launch_ms, sms, clk, peaks)
     # the step's kernel with the largest share is the dominant one; the rank-code route's
     # kernels (timed beside the step, not in it) are reported among the others
     dominant = max(kernels, key=lambda k: kernels[k]["launch_ms"])
     if rc_ms is not None:
         if rc_eval_n:
             kernels["evaluate (rank-code route)"] = roofline_eval(
-                pops, R, m, rc_eval_ms / rc_eval_n, sms, clk, peaks)
+                X, pops, R, m, rc_eval_ms / rc_eval_n, sms, clk, peaks)
         if rc_ov_n:
             kernels["overlap (rank-code route)"] = roofline_overlap(pops, K, m, rc_ov_ms / rc_ov_n,
                                                                     sms, clk, peaks)
@@ -807,26 +807,57 @@ def roofline_overlap(pops, K, m, launch_ms, sms, clk, peaks):
                                  "ratio_to_alu_peak": alu_ops / t / (64 * sms * clock_hz)}}
 
 
-def roofline_eval(pops, R, m, launch_ms, sms, clk, peaks):
+def walked_columns(X, pops, segment=1024, segments=64, cands=200):
+    """Columns of a candidate that the evaluator's walk reads, on average over candidates and
+    `segment`-row segments (the rows of a warp's 32 bitmap words): the walk takes columns two at a
+    time and ends when no row of the segment follows any more. From a sample of the segments and of
+    each population's candidates, increasing trends, missing values excluded."""
+    R = X.shape[0]
+    n = max(1, R // segment)
+    picks = np.unique(np.linspace(0, n - 1, min(segments, n)).astype(int))
+    S = np.stack([X[k * segment:min(R, (k + 1) * segment)] for k in picks])  # [segment][row][col]
+    walked = []
+    for cols, offs in pops:
+        some = np.unique(np.linspace(0, len(offs) - 2, min(cands, len(offs) - 1)).astype(int))
+        for i in some:
+            c = cols[offs[i]:offs[i + 1]].astype(int)
+            rows = ~np.isnan(S[:, :, c[0]])
+            read = np.ones(len(picks))
+            for k in range(1, len(c), 2):
+                going = rows.any(axis=1)
+                if not going.any():
+                    break
+                read[going] = min(k + 2, len(c))
+                for j in range(k, min(k + 2, len(c))):
+                    rows &= S[:, :, c[j]] >= S[:, :, c[j - 1]]
+            walked.append(read.mean())
+    return float(np.mean(walked))
+
+
+def roofline_eval(X, pops, R, m, launch_ms, sms, clk, peaks):
     """The evaluator against the roof that binds it.
 
-    Algorithmic work per launch (one population): every candidate column is read for every row,
-    sum_c L_c * R codes of NB bits each (NB = the bits of the column count), out of shared memory
-    (the row tile is staged there by bulk copies); and each is one three-input logic operation
-    per bit and 32 rows. The walk ends where no row follows any more, so long candidates read
-    less than that and the fraction can pass 1 for them. Peaks from the recipe's unit counts and
+    Work per launch (one population): the columns that the walk reads before it ends
+    (walked_columns) for every candidate and row, NB bits a code (NB = the bits of the column
+    count), out of shared memory (the row tile is staged there by bulk copies); and each is one
+    three-input logic operation per bit and 32 rows. The same with every column counted, also
+    those that the early end leaves out, is reported as "all_columns"; that is no fraction of a
+    roof. Peaks from the recipe's unit counts and
     the median SM clock sampled during the timed region: shared memory 128 B/clk/SM, ALU 64
     lanes/clk/SM. Shared memory is the binding roof ("bound"); the ALU and HBM roofs are
     reported beside it. HBM: rank matrix + bitmaps against the measured copy bandwidth
     (MEASURED_PEAKS.json).
     """
     sum_l = float(np.mean([int(o[-1]) for _, o in pops]))
+    n_cand = float(np.mean([len(o) - 1 for _, o in pops]))
+    walked = walked_columns(X, pops[:2])
     planes = int(m.cols).bit_length()
     clock_hz = (clk.get("sm_mhz") or peaks.get("sm_max_mhz") or 2070.0) * 1e6
     t = launch_ms / 1000.0
-    smem_bytes = sum_l * R * planes / 8
+    all_bytes = sum_l * R * planes / 8
+    smem_bytes = n_cand * walked * R * planes / 8
     smem_peak = 128 * sms * clock_hz
-    lane_ops = sum_l * R / 32 * planes
+    lane_ops = n_cand * walked * R / 32 * planes
     alu_peak = 64 * sms * clock_hz
     hbm_bytes = m.cols * R * planes / 8 + 1600 * m.words * 4
     return {"bound": "smem", "achieved": smem_bytes / t / 1e9, "peak": smem_peak / 1e9,
@@ -837,6 +868,8 @@ def roofline_eval(pops, R, m, launch_ms, sms, clk, peaks):
                             "changed since that capture",
             "kernel": "eval_population_kernel", "launch_ms": launch_ms,
             "algorithmic_bytes_per_launch": smem_bytes,
+            "columns_walked": walked, "columns": sum_l / n_cand,
+            "all_columns": {"bytes": all_bytes, "ratio_to_smem_peak": all_bytes / t / smem_peak},
             "peak_basis": "shared memory 128 B/clk/SM x SMs x median SM clock in the timed region",
             "alu": {"achieved_gops": lane_ops / t / 1e9, "peak_gops": alu_peak / 1e9,
                     "frac": (lane_ops / t) / alu_peak,
