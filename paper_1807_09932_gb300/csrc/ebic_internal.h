@@ -39,16 +39,14 @@ __host__ __device__ inline bool offsets_sane(uint32_t lo, uint32_t hi, uint32_t 
   return !(first && lo != 0u) && hi > lo && hi - lo <= (uint32_t)kMaxLen && hi <= total;
 }
 
-// The candidate of a CSR list (offsets[0 .. n]) that holds entry t of its columns, or n where no
-// candidate with sane offsets does: such an entry may lie past the columns and is not to be read.
+// The candidate of a CSR list in order (offsets[0 .. n]) that holds entry t of its columns.
 __host__ __device__ inline uint32_t entry_member(const uint32_t* offsets, uint32_t n, uint32_t t) {
   uint32_t m = 0, end = n;  // the last candidate whose columns start at or before t
   while (end - m > 1) {
     const uint32_t mid = (m + end) / 2;
     if (offsets[mid] <= t) m = mid; else end = mid;
   }
-  const uint32_t lo = offsets[m], hi = offsets[m + 1];
-  return t >= lo && t < hi && offsets_sane(lo, hi, offsets[n], m == 0) ? m : n;
+  return m;
 }
 
 // error bits written by kernels into the per-call error word and the matrix status word

@@ -203,7 +203,16 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
   const int slots = term_slots(a.negative);
 
   // (A)
-  if (threadIdx.x <= na && na) sh.aoff[threadIdx.x] = a.aoffsets[threadIdx.x];
+  // (na <= 64, fewer than the block's threads: a thread per member checks its offsets)
+  uint32_t a_lo = 0, a_hi = 0, a_tot = 0;
+  if (threadIdx.x <= na && na) {
+    a_lo = a.aoffsets[threadIdx.x];
+    if (a.check_arch && threadIdx.x < na) {
+      a_hi = a.aoffsets[threadIdx.x + 1];
+      a_tot = a.aoffsets[na];
+    }
+    sh.aoff[threadIdx.x] = a_lo;
+  }
   for (int i = threadIdx.x; i < (int)na * kSetWords; i += blockDim.x) (&sh.msets[0][0])[i] = 0u;
   for (int w = lane; w < nw; w += 32) set[w] = 0u;
   uint32_t lo0 = 0, hi0 = 0, tot0 = 0;
@@ -218,42 +227,37 @@ __device__ bool fused_prepare_body(const FusedPrepareArgs& a, PrepShared<WARPS>&
   }
   copy_archive_padded(a.arch_src, a.arch_pad, na, a.W, a.stride, tid, nthreads);
   for (size_t i = tid; i < na; i += nthreads) a.arch_counts[i] = 0u;
-  __syncthreads();
+  bool abad = a.check_arch && threadIdx.x < na &&
+              !offsets_sane(a_lo, a_hi, a_tot, threadIdx.x == 0);
+  const bool aoffs_bad = __syncthreads_or(abad) != 0;
 
   // (B) the first candidate's columns are requested first, then every block builds the
   // members' column sets, one list entry per thread (loads coalesced, the member found in the
-  // shared offsets; a thread per possible position took four rounds of loads for 64 members). Of
-  // a list whose offsets fail, only entries of members whose own offsets hold are read: the list's
-  // total may be one of the wrong ones, and its columns end before it. The sets are then
-  // arbitrary (the list is rejected, and the pass that follows does nothing)
+  // shared offsets; a thread per possible position took four rounds of loads for 64 members). A
+  // device list's offsets have been checked: of a list whose offsets fail, no entry is read (the
+  // total may be what is wrong, and the columns may end before it), the sets stay empty, the list
+  // is rejected, and the pass that follows does nothing
   const bool first_sane = gw < a.n_cand && offsets_sane(lo0, hi0, tot0, gw == 0);
   uint32_t c_lo = 0, c_hi = 0;
   if (first_sane) load_cols_regs(a.cols, lo0, hi0, lane, c_lo, c_hi);
-  const uint32_t atotal = na ? sh.aoff[na] : 0u;
-  // the archive list is checked on the way (when the caller keeps it on the device): offsets, a
-  // column out of range, a column repeated within a member (seen by the atomic OR)
-  bool abad = false;
-  if (a.check_arch)
-    for (uint32_t m = threadIdx.x; m < na; m += blockDim.x) {
-      const uint32_t lo = sh.aoff[m], hi = sh.aoff[m + 1];
-      abad |= !offsets_sane(lo, hi, atotal, m == 0);
-    }
-  // (a list whose total exceeds 64 columns a member is rejected above; none of it is read)
-  const uint32_t n_entries = atotal <= na * (uint32_t)kMaxLen ? atotal : 0u;
+  // a list that the caller keeps on the device is checked on the way: a column out of range, a column
+  // repeated within a member (seen by the atomic OR)
+  const uint32_t n_entries = na && !aoffs_bad ? sh.aoff[na] : 0u;
   for (uint32_t t0 = threadIdx.x; t0 < n_entries; t0 += 4 * blockDim.x) {
-    uint32_t c[4], m[4];
+    uint32_t c[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t t = t0 + k * blockDim.x;
-      m[k] = t < n_entries ? entry_member(sh.aoff, na, t) : na;
-      c[k] = m[k] < na ? a.acols[t] : 0u;
+      c[k] = t < n_entries ? a.acols[t] : 0u;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (m[k] >= na) continue;
+      const uint32_t t = t0 + k * blockDim.x;
+      if (t >= n_entries) continue;
+      const uint32_t m = entry_member(sh.aoff, na, t);
       if (c[k] < (uint32_t)a.ncols) {
         const uint32_t bit = 1u << (c[k] & 31u);
-        const bool seen = (atomicOr(&sh.msets[m[k]][c[k] >> 5], bit) & bit) != 0u;
+        const bool seen = (atomicOr(&sh.msets[m][c[k] >> 5], bit) & bit) != 0u;
         abad |= a.check_arch && seen;
       } else {
         abad |= a.check_arch;

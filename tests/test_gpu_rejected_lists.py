@@ -42,3 +42,34 @@ def test_list_without_columns(n, noalloc):
                 run(dc, do, 50, got)
                 assert m.status() == ebic.EBIC_OK
                 assert np.array_equal(got.cpu().numpy().view(np.uint32), want)
+
+
+def test_archive_list_whose_total_is_past_its_columns():
+    """The last offset of a device archive list is wrong: the list is rejected (its columns are not
+    read up to that total), nothing is written, and the next call is right."""
+    import torch
+    torch.cuda.init()
+    from paper_1807_09932_gb300 import ebic
+    X = np.random.default_rng(5).standard_normal((900, 20)).astype(np.float32)
+    c, o = synth.make_population(3, 50, 20, 2, 6)
+    ac, ao = synth.make_population(4, 20, 20, 2, 6)
+    cnt, bm = oracle.eval_population(X, c, o)
+    _, abm = oracle.eval_population(X, ac, ao)
+    fit, _ = oracle.fitness(900, c, o, cnt, bm, ac, ao, abm)
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a).view(t)).cuda()  # noqa: E731
+    with ebic.Matrix(X) as m:
+        m.build_pairs()
+        for total in (int(ao[-1]) + 100, 20 * 64, 2**31):
+            bad = ao.astype(np.uint32).copy()
+            bad[-1] = total
+            for offs, status in ((bad, ebic.EBIC_ERR_INVALID_ARG), (ao, ebic.EBIC_OK)):
+                f = torch.full((50,), 5, dtype=torch.int64, device="cuda")
+                n = torch.zeros(50, dtype=torch.int32, device="cuda")
+                rc = ebic.ebic_eval_fitness(m.handle, dev(c, np.int16), dev(o, np.int32), 50, 0,
+                                            dev(ac, np.int16), dev(offs, np.int32),
+                                            dev(abm, np.int32), 20, n, None, f, None)
+                assert rc == ebic.EBIC_OK and m.status() == status
+                if status == ebic.EBIC_OK:
+                    assert np.array_equal(f.cpu().numpy().view(np.uint64), fit)
+                else:
+                    assert bool((f == 5).all())
