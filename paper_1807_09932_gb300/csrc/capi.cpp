@@ -412,14 +412,14 @@ const char* check_candidates_host_c(const uint16_t* cols, const uint32_t* offset
 }  // namespace ebic
 
 // Words per row (a multiple of the table's) of the pair table that a call on a matrix without one
-// builds for itself in scratch, or 0 where the evaluator is the faster way. A table costs C * C
-// comparisons of every row; through it a candidate costs a quarter of what it costs the
-// evaluator. So it pays from C * C / 3 candidates on, and only where the evaluator takes some 40
-// us (candidates times words), since it adds launches. Counts and bitmaps, evaluator against
-// table: 436,444 x 64, 1,600 candidates of 2-16 columns 191 against 130 us, of 2-6 columns 162
-// against 124, 6,400 candidates 827 against 222; 100,000 x 64, 1,600 candidates 54 against 44, 400
-// (C * C / 10) 23 against 37; 436,444 x 32, 400 candidates 51 against 42; 30,000 x 50, 1,600 24
-// against 26. The table is at most kCallTable bytes; more rows are taken in ranges.
+// builds for itself, or 0 where the evaluator is the faster way. A table costs C * C comparisons of
+// every row; through it a candidate costs a fifth of what it costs the evaluator. So it pays from
+// some C * C / 3 candidates on (of 2-16 columns; of 2-6 from C * C / 2), and only where the evaluator
+// takes some 35 us (candidates times words), since it adds launches. Counts and bitmaps, calls queued
+// one behind the other, evaluator against table: 436,444 x 64, 1,600 candidates of 2-16 columns 145
+// against 128 us, of 2-6 columns 107 against 120, 1,400 of 2-16 126 against 125, 6,400 612 against
+// 223; 100,000 x 64, 1,400 39 against 41; 80,000 x 50, 1,700 35 against 33; 436,444 x 32, 400 40
+// against 41. The table is at most kCallTable bytes; more rows are taken in ranges.
 constexpr int64_t kCallTable = 256ll << 20;
 static int64_t call_table_words(const Layout& L, uint32_t n_cand) {
   const int64_t cc = (int64_t)L.cols * L.cols;

@@ -30,12 +30,13 @@
 // counter, and move on to the next item without waiting for each other: the last warp to leave
 // a stage has it refilled.
 //
-// What bounds it: shared-memory reads (128 bytes per clock and SM), 4 NB / 32 bytes per row and
-// column walked. One warp covers one candidate over 32 words where a tile has them; matrices of
-// more than 208 columns, whose slabs are 8, 4 or 2 words high, put 4 to 16 candidates into a
-// warp, whose reads then meet in banks by chance (2 to 3 wavefronts instead of one).
+// What bounds it: instruction issue and shared-memory reads (128 bytes per clock and SM), 4 NB / 32
+// bytes per row and column walked. One warp covers one candidate over 32 or 64 words where a tile has
+// them (eval_wide_tile; up to 104 columns by default); other matrices put several candidates into a
+// warp, those of more than 208 columns, whose slabs are 8, 4 or 2 words high, 4 to 16, whose reads
+// then meet in banks by chance (2 to 3 wavefronts instead of one).
 // Measured, counts and bitmaps of 1,600 candidates, against packed byte and half compares of
-// every column (the form before): 436,444 x 64, 2-16 columns 251 -> 184 us; 20,000 x 200, 2-20
+// every column (the form before): 436,444 x 64, 2-16 columns 251 -> 140 us; 20,000 x 200, 2-20
 // columns, both trends 66 -> 26 us; 50,021 x 457, 2-64 columns 487 -> 76 us.
 #pragma once
 
@@ -89,9 +90,63 @@ struct Walk {
     return o;
   }
 
+  // The bitmap words of one candidate, the whole warp's, for the lane's WPL words of the tile (word i
+  // at base + i * apart; in[i]: it is a row's). Columns two at a time and a last one by itself.
+  template <bool NEG, int WPL>
+  __device__ __forceinline__ void chain_one(const uint8_t* base, uint32_t apart,
+                                            const bool (&in)[WPL], const uint16_t* ccols, int L,
+                                            uint32_t (&out)[WPL]) const {
+    uint32_t a[WPL][kPlanes], b[WPL][kPlanes], acc[WPL], dec[WPL];
+    uint32_t n0 = ccols[0];
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) load(base + i * apart, n0, a[i]);
+    // (the list is read ahead of the columns: past a candidate's end lies the next one or the
+    // chunk's slack, and what is read there is never used)
+    n0 = ccols[1];
+    uint32_t n1 = ccols[2];
+    uint32_t any = 0u;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+      acc[i] = in[i] ? present(a[i]) : 0u;
+      dec[i] = NEG && in[i] ? ~0u : 0u;
+      any |= acc[i] | dec[i];
+    }
+    int k = 1;
+    while (k + 1 < L && __any_sync(0xFFFFFFFFu, any != 0u)) {
+      const uint32_t c0 = n0, c1 = n1;
+      n0 = ccols[k + 2];
+      n1 = ccols[k + 3];
+      any = 0u;
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) {
+        load(base + i * apart, c0, b[i]);
+        const uint32_t up = ge(b[i], a[i]), dn = NEG ? ge(a[i], b[i]) : 0u;
+        load(base + i * apart, c1, a[i]);
+        acc[i] &= up & ge(a[i], b[i]);
+        if (NEG) dec[i] &= dn & ge(b[i], a[i]);
+        any |= acc[i] | (NEG ? dec[i] : 0u);
+      }
+      k += 2;
+    }
+    if (k + 1 == L) {  // (after an early end k + 1 < L: nothing follows any more)
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) {
+        load(base + i * apart, n0, b[i]);
+        acc[i] &= ge(b[i], a[i]);
+        if (NEG) dec[i] &= ge(a[i], b[i]);
+        if (NEG) dec[i] &= present(b[i]);
+      }
+    } else if (NEG) {
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) dec[i] &= present(a[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) out[i] = NEG ? acc[i] | dec[i] : acc[i];
+  }
+
   // The candidate's bitmap word for the lane's word of the tile (`base`: that word of column 0's
-  // plane 0); 0 for a lane without a candidate (L 0, list not read past its first entry). A warp's
-  // lanes may walk several candidates at once: a lane past its own end compares its last column
+  // plane 0); 0 for a lane without a candidate (L 0, list not read past its first entry). The
+  // warp's lanes walk several candidates at once: a lane past its own end compares its last column
   // with itself, and the walk goes on while a lane has rows left and columns to go.
   template <bool NEG>
   __device__ __forceinline__ uint32_t chain(const uint8_t* base, const uint16_t* ccols,
@@ -121,6 +176,39 @@ __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* a, uint32_t 
     if ((uint64_t)a[mid] < v) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+
+// eval_tile where the warp has one candidate at a time: slabs of 16 words in tiles of 32 words (WPL 1)
+// or 64 (WPL 2: each lane has two words, so that the walk's steps and votes serve 2,048 rows). An odd
+// last column is compared by itself, and the list is read without bounds. Counts of 3,000
+// candidates of 2-10 columns, calls queued one behind the other, through eval_tile's walk and through
+// this one: 100,000 x 20 113 and 74 us, 400,000 x 52 433 and 297, 400,000 x 100 407 and 292 (the packed
+// byte compares at their best 91, 344 and 327); 436,444 x 64, 1,600 of 2-16 columns with bitmaps 189
+// and 144.
+template <int NB, int WPL, bool NEG, class Take>
+__device__ __forceinline__ void eval_wide_tile(const TileShape& sh, const uint8_t* stage,
+                                               const uint16_t* ccols, const uint16_t* coffs,
+                                               uint32_t lo, uint32_t c1, int64_t first_word,
+                                               int64_t n_words, uint32_t* counts,
+                                               uint32_t* bitmaps, int lane, Take take) {
+  const Walk<NB, 16> walk{sh};
+  const uint8_t* base = stage + (uint32_t)(lane >> 4) * sh.pitch + (uint32_t)(lane & 15) * 4u;
+  bool in[WPL];  // (past the last word the stage may hold another tile's slabs)
+#pragma unroll
+  for (int i = 0; i < WPL; ++i) in[i] = first_word + lane + 32 * i < n_words;
+  for (uint32_t c = take(); c < c1; c = take()) {
+    const int o = coffs[c], L = coffs[c + 1] - o;
+    uint32_t x[WPL], cnt = 0;
+    walk.template chain_one<NEG, WPL>(base, 2u * sh.pitch, in, ccols + o, L, x);
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+      cnt += __popc(x[i]);
+      if (bitmaps && in[i])
+        bitmaps[(size_t)(lo + c) * (size_t)n_words + first_word + lane + 32 * i] = x[i];
+    }
+    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    if (lane == 0 && cnt) atomicAdd(&counts[lo + c], cnt);
+  }
 }
 
 // Candidates [c0, c1) of a staged chunk on one staged tile, those that `take()` hands the warp
@@ -171,7 +259,8 @@ constexpr int kEvalWarps = kEvalThreads / 32;
 constexpr uint32_t kItemUnits = 1024;  // work units per item
 
 // Shared-memory plan (dynamic): [stage 0][stage 1][chunk columns][chunk offsets]
-template <int NB, int T, bool NEG>
+// WPL 0: tiles whose warps walk several candidates at once (eval_tile).
+template <int NB, int T, int WPL, bool NEG>
 __global__ void __launch_bounds__(kEvalThreads, 1) eval_population_kernel(const EvalArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t full_bar[2];
@@ -273,13 +362,18 @@ __global__ void __launch_bounds__(kEvalThreads, 1) eval_population_kernel(const 
       const uint32_t s1 = it + 1 == i1 ? (uint32_t)(u1 - it * kItemUnits) : kItemUnits;
       const uint32_t c0 = (uint32_t)((uint64_t)nc * s0 / kItemUnits);
       const uint32_t c1 = (uint32_t)((uint64_t)nc * s1 / kItemUnits);
-      eval_tile<NB, T, NEG>(sh, s ? stage1 : stage0, ccols, coffs, lo, c1,
-                            tile * a.ts * sh.words, a.words, a.counts, a.bitmaps, lane,
-                            [&]() {
-                              uint32_t u = 0;
-                              if (lane == 0) u = atomicAdd(&next_s[s], group);
-                              return c0 + __shfl_sync(0xFFFFFFFFu, u, 0);
-                            });
+      auto take = [&]() {
+        uint32_t u = 0;
+        if (lane == 0) u = atomicAdd(&next_s[s], group);
+        return c0 + __shfl_sync(0xFFFFFFFFu, u, 0);
+      };
+      const int64_t first_word = tile * a.ts * sh.words;
+      if constexpr (WPL > 0)
+        eval_wide_tile<NB, WPL, NEG>(sh, s ? stage1 : stage0, ccols, coffs, lo, c1, first_word,
+                                     a.words, a.counts, a.bitmaps, lane, take);
+      else
+        eval_tile<NB, T, NEG>(sh, s ? stage1 : stage0, ccols, coffs, lo, c1, first_word, a.words,
+                              a.counts, a.bitmaps, lane, take);
     }
     // the last warp to leave the stage has it refilled (its release of the counter orders every
     // warp's reads of the stage before the copy)
