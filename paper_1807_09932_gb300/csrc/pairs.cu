@@ -307,8 +307,11 @@ cudaError_t launch_variant(const PairArgs& p, int grid, bool pdl, cudaStream_t s
   if (p.arch)
     return launch_maybe_pdl(pdl, pair_eval_kernel<NEG, BITMAPS, true, WARPS>, dim3(grid),
                             dim3(WARPS * 32), 0, s, p);
-  return launch_maybe_pdl(pdl, pair_eval_kernel<NEG, BITMAPS, false, WARPS>, dim3(grid),
-                          dim3(WARPS * 32), 0, s, p);
+  if constexpr (BITMAPS && WARPS != kPairWarps)
+    return cudaErrorInvalidValue;  // (launch_pair_eval takes kPairWarps)
+  else
+    return launch_maybe_pdl(pdl, pair_eval_kernel<NEG, BITMAPS, false, WARPS>, dim3(grid),
+                            dim3(WARPS * 32), 0, s, p);
 }
 
 }  // namespace
@@ -321,14 +324,28 @@ cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pd
   if ((uint64_t)p.C * (uint64_t)p.C * p.stride > 0xFFFFFFFFull) return cudaErrorInvalidValue;
   if (p.arch && (p.ov_stride % 2 != 0 || p.ov_stride < p.n_arch)) return cudaErrorInvalidValue;
   count_launch();
-  // 28 warps where 72 registers suffice (increasing trends: 4 % off 65,535 candidates, 1 % off
-  // 1,600 on 436,444 x 64 against 24; 20 and 32 warps were slower); both trends need 80
   const bool bm = p.bitmaps != nullptr;
+  // 28 warps where 72 registers suffice (increasing trends: 4 % off 65,535 candidates, 1 % off
+  // 1,600 on 436,444 x 64 against 24; 20 and 32 warps were slower; both trends need 80), and where
+  // the fullest SM then has fewer items to go through. With as many items, or none to spare, the
+  // items of 28 candidates only take longer: calls with 24 and 28 warps, 20,000 rows, 1,600 candidates
+  // 13.0 and 13.7 us, 30,000 rows 13.1 and 13.9, 12,000 rows, 6,000 candidates 17.2 and 18.3. Without an
+  // archive the writing of bitmaps takes longer with 28: 436,444 x 64, 1,600 of 2-6 columns 46.0 and
+  // 47.9.
+  auto rounds = [&](uint32_t warps) {
+    const uint64_t items = (uint64_t)((p.W + kItemWords - 1) / kItemWords) *
+                           ((p.n_cand + (uint64_t)warps - 1) / warps);
+    return (items + grid - 1) / grid;
+  };
+  const bool wide = !negative && (p.arch || !bm) && rounds(28) < rounds(kPairWarps);
   if (negative)
     return bm ? launch_variant<true, true, kPairWarps>(p, grid, pdl, s)
               : launch_variant<true, false, kPairWarps>(p, grid, pdl, s);
-  return bm ? launch_variant<false, true, 28>(p, grid, pdl, s)
-            : launch_variant<false, false, 28>(p, grid, pdl, s);
+  if (wide)
+    return bm ? launch_variant<false, true, 28>(p, grid, pdl, s)
+              : launch_variant<false, false, 28>(p, grid, pdl, s);
+  return bm ? launch_variant<false, true, kPairWarps>(p, grid, pdl, s)
+            : launch_variant<false, false, kPairWarps>(p, grid, pdl, s);
 }
 
 // Where the pass's items of four parts are mostly empty and its finalize launch costs more than the
