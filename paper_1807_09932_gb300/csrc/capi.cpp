@@ -1099,7 +1099,7 @@ static int eval_fitness_impl(const ebic_matrix* cm, const uint16_t* cols, const 
   p.err_out = err;  // the OR of the flags, for the finalize and the host
   p.status = m->status;
   // (a shard's archive counts come from the pass)
-  if (!arch_counts_out && pair_score_fits(L.words, n_cand, neg)) {
+  if (!arch_counts_out && pair_score_fits(L.words, n_cand, neg, n_arch, !p.score && n_arch > 0, L.cols)) {
     Timed t(EBIC_TIMING_PAIR_EVALUATE, s);
     ScoreArgs f;
     f.offsets = doffs;

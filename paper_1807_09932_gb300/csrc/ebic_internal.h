@@ -221,8 +221,10 @@ struct ScoreArgs {
   uint32_t* counts_mirror = nullptr;       // pinned host copy of the counts, or null
   uint32_t* err_mirror = nullptr;          // pinned host copy of the error word, or null
 };
-// Whether launch_pair_score is the faster one for n_cand candidates of W-word bitmaps.
-bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative);
+// Whether launch_pair_score is the faster one for n_cand candidates of W-word bitmaps over `cols`
+// columns against n_arch members, whose overlaps are all wanted or only where a column is shared.
+bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative, uint32_t n_arch, bool all,
+                     int32_t cols);
 cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,
                               cudaStream_t s);
 

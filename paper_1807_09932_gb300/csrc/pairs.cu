@@ -92,7 +92,57 @@ __global__ void __launch_bounds__(WARPS * 32, 1) pair_eval_kernel(const PairArgs
 constexpr int kScoreMembers = 4;   // archive members whose words are in flight together
 constexpr int kScoreCands = 8;     // most candidates per block
 
-template <bool NEG>
+// The overlaps of the warp's words x (words 4 * lane .. of a part) with the wanted archive members, and
+// the members' own rows in these words, added to over[] and rows[] (shared). arch: member 0's words
+// of the part. SEG lanes per member: bitmaps of at most 32 words fill 8 lanes, and the warp then takes
+// 4 members side by side (all overlaps with 64 members, 16,000 candidates on
+// 1,000 rows: 63 us, one member at a time 109, the pass and its finalize 71).
+template <int SEG>
+__device__ __forceinline__ void member_overlaps(uint4 x, const uint32_t* arch, uint64_t stride,
+                                                uint64_t members, uint32_t* over, uint32_t* rows,
+                                                int lane) {
+  constexpr int kSide = 32 / SEG;
+  const int li = lane % SEG, side = lane / SEG;
+  if constexpr (SEG < 32) {
+    x.x = __shfl_sync(0xFFFFFFFFu, x.x, li);
+    x.y = __shfl_sync(0xFFFFFFFFu, x.y, li);
+    x.z = __shfl_sync(0xFFFFFFFFu, x.z, li);
+    x.w = __shfl_sync(0xFFFFFFFFu, x.w, li);
+  }
+  arch += 4 * li;
+  for (uint64_t left = members; left;) {  // warp-uniform
+    int m[kScoreMembers];
+    uint4 v[kScoreMembers];
+#pragma unroll
+    for (int k = 0; k < kScoreMembers; ++k) {
+      m[k] = -1;
+#pragma unroll
+      for (int s = 0; s < kSide; ++s) {
+        if (left && s == side) m[k] = __ffsll((long long)left) - 1;
+        left &= left - 1ull;
+      }
+      v[k] = m[k] >= 0 ? __ldg(reinterpret_cast<const uint4*>(arch + (uint64_t)m[k] * stride))
+                       : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int k = 0; k < kScoreMembers; ++k) {
+      // both sums are at most 4,096
+      uint32_t r = popc4(and4(x, v[k])) | (popc4(v[k]) << 16);
+      if constexpr (SEG == 32) {
+        r = __reduce_add_sync(0xFFFFFFFFu, r);
+      } else {
+#pragma unroll
+        for (int d = SEG / 2; d > 0; d >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, d);
+      }
+      if (li == 0 && r) {
+        atomicAdd(&over[m[k]], r & 0xFFFFu);
+        atomicAdd(&rows[m[k]], r >> 16);
+      }
+    }
+  }
+}
+
+template <bool NEG, int SEG>
 __global__ void __launch_bounds__(kScoreWarps * 32)
     pair_score_kernel(const PairArgs p, const ScoreArgs f, int parts) {
   __shared__ uint32_t count_s[kScoreCands];
@@ -146,28 +196,8 @@ __global__ void __launch_bounds__(kScoreWarps * 32)
   __syncthreads();
   const uint32_t n = count_s[team];
   if (n) {
-    const uint32_t* arch = p.arch + word;
-    for (uint64_t left = members; left;) {  // warp-uniform
-      int m[kScoreMembers];
-      uint4 v[kScoreMembers];
-#pragma unroll
-      for (int k = 0; k < kScoreMembers; ++k) {
-        m[k] = left ? __ffsll((long long)left) - 1 : -1;
-        left &= left - 1ull;
-        v[k] = m[k] >= 0 ? __ldg(reinterpret_cast<const uint4*>(arch + (uint64_t)m[k] * p.stride))
-                         : make_uint4(0u, 0u, 0u, 0u);
-      }
-#pragma unroll
-      for (int k = 0; k < kScoreMembers; ++k) {
-        // both sums are at most 4,096
-        const uint32_t r = __reduce_add_sync(
-            0xFFFFFFFFu, popc4(and4(x[0], v[k])) | (popc4(v[k]) << 16));
-        if (lane == 0 && r) {
-          atomicAdd(&over_s[team][m[k]], r & 0xFFFFu);
-          atomicAdd(&rows_s[team][m[k]], r >> 16);
-        }
-      }
-    }
+    const uint32_t* arch = p.arch + part * kRangeWords;
+    member_overlaps<SEG>(x[0], arch, p.stride, members, over_s[team], rows_s[team], lane);
   }
   __syncthreads();
   if (part != 0 || !live) return;
@@ -350,20 +380,30 @@ cudaError_t launch_pair_eval(const PairArgs& p, bool negative, int grid, bool pd
 
 // Where the pass's items of four parts are mostly empty and its finalize launch costs more than the
 // work, up to some waves of warps; beyond, its order, which keeps a range's rows in L1 and L2 for
-// all candidates, counts for more. Measured, a call queued among others, the pass against one
-// launch (us):
-//   one part (up to 4,096 rows): 200 candidates on 1,000 rows 17.3 and 14.2; on 2,000 rows with 20
-//     members 8,000 candidates 29.3 and 25.9, 20,000 46 and 40, with 64 members 20,000 65.1 and
-//     63.4, 60,000 131 and 139;
-//   two parts: 4,756 rows 1,600 candidates 22.5 and 18.9, 3,500 23.3 and 22.7, 8,000 36 and 40;
-//   both trends, where the pass takes one term a step, up to eight parts: 20,000 x 200, 800
-//     candidates 20.3 and 14.9, 1,600 24.6 and 21.2, 3,200 32.5 and 30.5, 6,400 48.3 and 49.6;
-//   one trend over more parts stays with the pass: 20,000 rows, 1,600 candidates 18.9 and 19.2.
-bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative) {
+// all candidates, counts for more. The members make the line: a warp here goes over every member
+// whose overlap is wanted, the pass drops most of a sparse candidate's work before it gets to them.
+// Wanted are all (`all`: the caller reads every overlap) or those that share a column, 18 / cols of
+// them taken as typical. Measured, calls queued one behind the other, the pass's time over this
+// kernel's at its side of the line and past it:
+//   one part: 1.06-1.66 throughout for 33 to 128 words; up to 32 words with 64 members wanted 1.02 at
+//     6,000 candidates, 0.95 at 10,000;
+//   two parts: without members 1.18 at 12,000 warps, 1.04 at 20,000; 20 wanted 1.24 at 3,200, 1.00 at
+//     12,000, 0.92 at 20,000; 64 wanted 1.19 at 3,200, 0.87 at 6,000;
+//   three to eight parts: without members 1.12 at 9,000 warps, 0.97 at 12,000; 20 wanted 1.08 at 4,800,
+//     0.99 at 5,600, 0.92 at 8,000, 0.75 at 12,800; 64 wanted 1.23 at 3,200, 1.05 at 4,000, 0.94 at
+//     4,800, 0.58 at 12,800.
+// One trend over more than two parts stays with the pass.
+static int64_t wanted_members(uint32_t n_arch, bool all, int32_t cols) {
+  return all || cols <= 18 ? n_arch : (int64_t)n_arch * 18 / cols;
+}
+
+bool pair_score_fits(int64_t W, uint32_t n_cand, bool negative, uint32_t n_arch, bool all,
+                     int32_t cols) {
   const int64_t parts = (W + kRangeWords - 1) / kRangeWords, warps = (int64_t)n_cand * parts;
-  if (parts == 1) return warps <= 32000;
-  if (negative) return parts <= kScoreWarps && warps <= 16000;
-  return parts == 2 && warps <= 7000;
+  const int64_t wanted = wanted_members(n_arch, all, cols);
+  if (parts == 1) return warps <= (W <= 32 && wanted > 32 ? 8000 : 32000);
+  if (parts > (negative ? kScoreWarps : 2)) return false;
+  return warps <= 3200 + (parts == 2 ? 153600 : 75600) / (12 + wanted);
 }
 
 cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negative, bool pdl,
@@ -372,9 +412,12 @@ cudaError_t launch_pair_score(const PairArgs& p, const ScoreArgs& f, bool negati
   // several candidates per block while their warps are few
   const int cands = parts >= kScoreCands ? 1 : kScoreCands / parts;
   const unsigned blocks = (unsigned)(((uint64_t)p.n_cand + cands - 1) / cands);
+  // (a few members are in flight together anyway)
+  const bool side = p.W <= 32 && wanted_members(p.n_arch, !p.score, p.C) > 2 * kScoreMembers;
+  auto kern = negative ? (side ? pair_score_kernel<true, 8> : pair_score_kernel<true, 32>)
+                       : (side ? pair_score_kernel<false, 8> : pair_score_kernel<false, 32>);
   count_launch();
-  return launch_maybe_pdl(pdl, negative ? pair_score_kernel<true> : pair_score_kernel<false>,
-                          dim3(blocks), dim3(32 * parts * cands), 0, s, p, f, parts);
+  return launch_maybe_pdl(pdl, kern, dim3(blocks), dim3(32 * parts * cands), 0, s, p, f, parts);
 }
 
 cudaError_t launch_pair_build(const Layout& L, const uint32_t* ranks, uint32_t* table,

@@ -219,7 +219,7 @@ cudaError_t launch_pair_eval(const PairArgs&, bool, int, bool, cudaStream_t) {
   note("pair evaluate");
   return cudaSuccess;
 }
-bool pair_score_fits(int64_t, uint32_t, bool) { return false; }
+bool pair_score_fits(int64_t, uint32_t, bool, uint32_t, bool, int32_t) { return false; }
 cudaError_t launch_pair_score(const PairArgs&, const ScoreArgs&, bool, bool, cudaStream_t) {
   return cudaSuccess;
 }
