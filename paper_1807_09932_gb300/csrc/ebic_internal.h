@@ -166,10 +166,6 @@ constexpr int kPairMaxArch = 64;      // archive members the fused overlap pass 
 // table rows): a lane of a chain step reads its first 16 bytes in place of a segment whose
 // words it has already zeroed.
 constexpr int kOnesWords = 128;
-__host__ __device__ inline const uint32_t* pair_ones(const uint32_t* table, uint64_t cols,
-                                                    uint64_t stride) {
-  return table + cols * cols * stride;
-}
 inline int64_t pair_stride(int64_t words) {
   return (words + kPairRangeWords - 1) / kPairRangeWords * kPairRangeWords;
 }

@@ -50,38 +50,6 @@ __device__ __forceinline__ void load_terms(const PairArgs& p, uint32_t cand, int
   }
 }
 
-// The term list of candidate `cand` of a checked CSR list, computed in registers (the batched
-// pass has no preparation kernel to build it): the same words the preparation writes, lane i
-// holding terms i and 32 + i, lane 31's hi word the length L.
-// From the candidate's L columns in registers (lane i: columns i and 32 + i).
-template <bool NEG>
-__device__ __forceinline__ void terms_from_cols(uint32_t c_lo, uint32_t c_hi, int L, uint32_t C,
-                                                uint32_t S, int lane, Terms& t) {
-  const uint32_t n_lo = __shfl_down_sync(0xFFFFFFFFu, c_lo, 1);
-  const uint32_t n_hi = __shfl_down_sync(0xFFFFFFFFu, c_hi, 1);
-  const uint32_t h0 = __shfl_sync(0xFFFFFFFFu, c_hi, 0);
-  const uint32_t next_lo = lane == 31 ? h0 : n_lo;  // c_{i+1} for i = lane
-  const int n_terms = L == 1 ? 1 : L - 1;
-  const bool t_lo = lane < n_terms, t_hi = lane + 32 < n_terms;
-  t.lo = t_lo ? (L == 1 ? c_lo * C + c_lo : c_lo * C + next_lo) * S : 0u;
-  t.hi = lane == 31 ? (uint32_t)L : (t_hi ? (c_hi * C + n_hi) * S : 0u);
-  if (NEG) {
-    t.blo = t_lo && L > 1 ? (next_lo * C + c_lo) * S : 0u;
-    t.bhi = t_hi ? (n_hi * C + c_hi) * S : 0u;
-  }
-}
-
-template <bool NEG>
-__device__ __forceinline__ void terms_from_list(const uint16_t* __restrict__ cols,
-                                                const uint32_t* __restrict__ offs, uint32_t cand,
-                                                uint32_t C, uint32_t S, int lane, Terms& t) {
-  const uint32_t o = offs[cand];
-  const int L = (int)(offs[cand + 1] - o);
-  const uint32_t c_lo = lane < L ? cols[o + lane] : 0u;
-  const uint32_t c_hi = lane + 32 < L ? cols[o + 32 + lane] : 0u;
-  terms_from_cols<NEG>(c_lo, c_hi, L, C, S, lane, t);
-}
-
 // L2 prefetch of the table rows' segments that the first chain step of a term list reads, in the
 // item that starts `word` words into the rows: 128 bytes per lane, kStepLoads / PARTS rows of
 // 4 PARTS lines. A prefetch holds no register: the pass issues one for the next candidate's first
