@@ -534,8 +534,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 // trend flag is NEG, its items (range of kItemWords words, group of kPairWarps candidates) laid
 // end to end in request order and taken round-robin by a persistent grid, so the CTAs walk each
 // request's ranges in order and its table rows stay in L2 while its candidates read them. The
-// chain and epilogue are the single-population pass's (pair_chain.cuh); the term list is
-// computed in registers from the checked candidate list.
+// chain and epilogue are the single-population pass's (pair_chain.cuh); the term lists are
+// written by the check kernel.
 constexpr uint32_t kStartCache = 1024;  // item starts kept in shared memory (requests)
 
 template <bool NEG, bool FIT>
@@ -1079,7 +1079,7 @@ int ebic_batch_create(uint32_t max_requests, ebic_batch** out) {
   int arc = ensure_batch_attr();  // before the capture: not a stream operation
   if (arc != EBIC_OK) return fail_free(arc);
   // capture: copy the descriptor block (pinned -> device), clear the error words, then the
-  // three kernels; the stage size is fixed at the largest tile so any batch composition fits
+  // kernels; the stage size is fixed at the largest tile so any batch composition fits
   cudaStream_t cs = nullptr;
   e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   if (e != cudaSuccess) return fail_free(cerr(e, "capture stream"));

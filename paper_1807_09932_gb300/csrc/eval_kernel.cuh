@@ -36,7 +36,7 @@
 // warp, those of more than 208 columns, whose slabs are 8, 4 or 2 words high, 4 to 16, whose reads
 // then meet in banks by chance (2 to 3 wavefronts instead of one).
 // Measured, counts and bitmaps of 1,600 candidates, against packed byte and half compares of
-// every column (the form before): 436,444 x 64, 2-16 columns 251 -> 140 us; 20,000 x 200, 2-20
+// every column (the form before): 436,444 x 64, 2-16 columns 251 -> 142 us; 20,000 x 200, 2-20
 // columns, both trends 66 -> 26 us; 50,021 x 457, 2-64 columns 487 -> 76 us.
 #pragma once
 

@@ -384,7 +384,7 @@ class GpuBackend:
         hin = slot["hin"][0].data_ptr()
         din, dout = slot["din"].data_ptr(), slot["dout"].data_ptr()
         if len(reqs) == 1 and self.runs[reqs[0].run_id]["pairs"]:
-            # a batch of one: the per-population fused call (three launches) costs less than the
+            # a batch of one: the per-population fused call (two or three launches) costs less than the
             # batch graph's fixed launches, with the same results; its kernels read the pinned
             # lists in place, so nothing is uploaded
             r = reqs[0]
