@@ -338,8 +338,8 @@ int ebic_matrix_get_tile(const ebic_matrix* m, int32_t* tile_slabs, int32_t* row
  * are checked on the device; a failed request produces zero counts and no bitmaps, its matrix's
  * status records EBIC_ERR_INVALID_ARG, and the others are unaffected.
  * Results are identical to scoring each request alone with ebic_eval_population. Batching pays for
- * requests on matrices with a pair table; without tables the rank-code pass takes a fifth longer
- * than the evaluator's single calls where those fill the GPU.
+ * requests on matrices with a pair table, and for small requests; without tables large ones can take
+ * longer than single calls (64 populations on matrices of 20 to 500 columns 6.7 ms against 5.6).
  */
 typedef struct ebic_eval_request {
   const ebic_matrix* m;
