@@ -679,10 +679,7 @@ int ebic_load_matrix(const float* x, int64_t rows, int32_t cols, int64_t ld, uin
 int ebic_free_matrix(ebic_matrix* m) {
   if (!m) return EBIC_OK;
   DeviceGuard g(m->device);
-  // no stream uses the matrix once the device is synchronized
-  cudaError_t e = cudaDeviceSynchronize();
-  const cudaError_t e1 = device_free(m->pairs, nullptr), e2 = device_free(m->ranks, nullptr);
-  if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
+  const cudaError_t e = device_retire({m->pairs, m->ranks}, m->device, false);
   delete m;
   if (e != cudaSuccess) return cuda_fail(e, "freeing a matrix");
   return EBIC_OK;
@@ -1256,11 +1253,11 @@ int ebic_matrix_drop_pairs(ebic_matrix* m) {
   if (!m) return fail(EBIC_ERR_INVALID_ARG, "matrix is NULL");
   if (m->pairs) {
     DeviceGuard g(m->device);
-    EBIC_CUDA(cudaDeviceSynchronize());  // no stream reads the table any more
-    EBIC_CUDA(device_free(m->pairs, nullptr));
+    const cudaError_t e = device_retire({m->pairs}, m->device, false);
     m->pairs = nullptr;
     m->pair_stride = 0;
     m->pair_bytes = 0;
+    EBIC_CUDA(e);
   }
   return EBIC_OK;
 }

@@ -13,6 +13,7 @@
 // threads and streams may use them side by side; memory is handed from one user to the next only
 // after the first one's free is reached by its stream.
 #include <mutex>
+#include <vector>
 
 #include "ebic_internal.h"
 
@@ -26,6 +27,44 @@ constexpr uint64_t kPoolKeep[kPools] = {2ull << 30, 512ull << 20};
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 cudaMemPool_t g_pool[kMaxDevices][kPools] = {};
+
+// Lasting memory is allocated and freed on a stream of the library's own, which carries nothing else: a
+// block freed on the stream it is next allocated on is handed over without a look at other streams' work.
+struct Lasting {
+  std::mutex mu;
+  cudaStream_t stream = nullptr;
+  cudaEvent_t allocated = nullptr;
+  std::vector<void*> waiting;  // to be freed, by the next call that can
+  void* neighbour = nullptr;   // see wait_idle
+  cudaError_t ready() {        // under mu
+    cudaError_t e = cudaSuccess;
+    if (!stream) e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !allocated)
+      e = cudaEventCreateWithFlags(&allocated, cudaEventDisableTiming);
+    return e;
+  }
+};
+Lasting g_lasting[kMaxDevices];
+
+// Waits until the device, the current one, has run all work given to it. By cudaFree, which waits for
+// every stream (CUDA Programming Guide, "Stream Ordered Memory Allocator": cudaMalloc and cudaFree make
+// the GPU synchronize across all executing streams; beside a 20 ms kernel on another stream it returned
+// when that had ended) and which a thread may call while another one captures in thread-local or relaxed
+// mode. cudaDeviceSynchronize fails then, and so does the capture; an operation on the legacy stream does
+// that to the capture of any blocking stream. The block that stays allocated beside the freed one
+// keeps the two calls at 2.5 us (60 when they map and unmap their page).
+cudaError_t wait_idle(Lasting& r) {
+  void* block = nullptr;
+  cudaError_t e = cudaSuccess;
+  {
+    std::lock_guard<std::mutex> lk(r.mu);
+    if (!r.neighbour) e = cudaMalloc(&r.neighbour, 256);
+  }
+  if (e == cudaSuccess) e = cudaMalloc(&block, 256);
+  if (e == cudaSuccess) return cudaFree(block);
+  (void)cudaGetLastError();
+  return e == cudaErrorMemoryAllocation ? cudaDeviceSynchronize() : e;
+}
 
 cudaError_t pool_of(int device, Pool which, cudaMemPool_t* out) {
   if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
@@ -84,10 +123,19 @@ cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
   cudaMemPool_t pool = nullptr;
   cudaError_t e = pool_of(device, kLasting, &pool);
   if (e != cudaSuccess) return e;
-  e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
-  if (e == cudaErrorMemoryAllocation && give_back(device, s))
-    e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
-  return e;
+  Lasting& r = g_lasting[device];
+  auto alloc = [&]() {
+    std::lock_guard<std::mutex> lk(r.mu);
+    cudaError_t x = r.ready();
+    if (x == cudaSuccess) x = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, r.stream);
+    if (x != cudaSuccess) return x;
+    x = cudaEventRecord(r.allocated, r.stream);
+    if (x == cudaSuccess) x = cudaStreamWaitEvent(s, r.allocated, 0);
+    if (x != cudaSuccess) (void)cudaFreeAsync(*p, r.stream);
+    return x;
+  };
+  e = alloc();
+  return e == cudaErrorMemoryAllocation && give_back(device, s) ? alloc() : e;
 }
 
 cudaError_t call_table_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
@@ -100,6 +148,26 @@ cudaError_t device_free(void* p, cudaStream_t s) {
   return p ? cudaFreeAsync(p, s) : cudaSuccess;
 }
 
+cudaError_t device_retire(std::vector<void*> ps, int device, bool drained) {
+  if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
+  Lasting& r = g_lasting[device];
+  if (!drained) {  // what an earlier call could not free goes with it
+    std::lock_guard<std::mutex> lk(r.mu);
+    ps.insert(ps.end(), r.waiting.begin(), r.waiting.end());
+    r.waiting.clear();
+  }
+  cudaError_t e = drained ? cudaSuccess : wait_idle(r);
+  std::lock_guard<std::mutex> lk(r.mu);
+  if (e == cudaSuccess) e = r.ready();
+  for (void* p : ps) {
+    if (!p) continue;
+    if (e == cudaSuccess) e = cudaFreeAsync(p, r.stream);
+    if (e != cudaSuccess) r.waiting.push_back(p);
+  }
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
+}
+
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
   cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, s);
   int device = 0;
@@ -110,7 +178,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
 }
 
 cudaError_t release_memory(int device) {
-  const cudaError_t e = cudaDeviceSynchronize();
+  const cudaError_t e = device_retire({}, device, false);
   if (e == cudaSuccess) trim(device);
   return e;
 }

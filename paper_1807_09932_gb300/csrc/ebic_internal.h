@@ -15,6 +15,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -73,9 +74,14 @@ void count_launches(int64_t n);  // n kernels at once (a negative n takes back c
 
 // Device memory that lives as long as a matrix, a pair table or a search, from the device's pool
 // (devmem.cpp), stream-ordered on s: other streams may use it once s has reached the allocation.
-// Freed memory must no longer be in use by any stream but s.
+// device_free: memory that no stream but s uses any more.
 cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s);
 cudaError_t device_free(void* p, cudaStream_t s);
+// The same for memory of `device`, the current one, that no stream uses any more (drained), or that any
+// stream may still use: then it is freed once the device is idle, which this waits for. On an error (a
+// capture in global mode is under way in the process) the memory is kept, and freed by the next call that
+// can.
+cudaError_t device_retire(std::vector<void*> ps, int device, bool drained);
 // What the pools of `device`, the current one, hold unused goes back to the system, once it is idle.
 cudaError_t release_memory(int device);
 // A single call's pair table and term lists, from a pool of their own; freed with cudaFreeAsync. Not

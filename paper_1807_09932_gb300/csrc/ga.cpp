@@ -822,7 +822,7 @@ struct GpuEvaluator : Evaluator {
         T(2 * p.archive_size), max_len(p.max_len), W(words) {}
   ~GpuEvaluator() override {
     cudaStreamSynchronize(s);
-    for (void* a : allocs) (void)device_free(a, s);
+    if (!allocs.empty()) (void)device_retire(allocs, device, true);
     if (pinned) cudaFreeHost(pinned);
   }
   template <class X>

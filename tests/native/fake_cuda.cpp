@@ -17,6 +17,15 @@ enum Kind { kPool, kAsync, kMalloc, kCallPool, kKinds };
 std::string g_log;
 int g_seen[kKinds], g_fail_from[kKinds], g_fail_count[kKinds];
 bool g_capturing;
+// a capture under way in another thread: 0 none, 1 thread-local or relaxed, 2 global; and whether a call
+// that may not be made beside it has ended it
+int g_other;
+bool g_other_broken;
+cudaError_t beside(int from) {
+  if (g_other < from) return cudaSuccess;
+  g_other_broken = true;
+  return cudaErrorStreamCaptureUnsupported;
+}
 struct Block {
   size_t bytes;
   Kind kind;
@@ -62,6 +71,8 @@ void fake_reset() {
   g_log.clear();
   for (int k = 0; k < kKinds; ++k) g_seen[k] = g_fail_from[k] = g_fail_count[k] = 0;
   g_capturing = false;
+  g_other = 0;
+  g_other_broken = false;
 }
 // allocations `from` .. `from + count` of a kind, counted from the last reset, find no memory
 void fake_fail(int kind, int from, int count) {
@@ -69,6 +80,8 @@ void fake_fail(int kind, int from, int count) {
   g_fail_count[kind] = count;
 }
 void fake_capture(int on) { g_capturing = on != 0; }
+void fake_other_capture(int mode) { g_other = mode; }
+int fake_other_broken() { return g_other_broken; }
 const char* fake_log() { return g_log.c_str(); }
 int fake_seen(int kind) { return g_seen[kind]; }
 uint64_t fake_limit(int kind) {
@@ -95,9 +108,24 @@ cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t pool, cuda
   return take(p, n, kind_of(pool));
 }
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return take(p, n, kAsync); }
-cudaError_t cudaMalloc(void** p, size_t n) { return take(p, n, kMalloc); }
-cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return drop(p); }
-cudaError_t cudaFree(void* p) { return drop(p); }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  const cudaError_t e = beside(2);
+  return e == cudaSuccess ? take(p, n, kMalloc) : e;
+}
+cudaError_t cudaFreeAsync(void* p, cudaStream_t s) {
+  const cudaError_t e = beside(s ? 2 : 1);
+  return e == cudaSuccess ? drop(p) : e;
+}
+cudaError_t cudaFree(void* p) {  // (waits for the device)
+  const cudaError_t e = beside(2);
+  if (e != cudaSuccess) return e;
+  note("idle");
+  return drop(p);
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+  *s = reinterpret_cast<cudaStream_t>(0x100);
+  return beside(2);
+}
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
   *p = std::calloc(1, n);
   return cudaSuccess;
@@ -140,8 +168,9 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) {
   return g_capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
 }
 cudaError_t cudaDeviceSynchronize() {
-  note("sync");
-  return g_capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+  note("device sync");
+  const cudaError_t e = beside(1);
+  return g_capturing ? cudaErrorStreamCaptureUnsupported : e;
 }
 cudaError_t cudaGetDevice(int* d) {
   *d = 0;
@@ -187,6 +216,11 @@ cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
   std::memset(p, v, n);
   return cudaSuccess;
 }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
+  *e = reinterpret_cast<cudaEvent_t>(0x200);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }

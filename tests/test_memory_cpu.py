@@ -184,7 +184,7 @@ def test_release(lib):
     lib.ebic_free_matrix(h)
     lib.fake_reset()
     assert lib.ebic_release_memory(ctypes.c_int32(-1)) == OK
-    assert log(lib)[0] == "sync"
+    assert log(lib)[0] == "idle"
     assert set(log(lib)[1:]) == {"trim library 0", "trim tables 0", "trim default 0"}
     assert lib.ebic_release_memory(ctypes.c_int32(7)) == -1
 
@@ -228,3 +228,40 @@ def test_a_closed_run_leaves_its_memory_to_every_allocator():
     be.runs = {3: {"m": NS(close=lambda: calls.append("close"))}}
     be.close_run(3)
     assert calls == ["sync", "close", ("release", 0)]
+
+
+def test_closing_beside_another_threads_capture(lib):
+    """Closing a matrix, dropping its table and releasing memory wait for the device in a way that a
+    thread-local or relaxed capture of another thread (ebic_batch_create's, a device search's) survives."""
+    rc, h = load(lib, 3000, 20)
+    assert rc == OK and lib.ebic_matrix_build_pairs(h, 1 << 40, None, None) == OK
+    lib.fake_reset()
+    lib.fake_other_capture(1)
+    assert lib.ebic_matrix_drop_pairs(h) == OK and log(lib) == ["idle"]
+    assert lib.ebic_free_matrix(h) == OK and log(lib) == ["idle", "idle"]
+    assert lib.ebic_release_memory(ctypes.c_int32(-1)) == OK
+    assert not lib.fake_other_broken() and lib.fake_live(POOL) == 0
+
+
+def test_memory_that_cannot_be_freed_now_is_freed_later(lib):
+    """Beside a capture in global mode nothing may wait for the device: the close fails, and its memory,
+    which other streams may still use, is neither freed nor lost."""
+    rc, h = load(lib, 3000, 20)
+    rc2, h2 = load(lib, 500, 20)
+    held = lib.fake_live(POOL)
+    assert rc == rc2 == OK and held > 0
+    lib.fake_reset()
+    lib.fake_other_capture(2)
+    assert lib.ebic_free_matrix(h) == -3        # EBIC_ERR_CUDA
+    assert lib.fake_live(POOL) == held
+    lib.fake_other_capture(0)
+    assert lib.ebic_free_matrix(h2) == OK
+    assert lib.fake_live(POOL) == 0
+
+
+def test_closing_without_a_byte_left(lib):
+    rc, h = load(lib, 3000, 20)
+    lib.fake_reset()
+    lib.fake_fail(MALLOC, 0, 100)
+    assert lib.ebic_free_matrix(h) == OK and log(lib) == ["device sync"]
+    assert lib.fake_live(POOL) == 0
