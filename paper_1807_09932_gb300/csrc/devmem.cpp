@@ -28,20 +28,14 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 cudaMemPool_t g_pool[kMaxDevices][kPools] = {};
 
-// Lasting memory is allocated and freed on a stream of the library's own, which carries nothing else: a
-// block freed on the stream it is next allocated on is handed over without a look at other streams' work.
+// Memory that its owner has given up is freed, once no stream uses it, on a stream of the library's own.
 struct Lasting {
   std::mutex mu;
   cudaStream_t stream = nullptr;
-  cudaEvent_t allocated = nullptr;
   std::vector<void*> waiting;  // to be freed, by the next call that can
   void* neighbour = nullptr;   // see wait_idle
   cudaError_t ready() {        // under mu
-    cudaError_t e = cudaSuccess;
-    if (!stream) e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess && !allocated)
-      e = cudaEventCreateWithFlags(&allocated, cudaEventDisableTiming);
-    return e;
+    return stream ? cudaSuccess : cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
   }
 };
 Lasting g_lasting[kMaxDevices];
@@ -123,19 +117,10 @@ cudaError_t device_alloc(void** p, size_t bytes, int device, cudaStream_t s) {
   cudaMemPool_t pool = nullptr;
   cudaError_t e = pool_of(device, kLasting, &pool);
   if (e != cudaSuccess) return e;
-  Lasting& r = g_lasting[device];
-  auto alloc = [&]() {
-    std::lock_guard<std::mutex> lk(r.mu);
-    cudaError_t x = r.ready();
-    if (x == cudaSuccess) x = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, r.stream);
-    if (x != cudaSuccess) return x;
-    x = cudaEventRecord(r.allocated, r.stream);
-    if (x == cudaSuccess) x = cudaStreamWaitEvent(s, r.allocated, 0);
-    if (x != cudaSuccess) (void)cudaFreeAsync(*p, r.stream);
-    return x;
-  };
-  e = alloc();
-  return e == cudaErrorMemoryAllocation && give_back(device, s) ? alloc() : e;
+  e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
+  if (e == cudaErrorMemoryAllocation && give_back(device, s))
+    e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, pool, s);
+  return e;
 }
 
 cudaError_t call_table_alloc(void** p, size_t bytes, int device, cudaStream_t s) {

@@ -54,6 +54,7 @@ cudaError_t drop(void* p) {
 
 // pools by their handles: the library's, told apart by their limits, then the default one
 char g_handles[3];
+const cudaStream_t kOwnStream = reinterpret_cast<cudaStream_t>(0x100);
 const cudaMemPool_t kDefaultPool = reinterpret_cast<cudaMemPool_t>(&g_handles[2]);
 int g_pools;
 uint64_t g_limit[2];
@@ -123,7 +124,7 @@ cudaError_t cudaFree(void* p) {  // (waits for the device)
   return drop(p);
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
-  *s = reinterpret_cast<cudaStream_t>(0x100);
+  *s = kOwnStream;
   return beside(2);
 }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
@@ -163,7 +164,8 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) {
   *st = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) {
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  if (s == kOwnStream) return beside(2);  // (the library's own, for an allocation)
   note("sync");
   return g_capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
 }
@@ -216,11 +218,6 @@ cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
   std::memset(p, v, n);
   return cudaSuccess;
 }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
-  *e = reinterpret_cast<cudaEvent_t>(0x200);
-  return cudaSuccess;
-}
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
