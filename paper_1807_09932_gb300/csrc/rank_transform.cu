@@ -136,7 +136,7 @@ __device__ __forceinline__ void sort_keys(uint32_t (&x)[E], int lane) {
 // 560, 755 and 176 (61 of 85 million wavefronts were bank conflicts); 50,021 x 457 with (key,
 // column) pairs sorted in shared memory 1,328. A CTA takes 132 bytes a column and 16 KB (and the 1 KB
 // that every CTA does): three fit on an SM up to 457 columns, two from 458 to 512 (50,021 rows: 457
-// columns 234 us, 458 254, 480 256, 512 258, by library events on one box; the former 1,338 to 1,376).
+// columns 234 us, 458 254, 480 256, 512 258, by library events on one GPU; the former 1,338 to 1,376).
 // Beyond, one of 16 warps.
 template <int E>
 constexpr int kWideWarps = E == 32 ? 16 : 8;
